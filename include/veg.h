@@ -277,11 +277,13 @@ veg_status veg_sync_status(const void* workspace, cudaStream_t stream, int64_t* 
  * tile_order: optional device int32 [global tiles] from veg_tile_order
  * (the order in which tiles are scheduled; NULL = row-major; results do
  * not depend on it).
- * tf_group: TFs composited per pass (1, 2, 4 or 8; 0 = library default, 1;
- * the autotuner of the Python package picks per shape).
+ * tf_group: TFs composited per pass (0..8): a hint of earlier kernels, kept
+ * for its callers; every pass composites one table, results never depend on
+ * it.
  * tile_batch: splats of a tile's list staged per pass through shared memory
- * (128, 256 or 512; 0 = 256; the autotuner picks per shape); results do not
- * depend on it.  The instrumented build (stats) stages 256.
+ * (128, 256 or 512; 0 = 256; the autotuner of the Python package picks per
+ * shape); results do not depend on it.  The instrumented build (stats)
+ * stages 256.
  * splat_shade: optional device float [V][n][2] of Blinn-Phong factors
  * (s_d, s_s) from veg_shade (8-byte aligned); when given, each splat is
  * blended with the colour s_d rgb + s_s of Eq. 2 instead of rgb.  Opacity,
@@ -323,8 +325,9 @@ veg_status veg_composite_fwd(const veg_camera* cams, int32_t n_views, int64_t n,
  * dL/ds_d and dL/ds_s per record, and veg_shade_bwd chains them to the
  * normals, the material coefficients and the means; the colour slopes in dv
  * are scaled by s_d.  Shading with stats returns VEG_ERR_UNSUPPORTED.
- * tf_group (1, 2 or 4; 0 = min(n_tf, 4)) and tile_batch (128, 256 or 512;
- * 0 = 256) as in veg_composite_fwd; results do not depend on them.
+ * tf_group (0..8) and tile_batch (0, 128, 256 or 512) are checked and have
+ * no effect: every pass takes one table and each warp stages the list chunks
+ * it walks.
  * stats: optional device uint64[7] accumulating (replayed pixel-splat pairs,
  * pairs walked after culling, pairs above the exponent cutoff, alpha
  * evaluations, blended pairs, blended pairs below the 0.99 clamp, pairs with
@@ -679,8 +682,7 @@ veg_status veg_train_step(const veg_train_args* args, int32_t view, int32_t map,
  * longest-first tile schedule (veg_tile_order) and Eq. 1 compositing
  * (veg_composite_fwd), all scratch in `workspace` (device, 256-byte
  * aligned, >= veg_render_workspace_size bytes; width and height there are
- * the largest view's).  tf_group: TFs per compositing pass, 0 = the
- * library's default (1), else 1, 2, 4 or 8; results do not depend on it.
+ * the largest view's).  tf_group: 0..8, no effect (veg_composite_fwd).
  * Outputs out and n_contrib as veg_composite_fwd (caller-owned device
  * memory, overwritten).  Overflow of `capacity` is reported by
  * veg_sync_status on the same workspace.  Returns VEG_ERR_INVALID_ARGUMENT

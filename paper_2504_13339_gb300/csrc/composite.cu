@@ -18,33 +18,13 @@ veg_status composite_fwd_launch(const veg_camera* cams, int n_views, int64_t n,
                                 unsigned long long* stats, cudaStream_t stream) {
   CompArgs A = make_args(cams, n_views, geo, aux, vals, ranges, order, tf, bg, shade);
   (void)n;
+  (void)tf_group;  // every pass composites one table
   const int B = pick_batch(tile_batch);
-  const int TG = tf.view_tf ? 1
-                            : pick_group(tf_group, tf.n_tf, false, tf.lut_size, shade != nullptr,
-                                         stats ? 256 : B);
-  if (shade) {
-    if (stats) return VEG_ERR_UNSUPPORTED;
-    switch (TG) {
-      case 1: return fwd_batch<1, false, true>(B, A, n_views, out, n_contrib, nullptr, stream);
-      case 2: return fwd_batch<2, false, true>(B, A, n_views, out, n_contrib, nullptr, stream);
-      case 4: return fwd_batch<4, false, true>(B, A, n_views, out, n_contrib, nullptr, stream);
-      default: return fwd_batch<8, false, true>(B, A, n_views, out, n_contrib, nullptr, stream);
-    }
-  }
-  if (stats) {
-    switch (TG) {
-      case 1: return fwd_batch<1, true, false>(B, A, n_views, out, n_contrib, stats, stream);
-      case 2: return fwd_batch<2, true, false>(B, A, n_views, out, n_contrib, stats, stream);
-      case 4: return fwd_batch<4, true, false>(B, A, n_views, out, n_contrib, stats, stream);
-      default: return fwd_batch<8, true, false>(B, A, n_views, out, n_contrib, stats, stream);
-    }
-  }
-  switch (TG) {
-    case 1: return fwd_batch<1, false, false>(B, A, n_views, out, n_contrib, nullptr, stream);
-    case 2: return fwd_batch<2, false, false>(B, A, n_views, out, n_contrib, nullptr, stream);
-    case 4: return fwd_batch<4, false, false>(B, A, n_views, out, n_contrib, nullptr, stream);
-    default: return fwd_batch<8, false, false>(B, A, n_views, out, n_contrib, nullptr, stream);
-  }
+  if (stats)
+    return shade ? VEG_ERR_UNSUPPORTED
+                 : launch_fwd<256, true, false>(A, n_views, out, n_contrib, stats, stream);
+  return shade ? fwd_batch<true>(B, A, n_views, out, n_contrib, stream)
+               : fwd_batch<false>(B, A, n_views, out, n_contrib, stream);
 }
 
 size_t composite_bwd_ws_bytes(int64_t n, int n_views) {
@@ -153,31 +133,14 @@ extern "C" veg_status veg_composite_bwd(const veg_camera* cams, int32_t n_views,
                          reinterpret_cast<const float4*>(splat_aux), vals,
                          reinterpret_cast<const int2*>(tile_ranges), tile_order, tf, bg,
                          splat_shade);
-  const int B = pick_batch(tile_batch);
-  const int TG = tf.view_tf ? 1
-                            : pick_group(tf_group, tf.n_tf, true, tf.lut_size, lit,
-                                         stats ? 256 : B);
   const float4* o4 = reinterpret_cast<const float4*>(out);
   const float4* d4 = reinterpret_cast<const float4*>(dL_dout);
-  if (lit) {
-    switch (TG) {
-      case 1: st = bwd_batch<1, false, true>(B, A, n_views, o4, n_contrib, d4, g2, gsh, nullptr, stream); break;
-      case 2: st = bwd_batch<2, false, true>(B, A, n_views, o4, n_contrib, d4, g2, gsh, nullptr, stream); break;
-      default: st = bwd_batch<4, false, true>(B, A, n_views, o4, n_contrib, d4, g2, gsh, nullptr, stream); break;
-    }
-  } else if (stats) {
-    switch (TG) {
-      case 1: st = bwd_batch<1, true, false>(B, A, n_views, o4, n_contrib, d4, g2, nullptr, stats, stream); break;
-      case 2: st = bwd_batch<2, true, false>(B, A, n_views, o4, n_contrib, d4, g2, nullptr, stats, stream); break;
-      default: st = bwd_batch<4, true, false>(B, A, n_views, o4, n_contrib, d4, g2, nullptr, stats, stream); break;
-    }
-  } else {
-    switch (TG) {
-      case 1: st = bwd_batch<1, false, false>(B, A, n_views, o4, n_contrib, d4, g2, nullptr, nullptr, stream); break;
-      case 2: st = bwd_batch<2, false, false>(B, A, n_views, o4, n_contrib, d4, g2, nullptr, nullptr, stream); break;
-      default: st = bwd_batch<4, false, false>(B, A, n_views, o4, n_contrib, d4, g2, nullptr, nullptr, stream); break;
-    }
-  }
+  if (lit)
+    st = launch_bwd<false, true>(A, n_views, o4, n_contrib, d4, g2, gsh, nullptr, stream);
+  else if (stats)
+    st = launch_bwd<true, false>(A, n_views, o4, n_contrib, d4, g2, nullptr, stats, stream);
+  else
+    st = launch_bwd<false, false>(A, n_views, o4, n_contrib, d4, g2, nullptr, nullptr, stream);
   if (st != VEG_OK || only_2d) return st;
   CamSet cs;
   fill_camset(cams, n_views, &cs);

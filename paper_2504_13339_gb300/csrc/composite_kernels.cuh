@@ -1,20 +1,33 @@
 // Compositing kernels: front-to-back blending (Eq. 1) of depth-sorted splats
-// per 16x16 tile for a group of transfer functions, and its backward pass.
+// per 16x16 tile under each transfer function, and its backward pass.
 //
-// One CTA of 256 threads owns one (view, tile, TF group) work item, in the
-// longest-first order of the tiles; each thread owns one pixel and each warp
-// an 8x4 pixel block.  The tile's list is staged in batches of B splats (the
-// tile batch: 128, 256 or 512, chosen by the caller or its autotuner)
-// through shared memory.  The stager evaluates every
-// splat's colour and opacity under each TF of the group once (linear
-// interpolation in the TF tables: held in shared memory by the forward, read
-// through the L1 cache by the backward), the exponent below which
-// no TF of the group can reach alpha = 1/255, and a conservative mask of the
-// warp blocks that the splat's visible ellipse can touch.  Each warp then
-// compacts the batch into its own list (ballots) and walks only that list,
-// so pairs that provably cannot blend cost nothing.  A pixel leaves once
-// every TF of the group has terminated (T (1 - alpha) < 1e-4); the block
-// stops staging once all its pixels have left.
+// One CTA of 128 threads owns one (view, tile, table) work item, in the
+// longest-first order of the tiles; each warp owns an 8x8 pixel block and
+// each lane two of its pixels, (x, y) and (x, y + 4).  The forward stages the
+// tile's list in batches of B splats (the tile batch: 128, 256 or 512,
+// chosen by the caller or its autotuner) through shared memory; the
+// backward's warps each stage the chunks of 32 that they walk.  The stager
+// evaluates a splat's colour and opacity under the table (linear
+// interpolation, the table in shared memory), the exponent below which it
+// cannot reach alpha = 1/255, and which warp blocks its visible ellipse can
+// touch; each warp walks only the splats that touch its block, so pairs that
+// provably cannot blend cost nothing.  A pixel leaves once it has terminated
+// (T (1 - alpha) < 1e-4); a work item ends once all its pixels have left.
+//
+// One table per work item: a splat that a table maps to no opacity never
+// enters that item's lists, and each table stops at its own termination.
+// Walking a group of 2 or 4 tables at once shares a splat's geometry but
+// walks the union of their lists: on the 1M-Gaussian scene it took 2 to 4
+// times as long forward and 1.5 times backward.
+//
+// What bounds both kernels is instruction issue: a tile's splats are read
+// from DRAM once (1-2% of its rate) and then meet up to 256 pixels each.  Two
+// pixels per lane halve what a splat costs per pixel beyond its own
+// arithmetic (list entry, shared-memory loads, loop, warp votes and, in the
+// backward, the warp reduction), and most of the pair's arithmetic runs in
+// the two-wide float32 instructions.  With one pixel per lane the 1M-Gaussian
+// scene (1024x1024, 4 tables) took 633 us forward and 1254 us backward
+// (1778 us with four tables per pass); with two 500 and 940 us.
 //
 // The per-pair arithmetic that decides skips, the 0.99 clamp and
 // termination uses explicitly rounded operations shared by the forward and
@@ -31,53 +44,54 @@ namespace veg {
 
 namespace {
 
-constexpr int kWarps = 8;  // 256 threads
-// Every per-splat shared array is indexed by the splat's batch slot, which
-// a thread loops over in steps of the block size (B / 256 slots per thread
-// for B = 512; threads past the slots stage nothing for B = 128).
-
-// A warp list entry is a batch slot: one byte for batches up to 256 splats.
-template <int B>
-struct ListEntry {
-  using T = unsigned char;
-};
-template <>
-struct ListEntry<512> {
-  using T = unsigned short;
-};
+constexpr int kWarps = 4;
+constexpr int kCompThreads = 32 * kWarps;
+constexpr float kLog2e = 1.44269502162933349609375f;
+// Every per-splat shared array of the forward is indexed by the splat's batch
+// slot, which a thread loops over in steps of the block size; slot B is a
+// splat that no pixel blends (it pads the warp lists to whole steps of the
+// walk).  A warp list entry is 16 times the batch slot: the byte offset of the slot
+// in every 16-byte shared array.
+using ListEntry = unsigned short;
 
 // 2^x with the hardware approximation (ex2.approx.ftz), x = power * log2(e).
-__device__ __forceinline__ float gauss_of(float power) {
+// For x <= 0 the result is at most 1 (checked over every float32 below zero).
+__device__ __forceinline__ float ex2_approx(float x) {
   float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(mul(power, 1.44269502162933349609375f)));
-  return fminf(y, 1.0f);
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
-// power = -1/2 (a dx^2 + c dy^2) - b dx dy with (na, nb, nc) = (-a/2, -b, -c/2).
-__device__ __forceinline__ float power_of(float dx, float dy, float na, float nb, float nc) {
-  return __fmaf_rn(na, mul(dx, dx), __fmaf_rn(nc, mul(dy, dy), mul(nb, mul(dx, dy))));
+__device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
+
+// The Gaussians of a lane's two pixels: e^power with
+//   power = -1/2 (a dx^2 + c dy^2) - b dx dy,
+// u = (ux, ux, uy, uy), q = (-a/2, -a/2, -b, -b), r = (-c/2, -c/2, ..).
+// Both halves are rounded exactly like the scalar operations.
+struct Offsets {
+  float2 dx, dy, dxx, dyy, dxy;  // of the splat centre from the two pixels
+};
+__device__ __forceinline__ float2 power2(float4 u, float4 q, float4 r, float2 px, float2 py,
+                                         Offsets& o) {
+  o.dx = sub2(lo2(u), px);
+  o.dy = sub2(hi2(u), py);
+  o.dxx = mul2(o.dx, o.dx);
+  o.dyy = mul2(o.dy, o.dy);
+  o.dxy = mul2(o.dx, o.dy);
+  return fma2(lo2(q), o.dxx, fma2(lo2(r), o.dyy, mul2(hi2(q), o.dxy)));
 }
 
-// The same exponent from the splat centre (ux, uy) and the pixel pxy, with
-// the offsets d = u - p and their squares d2 formed as float32 pairs (same
-// rounding as the scalar form); also returns dxy = dx dy.
-__device__ __forceinline__ float power_at(float ux, float uy, float2 pxy, float na, float nb,
-                                          float nc, float2& d, float2& d2, float& dxy) {
-  d = sub2(make_float2(ux, uy), pxy);
-  d2 = mul2(d, d);
-  dxy = mul(d.x, d.y);
-  return __fmaf_rn(na, d2.x, __fmaf_rn(nc, d2.y, mul(nb, dxy)));
-}
-
-// Lowest exponent at which some TF of the group can still reach alpha >=
-// 1/255: alpha = A w G <= max_t(A_t w) e^power, which stays below 1/255 for
-// power < ln(1/(255 max_t A_t w)).  The bound is lowered by 1e-3 to absorb
-// the float32 rounding of the exponent, the exp2 approximation and the log,
-// so every pair above it still meets the exact per-TF test and the skip
-// never changes a decision.  With max_t A_t w < 1/255 no pair can blend.
-__device__ __forceinline__ float power_cutoff(float max_aw) {
-  if (!(max_aw >= kAlphaMin)) return 1.0f;
-  return __logf(kAlphaMin) - __logf(max_aw) - 1e-3f;
+// Lowest exponent at which a splat can still reach alpha >= 1/255: alpha =
+// A w G = A w e^power stays below 1/255 for power < ln(1/(255 A w)).  The
+// bound is lowered by 1e-3 to absorb the float32 rounding of the exponent,
+// the exp2 approximation and the log, so every pair above it still meets the
+// exact test and the cull never changes a decision.  With A w < 1/255 no
+// pair can blend (a cutoff above 0).
+__device__ __forceinline__ float power_cutoff(float aw) {
+  if (!(aw >= kAlphaMin)) return 1.0f;
+  return fmaxf(__logf(kAlphaMin) - __logf(aw) - 1e-3f, -1e30f);
 }
 
 // Hardware approximations (relative error of a few 1e-7), used only where
@@ -93,62 +107,66 @@ __device__ __forceinline__ float sqrt_approx(float x) {
   return y;
 }
 
-// Minimum of q(d) = a dx^2 + 2 b dx dy + c dy^2 (a, c > 0, positive
-// definite) over the rectangle [x0, x1] x [y0, y1]: zero when the rectangle
-// holds the origin, else the least of the four edge minima (on an edge q is
-// a 1-D convex quadratic, minimised at its vertex clamped to the edge).
-__device__ __forceinline__ float conic_min_over_rect(float a, float b, float c, float x0,
-                                                     float x1, float y0, float y1) {
-  if (x0 <= 0.0f && x1 >= 0.0f && y0 <= 0.0f && y1 >= 0.0f) return 0.0f;
-  auto qf = [&](float x, float y) { return a * x * x + 2.0f * b * x * y + c * y * y; };
-  const float ia = rcp_approx(a), ic = rcp_approx(c);
-  float m = qf(x0, fminf(fmaxf(-b * x0 * ic, y0), y1));
-  m = fminf(m, qf(x1, fminf(fmaxf(-b * x1 * ic, y0), y1)));
-  m = fminf(m, qf(fminf(fmaxf(-b * y0 * ia, x0), x1), y0));
-  m = fminf(m, qf(fminf(fmaxf(-b * y1 * ia, x0), x1), y1));
+// Where a splat's exponent can reach `cut`: the pixel centres d (relative to
+// the splat centre) with d^T Q d <= R = -2 cut (Q = conic), tested per block
+// of pixel rows by the ellipse's x extent over the rows' y range.  Its right
+// edge x+(y) = (-b y + sqrt(a R - det y^2)) / a is concave with its maximum
+// hx at y = -b hx / c, so over a range it is largest at that y clamped to the
+// range; the left edge mirrors it.  Extents are widened by 0.2% of hx + 0.02
+// px, the y ranges by 0.2% of hy + 0.02 px and R by 0.2% + 1e-4, far beyond
+// the float32 error of the extents (the cancellation in det and under the
+// root stays below 0.03% of hx while det > 1e-3 a c) and of the per-pixel
+// exponent, so the test never drops a pixel that the per-pixel decision
+// keeps.  An ill-conditioned conic reaches everywhere (the per-pixel test
+// decides).
+struct Reach {
+  bool none, all;
+  float a, b, det, aR, ia, ystar, wx, wy;
+  __device__ __forceinline__ Reach(float a_, float b_, float c, float cut) : a(a_), b(b_) {
+    det = a * c - b * b;
+    none = !(cut < 0.0f);
+    all = !(det > 1e-3f * a * c);
+    const float R = -2.0f * cut * 1.002f + 1e-4f, rd = R * rcp_approx(det);
+    const float hx = sqrt_approx(rd * c), hy = sqrt_approx(rd * a);
+    aR = a * R;
+    ia = rcp_approx(a);
+    ystar = -b * hx * rcp_approx(c);
+    wx = hx * 0.002f + 0.02f;
+    wy = hy * 1.002f + 0.02f;
+  }
+  // The x extent [x0, x1] over the rows [y0, y1]; false if they miss it.
+  __device__ __forceinline__ bool extent(float y0, float y1, float& x0, float& x1) const {
+    y0 = fmaxf(y0 - 0.01f, -wy);
+    y1 = fminf(y1 + 0.01f, wy);
+    const float yr = fminf(fmaxf(ystar, y0), y1), yl = fminf(fmaxf(-ystar, y0), y1);
+    x1 = (sqrt_approx(fmaxf(aR - det * yr * yr, 0.0f)) - b * yr) * ia + wx;
+    x0 = (-sqrt_approx(fmaxf(aR - det * yl * yl, 0.0f)) - b * yl) * ia - wx;
+    return y0 <= y1;
+  }
+};
+
+// The warp blocks a splat can reach, its centre at (rx, ry) from the tile's
+// first pixel: bit by * 2 + bx for the 8x8 block at (8 bx, 8 by).
+__device__ __forceinline__ unsigned warp_block_mask(float rx, float ry, const Reach& e) {
+  if (e.none) return 0u;
+  if (e.all) return 0xfu;
+  unsigned m = 0u;
+#pragma unroll
+  for (int by = 0; by < 2; ++by) {
+    float x0, x1;
+    if (!e.extent(8.0f * by - ry, 8.0f * by + 7.0f - ry, x0, x1)) continue;
+    if (x0 + rx <= 7.0f && x1 + rx >= 0.0f) m |= 1u << (2 * by);
+    if (x0 + rx <= 15.0f && x1 + rx >= 8.0f) m |= 2u << (2 * by);
+  }
   return m;
 }
 
-// Warp blocks (bit by*2+bx for the 8x4 block at tile-relative (8bx, 4by))
-// holding a pixel centre where the exponent can reach `cut`, i.e. a centre d
-// (relative to the splat centre) with d^T Q d <= -2 cut (Q = conic).  A
-// block's bounding-box test rejects far blocks; the rest are kept when the
-// quadratic's minimum over the block's rectangle of pixel centres is within
-// the radius.  Box half extents are widened by 0.2% + 0.02 px and the
-// squared radius by 0.2% + 1e-4, far beyond the float32 error of the
-// per-pixel exponent, so the mask never drops a pixel the exact test keeps.
-// An ill-conditioned conic keeps every block (the per-pixel test decides).
-// EXACT = false keeps every block passing the box test (cheaper to stage;
-// the forward pass, whose iterations are cheap, prefers it).
-template <bool EXACT>
-__device__ __forceinline__ unsigned warp_block_mask(float rx, float ry, float a, float b, float c,
-                                                    float cut) {
-  if (!(cut < 0.0f)) return 0u;
-  const float det = a * c - b * b;
-  if (!(det > 1e-3f * a * c)) return 0xffu;
-  const float r2 = -2.0f * cut, r2_det = r2 * rcp_approx(det);
-  const float hx = sqrt_approx(r2_det * c) * 1.002f + 0.02f;
-  const float hy = sqrt_approx(r2_det * a) * 1.002f + 0.02f;
-  const float r2m = r2 * 1.002f + 1e-4f;
-  const float x0 = rx - hx, x1 = rx + hx, y0 = ry - hy, y1 = ry + hy;
-  unsigned m = 0u;
-#pragma unroll
-  for (int by = 0; by < 4; ++by) {
-    if (y1 < 4.0f * by || y0 > 4.0f * by + 3.0f) continue;
-#pragma unroll
-    for (int bx = 0; bx < 2; ++bx) {
-      if (x1 < 8.0f * bx || x0 > 8.0f * bx + 7.0f) continue;
-      if (!EXACT) {
-        m |= 1u << (by * 2 + bx);
-        continue;
-      }
-      const float q = conic_min_over_rect(a, b, c, 8.0f * bx - rx - 0.01f,
-                                          8.0f * bx + 7.0f - rx + 0.01f,
-                                          4.0f * by - ry - 0.01f, 4.0f * by + 3.0f - ry + 0.01f);
-      if (q <= r2m) m |= 1u << (by * 2 + bx);
-    }
-  }
-  return m;
+// Whether it can reach the 8x8 block whose first pixel is (-rx, -ry) from
+// its centre.
+__device__ __forceinline__ bool block_hit(float rx, float ry, const Reach& e) {
+  float x0, x1;
+  const bool rows = e.extent(-ry, 7.0f - ry, x0, x1);
+  return !e.none && (e.all || (rows && x0 + rx <= 7.0f && x1 + rx >= 0.0f));
 }
 
 __device__ __forceinline__ unsigned lanemask_lt_() {
@@ -161,10 +179,10 @@ __device__ __forceinline__ unsigned lanemask_lt_() {
 // Lane l reads the masks of its P = B/32 consecutive positions P l .. P l +
 // P - 1 as one 32-bit word (B = 128) or P/8 64-bit words (positions past the
 // batch's count hold empty masks); an exclusive warp scan of the per-lane
-// hit counts places each lane's hits in the list.
+// hit counts places each lane's hits in the list, which ends in four entries
+// of the padding slot B.
 template <int B>
-__device__ __forceinline__ int build_warp_list(const unsigned char* s_mask,
-                                               typename ListEntry<B>::T* list) {
+__device__ __forceinline__ int build_warp_list(const unsigned char* s_mask, ListEntry* list) {
   static_assert(B == 128 || B == 256 || B == 512, "tile batch of 128, 256 or 512 splats");
   constexpr int P = B / 32;
   constexpr int NW = P >= 8 ? P / 8 : 1;
@@ -195,18 +213,21 @@ __device__ __forceinline__ int build_warp_list(const unsigned char* s_mask,
     unsigned long long bw = bits[w];
     while (bw) {
       const int bb = __ffsll((long long)bw) - 1;
-      list[pos++] = (typename ListEntry<B>::T)(P * lane + 8 * w + (bb >> 3));
+      list[pos++] = (ListEntry)(16 * (P * lane + 8 * w + (bb >> 3)));
       bw &= bw - 1;
     }
   }
+  const int total = __shfl_sync(0xffffffffu, incl, 31);
+  if (lane < 4) list[total + lane] = (ListEntry)(16 * B);
   __syncwarp();
-  return __shfl_sync(0xffffffffu, incl, 31);
+  return total;
 }
 
+// The lane's first pixel; its second is four rows below.
 __device__ __forceinline__ void pixel_of(int tile, int tiles_x, int& px, int& py) {
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   px = (tile % tiles_x) * VEG_TILE + (w & 1) * 8 + (l & 7);
-  py = (tile / tiles_x) * VEG_TILE + (w >> 1) * 4 + (l >> 3);
+  py = (tile / tiles_x) * VEG_TILE + (w >> 1) * 8 + (l >> 3);
 }
 
 struct CompArgs {
@@ -223,78 +244,149 @@ struct CompArgs {
   float bg0, bg1, bg2;
 };
 
-// Loads tables [lut0, lut0 + ntg) into shared memory; slots past ntg and
-// table indices outside [0, n_tf) read as fully transparent.
-template <int TG>
-__device__ __forceinline__ void stage_luts(const CompArgs& A, int lut0, int ntg, float4* s_lut) {
-  const int L = A.lut_size;
-  for (int e = threadIdx.x; e < TG * L; e += blockDim.x) {
-    const int t = e / L, k = e - t * L, ti = lut0 + t;
-    s_lut[e] = (t < ntg && ti >= 0 && ti < A.n_tf) ? __ldg(&A.lut[(int64_t)ti * L + k])
-                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
+// The work item of a CTA: its tile, output image and table.
+struct WorkItem {
+  int px, py;           // the lane's first pixel
+  int width, height;
+  float tx0, ty0;       // the tile's first pixel
+  long long image;      // first pixel of the output image
+  int2 rg;              // the tile's list
+};
+__device__ __forceinline__ WorkItem work_item(const CompArgs& A, float4* s_lut) {
+  WorkItem w;
+  const int item = (int)blockIdx.x;
+  const int wi = A.order ? A.order[item] : item;  // global tile id
+  const int view = view_of_tile(A.vm, wi), tile = wi - A.vm.tile_off[view];
+  const int tiles_x = A.vm.tiles_x[view], t = (int)blockIdx.z;
+  w.width = A.vm.width[view];
+  w.height = A.vm.height[view];
+  w.rg = A.ranges[wi];
+  w.image = A.vm.pix_off[view] + (long long)t * w.width * w.height;
+  pixel_of(tile, tiles_x, w.px, w.py);
+  w.tx0 = (float)((tile % tiles_x) * VEG_TILE);
+  w.ty0 = (float)((tile / tiles_x) * VEG_TILE);
+  // the table into shared memory; an index outside [0, n_tf) reads as fully
+  // transparent
+  const int ti = A.view_tf ? A.view_tf[view] : t;
+  const bool ok = ti >= 0 && ti < A.n_tf;
+  for (int e = threadIdx.x; e < A.lut_size; e += kCompThreads)
+    s_lut[e] = ok ? __ldg(&A.lut[(int64_t)ti * A.lut_size + e]) : make_float4(0.f, 0.f, 0.f, 0.f);
+  return w;
 }
 
-// Stages splat `i` of the tile list into batch slot `s`: geometry,
-// per-TF colour and A w (and, for the backward, the slopes), the exponent
-// cutoff and the warp-block mask.  Returns the record index.
-//
-// The forward (BWD = false) reads the group's tables from shared memory
-// (`lut`, TG tables of L entries, transparent where the group has no table).
-// The backward reads them from global memory through the L1 cache (`lut`
-// points at the group's first table; bit t of `valid` says whether table t
-// exists, a missing one reads as transparent): the 16 KB this frees at four
-// tables lets four backward CTAs share an SM instead of three.
-//
-// Shading (Eq. 2, LIT): the forward stages the shaded colour s_d C(v) + s_s;
-// the backward stages the unshaded C(v) and (s_d, s_s) in s_sh, with the
-// colour slopes already scaled by s_d.  Without shading s_sh is unused.
-template <int TG, int B, bool BWD, bool LIT>
-__device__ __forceinline__ uint32_t stage_splat(const CompArgs& A, int i, int s, const float4* lut,
-                                                unsigned valid, float tx0, float ty0,
-                                                float4* s_geo, float2* s_c, float4* s_col,
-                                                float4* s_slope, float2* s_sh,
-                                                unsigned char* s_mask) {
-  const int L = A.lut_size;
-  const uint32_t g = A.vals[i];
-  const float4 ge = A.geo[g], au = A.aux[g];
-  s_geo[s] = make_float4(ge.x, ge.y, -0.5f * au.x, -au.y);
-  const TfPos q = tf_pos(au.w, L);
-  const float sl = (au.w >= 0.0f && au.w <= 1.0f) ? (float)(L - 1) : 0.0f;
-  float2 sh = make_float2(1.0f, 0.0f);
-  if (LIT) sh = A.shade[g];
-  if (LIT && BWD) s_sh[s] = sh;
-  const float slc = LIT ? sl * sh.x : sl;  // colour slope scale
-  float max_aw = 0.0f;
+// Asynchronous copies of a chunk's records into shared memory: each lane
+// fetches its own record of the next chunk while the warp walks the current
+// one, and alone reads it back, so the gather's latency (a list entry, then
+// two or three reads at its record) stays off the warp's path.
+template <int N>
+__device__ __forceinline__ void async_copy(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(N) : "memory");
+}
+__device__ __forceinline__ void async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void async_wait() {
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+// One record on its way or arrived: geo and aux, and its shading factors.
+struct RawSlot {
+  float4* geo;  // geo[0]: geo, geo[32]: aux
+  float2* sh;
+};
+template <bool LIT>
+__device__ __forceinline__ void fetch_record(const CompArgs& A, RawSlot s, uint32_t g) {
+  async_copy<16>(s.geo, A.geo + g);
+  async_copy<16>(s.geo + 32, A.aux + g);
+  if (LIT) async_copy<8>(s.sh, A.shade + g);
+}
+
+// A record's colour and opacity under the item's table: lo and hi are the
+// table entries around its scalar, aw = A w.
+struct SplatTf {
+  float4 lo, hi;
+  TfPos q;
+  float aw;
+};
+__device__ __forceinline__ SplatTf splat_tf(const float4* lut, int L, float v, float w) {
+  SplatTf s;
+  s.q = tf_pos(v, L);
+  s.lo = lut[s.q.k];
+  s.hi = lut[s.q.k + 1];
+  s.aw = mul(lerp_rn(s.lo.w, s.hi.w, s.q), w);
+  return s;
+}
+
+// A conic with a NaN (an overflowed covariance) gives every pixel power NaN,
+// which Eq. 1 reads as G = 1: it is staged as the zero conic.
+__device__ __forceinline__ float4 clean_conic(float4 au) {
+  if (!(au.x == au.x && au.y == au.y && au.z == au.z)) au.x = au.y = au.z = 0.0f;
+  return au;
+}
+
+// Records of a batch on their way to shared memory: each thread fetches the
+// records of its own batch slots with asynchronous copies while the warps
+// walk the batch before, and alone reads them back, so the gather's latency
+// (a list entry, then two or three 16-byte reads at its record) stays off
+// the staging between two barriers.
+template <int B, bool LIT>
+struct Prefetch {
+  static constexpr int N = B / kCompThreads;  // slots per thread
+  float4* raw;       // [2][B]: geo, aux
+  float2* raw_sh;    // [B] (LIT)
+  uint32_t next[N];  // record of each slot in the batch to fetch next
+
+  static __device__ __forceinline__ int slot(int r) { return (int)threadIdx.x + kCompThreads * r; }
+  // the list entries of a batch of cnt splats at list index first
+  __device__ __forceinline__ void index(const CompArgs& A, int first, int cnt) {
 #pragma unroll
-  for (int t = 0; t < TG; ++t) {
-    float4 lo, hi;
-    if (BWD) {
-      const bool ok = (valid >> t) & 1u;
-      lo = ok ? __ldg(&lut[t * L + q.k]) : make_float4(0.f, 0.f, 0.f, 0.f);
-      hi = ok ? __ldg(&lut[t * L + q.k + 1]) : make_float4(0.f, 0.f, 0.f, 0.f);
-    } else {
-      lo = lut[t * L + q.k];
-      hi = lut[t * L + q.k + 1];
-    }
-    const float Aop = lerp_rn(lo.w, hi.w, q);
-    const float aw = mul(Aop, ge.w);
-    float r = lerp_rn(lo.x, hi.x, q), gc = lerp_rn(lo.y, hi.y, q), b = lerp_rn(lo.z, hi.z, q);
-    if (LIT && !BWD) {
-      r = __fmaf_rn(sh.x, r, sh.y);
-      gc = __fmaf_rn(sh.x, gc, sh.y);
-      b = __fmaf_rn(sh.x, b, sh.y);
-    }
-    s_col[t * B + s] = make_float4(r, gc, b, aw);
-    if (BWD)
-      s_slope[t * B + s] = make_float4(slc * (hi.x - lo.x), slc * (hi.y - lo.y),
-                                            slc * (hi.z - lo.z), ge.w * sl * (hi.w - lo.w));
-    max_aw = fmaxf(max_aw, aw);
+    for (int r = 0; r < N; ++r)
+      if (slot(r) < cnt) next[r] = __ldg(&A.vals[first + slot(r)]);
   }
-  const float cut = power_cutoff(max_aw);
-  s_c[s] = make_float2(-0.5f * au.z, cut);
-  s_mask[s] = (unsigned char)warp_block_mask<BWD>(ge.x - tx0, ge.y - ty0, au.x, au.y, au.z, cut);
-  return g;
+  __device__ __forceinline__ void fetch(const CompArgs& A, int cnt) {
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+      const int s = slot(r);
+      if (s >= cnt) continue;
+      async_copy<16>(raw + s, A.geo + next[r]);
+      async_copy<16>(raw + B + s, A.aux + next[r]);
+      if (LIT) async_copy<8>(raw_sh + s, A.shade + next[r]);
+    }
+    async_commit();
+  }
+};
+
+// Stages a fetched record into batch slot `s`: the exponent's coefficients,
+// the colour and A w under the item's table, and the mask of the warp blocks
+// that it can reach.  LIT: the shaded colour s_d C(v) + s_s (Eq. 2).
+template <int B, bool LIT>
+__device__ __forceinline__ void stage_splat(float4 ge, float4 au, float2 sh, int s,
+                                            const float4* lut, int L, float tx0, float ty0,
+                                            float4* s_geo, float2* s_ca, float4* s_col,
+                                            unsigned char* s_mask) {
+  const SplatTf t = splat_tf(lut, L, au.w, ge.w);
+  float r = lerp_rn(t.lo.x, t.hi.x, t.q), g = lerp_rn(t.lo.y, t.hi.y, t.q),
+        b = lerp_rn(t.lo.z, t.hi.z, t.q);
+  if (LIT) {
+    r = __fmaf_rn(sh.x, r, sh.y);
+    g = __fmaf_rn(sh.x, g, sh.y);
+    b = __fmaf_rn(sh.x, b, sh.y);
+  }
+  const float cut = power_cutoff(t.aw);
+  s_mask[s] = (unsigned char)warp_block_mask(ge.x - tx0, ge.y - ty0, Reach(au.x, au.y, au.z, cut));
+  au = clean_conic(au);
+  s_geo[s] = make_float4(ge.x, ge.y, -0.5f * au.x, -au.y);
+  s_ca[s] = make_float2(-0.5f * au.z, t.aw);
+  s_col[s] = make_float4(r, g, b, cut);
+}
+
+// Entry of a shared array at 16 times its slot (ListEntry).
+__device__ __forceinline__ float4 at16(const float4* a, unsigned off) {
+  return *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(a) + off);
+}
+__device__ __forceinline__ float2 at16(const float2* a, unsigned off) {
+  return *reinterpret_cast<const float2*>(reinterpret_cast<const char*>(a) + (off >> 1));
 }
 
 // ---------------------------------------------------------------------------
@@ -305,155 +397,149 @@ __device__ __forceinline__ uint32_t stage_splat(const CompArgs& A, int i, int s,
 // pixel's termination, the method's own count), iterated pairs (walked by
 // the warp lists), pairs above the cutoff, alpha evaluations, blended pairs.
 //
-// Resident CTAs per SM: 5 for one TF (48 registers; the extra CTA hides the
-// batch barriers, 7% faster than 4 on the training step), 4 for 2-4 TFs,
-// 2 for 8.
-template <int TG, int B, bool STATS, bool LIT>
-__global__ void __launch_bounds__(256, (TG >= 8 ? 2 : (TG == 1 ? 5 : 4)))
+// The transmittance of a terminated pixel is kept with its sign set:
+// T (1 - alpha) is then below the stop at every later splat, so the pair
+// needs no separate live flag.
+template <int B, bool STATS, bool LIT>
+__global__ void __launch_bounds__(kCompThreads, 7)
     composite_fwd_kernel(CompArgs A, float4* __restrict__ out,
                          int32_t* __restrict__ n_contrib, unsigned long long* __restrict__ stats) {
   pdl_enter();
-  extern __shared__ float4 s_lut[];  // [TG][L]
-  __shared__ float4 s_geo[B];        // u_x, u_y, -a/2, -b
-  __shared__ float2 s_c[B];          // -c/2, exponent cutoff
-  __shared__ float4 s_col[TG * B];
-  __shared__ __align__(16) unsigned char s_mask[B];
-  __shared__ typename ListEntry<B>::T s_list[kWarps][B];
-  const int t0 = blockIdx.z * TG;  // first output image of the group
-  const int ntg = A.view_tf ? 1 : min(TG, A.n_tf - t0);
+  constexpr int P = B + 1;
+  extern __shared__ float4 smem[];
+  float4* s_geo = smem;       // [P]: u_x, u_y, -a/2, -b
+  float4* s_col = s_geo + P;  // [P]: r, g, b, cutoff
+  Prefetch<B, LIT> pre;
+  pre.raw = s_col + P;        // [2][B]
+  float4* s_lut = pre.raw + 2 * B;                                 // [L]
+  float2* s_ca = reinterpret_cast<float2*>(s_lut + A.lut_size);    // [P]: -c/2, A w
+  pre.raw_sh = s_ca + P;                                           // [B] (LIT)
+  ListEntry* s_list = reinterpret_cast<ListEntry*>(pre.raw_sh + (LIT ? B : 0));  // [kWarps][B + 4]
+  unsigned char* s_mask = reinterpret_cast<unsigned char*>(s_list + kWarps * (B + 4));  // [B]
   const int warp = threadIdx.x >> 5;
-  unsigned long long n_vis = 0, n_it = 0, n_eval = 0, n_alpha = 0, n_blend = 0;
-  {
-    const int item = (int)blockIdx.x;
-    const int wi = A.order ? A.order[item] : item;  // global tile id
-    const int view = view_of_tile(A.vm, wi), tile = wi - A.vm.tile_off[view];
-    const int tiles_x = A.vm.tiles_x[view], width = A.vm.width[view], height = A.vm.height[view];
-    const long long pix0 = A.vm.pix_off[view];          // the view's first output pixel
-    const int lut0 = A.view_tf ? A.view_tf[view] : t0;  // first table of the group
-    stage_luts<TG>(A, lut0, ntg, s_lut);
-    int px, py;
-    pixel_of(tile, tiles_x, px, py);
-    const float tx0 = (float)((tile % tiles_x) * VEG_TILE);
-    const float ty0 = (float)((tile / tiles_x) * VEG_TILE);
-    const bool inside = px < width && py < height;
-    const float2 fxy = make_float2((float)px, (float)py);
-    const int2 rg = A.ranges[wi];
-    float T[TG], Cr[TG], Cg[TG], Cb[TG];
-    int last[TG];
+  ListEntry* my_list = s_list + warp * (B + 4);
+  unsigned long long n_vis = 0, n_it = 0, n_eval = 0, n_blend = 0;
+  const WorkItem W = work_item(A, s_lut);
+  if (threadIdx.x == 0) {  // the padding slot: A w = 0 never blends
+    s_geo[B] = s_col[B] = make_float4(0.f, 0.f, 0.f, 0.f);
+    s_ca[B] = make_float2(0.f, 0.f);
+  }
+  const float2 fx = dup((float)W.px), fy = make_float2((float)W.py, (float)(W.py + 4));
+  const int n = W.rg.y - W.rg.x;  // the list's length
+  pre.index(A, W.rg.x, n);
+  pre.fetch(A, n);
+  pre.index(A, W.rg.x + B, n - B);
+  float T[2], Cr[2], Cg[2], Cb[2];
+  int last[2];
 #pragma unroll
-    for (int t = 0; t < TG; ++t) {
-      T[t] = 1.0f;
-      Cr[t] = Cg[t] = Cb[t] = 0.0f;
-      last[t] = 0;
-    }
-    unsigned act = inside ? ((1u << ntg) - 1u) : 0u;
+  for (int i = 0; i < 2; ++i) {
+    T[i] = W.px < W.width && W.py + 4 * i < W.height ? 1.0f : -1.0f;
+    Cr[i] = Cg[i] = Cb[i] = 0.0f;
+    last[i] = 0;
+  }
 
-    for (int start = rg.x; start < rg.y; start += B) {
-      if (__syncthreads_count(act != 0u) == 0) break;
-      const int cnt = min(B, rg.y - start);
+  for (int start = 0; start < n; start += B) {
+    if (__syncthreads_count(T[0] > 0.0f || T[1] > 0.0f) == 0) break;
+    const int cnt = min(B, n - start);
+    async_wait();
 #pragma unroll
-      for (int r = 0; r < (B + 255) / 256; ++r) {
-        const int sl = (int)threadIdx.x + 256 * r;
-        if (sl < cnt)
-          stage_splat<TG, B, false, LIT>(A, start + sl, sl, s_lut, 0xffu, tx0, ty0, s_geo, s_c,
-                                         s_col, nullptr, nullptr, s_mask);
-        else if (sl < B)
-          s_mask[sl] = 0;
+    for (int r = 0; r < pre.N; ++r) {
+      const int sl = pre.slot(r);
+      if (sl < cnt)
+        stage_splat<B, LIT>(pre.raw[sl], pre.raw[B + sl],
+                            LIT ? pre.raw_sh[sl] : make_float2(1.f, 0.f), sl, s_lut, A.lut_size,
+                            W.tx0, W.ty0, s_geo, s_ca, s_col, s_mask);
+      else
+        s_mask[sl] = 0;
+    }
+    pre.fetch(A, n - start - B);
+    pre.index(A, W.rg.x + start + 2 * B, n - start - 2 * B);
+    __syncthreads();
+    const int nw = build_warp_list<B>(s_mask, my_list);
+    int lb[2] = {-1, -1};  // offset of the pixel's last blended splat of this batch
+    const bool act0[2] = {T[0] > 0.0f, T[1] > 0.0f};
+    int jstop[2] = {cnt, cnt};  // 1 + batch position where the pixel terminated
+    // four splats per step: first everything that does not depend on the
+    // transmittance (exponents, Gaussians, alpha: independent, so they
+    // overlap), then the blends in list order; a splat that no pixel of the
+    // warp blends is passed over by a vote (one vote for all four, or all
+    // votes ahead of the blends, measured 3-10% slower, two splats per step
+    // 4%).  The exponents
+    // are formed per pixel from (u, -a/2, -b) and -c/2: staging every value
+    // twice for two-wide operations saves five instructions and costs 24
+    // bytes of shared-memory reads per splat, the same time.
+    for (int k = 0; k < nw; k += 4) {
+      const uint2 en = *reinterpret_cast<const uint2*>(my_list + k);
+      const unsigned off[4] = {en.x & 0xffffu, en.x >> 16, en.y & 0xffffu, en.y >> 16};
+      float2 al[4];
+      bool ok[4][2];
+      float4 col[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        col[m] = at16(s_col, off[m]);
+        const float4 g = at16(s_geo, off[m]);
+        const float2 h = at16(s_ca, off[m]);
+        const float dx = sub(g.x, fx.x);
+        const float2 dy = make_float2(sub(g.y, fy.x), sub(g.y, fy.y));
+        const float dxx = mul(dx, dx);
+        const float2 dyy = mul2(dy, dy);
+        const float2 p = make_float2(
+            __fmaf_rn(g.z, dxx, __fmaf_rn(h.x, dyy.x, mul(g.w, mul(dx, dy.x)))),
+            __fmaf_rn(g.z, dxx, __fmaf_rn(h.x, dyy.y, mul(g.w, mul(dx, dy.y)))));
+        const float2 x = mul2(p, dup(kLog2e));
+        al[m] = make_float2(fminf(kAlphaMax, mul(h.y, ex2_approx(x.x))),
+                            fminf(kAlphaMax, mul(h.y, ex2_approx(x.y))));
+        ok[m][0] = !(p.x > 0.0f) && !(al[m].x < kAlphaMin);
+        ok[m][1] = !(p.y > 0.0f) && !(al[m].y < kAlphaMin);
+        if (STATS && k + m < nw) {
+          const float cut = col[m].w, pp[2] = {p.x, p.y};
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+            if (T[i] > 0.0f) {
+              ++n_it;
+              n_eval += (unsigned)(pp[i] <= 0.0f && pp[i] >= cut);
+            }
+        }
       }
-      __syncthreads();
-      const int nw = build_warp_list<B>(s_mask, s_list[warp]);
-      const bool act0 = act != 0u;
-      int jstop = cnt;  // 1 + batch position where this pixel terminated
-      // Eq. 1 update of every live TF of the group with splat j (exponent G).
-      auto blend = [&](int j, float G) {
 #pragma unroll
-        for (int t = 0; t < TG; ++t) {
-          if (!(act & (1u << t))) continue;
-          if (STATS) ++n_alpha;
-          const float4 c = s_col[t * B + j];
-          const float alpha = fminf(kAlphaMax, mul(c.w, G));
-          if (alpha < kAlphaMin) continue;
-          const float test = mul(T[t], sub(1.0f, alpha));
-          if (test < kTMin) {
-            act &= ~(1u << t);
-            continue;
+      for (int m = 0; m < 4; ++m) {
+        if (!__any_sync(0xffffffffu, ok[m][0] || ok[m][1])) continue;
+        // Eq. 1 update of the two pixels
+        const float4 c = col[m];
+        const float2 Tt = make_float2(T[0], T[1]);
+        const float2 test2 = mul2(Tt, sub2(dup(1.0f), al[m])), wgt2 = mul2(al[m], Tt);
+        const float test[2] = {test2.x, test2.y}, wgt[2] = {wgt2.x, wgt2.y};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const bool stop = test[i] < kTMin;
+          if (STATS && ok[m][i] && !stop) ++n_blend;
+          if (STATS && ok[m][i] && stop && T[i] > 0.0f) jstop[i] = (int)(off[m] >> 4) + 1;
+          if (ok[m][i] && stop) T[i] = -fabsf(T[i]);
+          if (ok[m][i] && !stop) {
+            Cr[i] = __fmaf_rn(c.x, wgt[i], Cr[i]);
+            Cg[i] = __fmaf_rn(c.y, wgt[i], Cg[i]);
+            Cb[i] = __fmaf_rn(c.z, wgt[i], Cb[i]);
+            T[i] = test[i];
+            lb[i] = (int)off[m];
           }
-          const float wgt = mul(alpha, T[t]);
-          Cr[t] = __fmaf_rn(c.x, wgt, Cr[t]);
-          Cg[t] = __fmaf_rn(c.y, wgt, Cg[t]);
-          Cb[t] = __fmaf_rn(c.z, wgt, Cb[t]);
-          T[t] = test;
-          last[t] = start + j - rg.x + 1;
-          if (STATS) ++n_blend;
-        }
-        if (STATS && !act) jstop = j + 1;
-      };
-      // four (then two, then one) splats per step: their exponents are
-      // independent and overlap, the blends stay in list order
-      int k = 0;
-      for (; k + 3 < nw && act; k += 4) {
-        const int j0 = s_list[warp][k], j1 = s_list[warp][k + 1];
-        const int j2 = s_list[warp][k + 2], j3 = s_list[warp][k + 3];
-        const float4 g0 = s_geo[j0], g1 = s_geo[j1], g2 = s_geo[j2], g3 = s_geo[j3];
-        const float2 c0 = s_c[j0], c1 = s_c[j1], c2 = s_c[j2], c3 = s_c[j3];
-        float2 d0, d1, d2, d3, q0, q1, q2, q3;
-        float x0, x1, x2, x3;
-        const float p0 = power_at(g0.x, g0.y, fxy, g0.z, g0.w, c0.x, d0, q0, x0);
-        const float p1 = power_at(g1.x, g1.y, fxy, g1.z, g1.w, c1.x, d1, q1, x1);
-        const float p2 = power_at(g2.x, g2.y, fxy, g2.z, g2.w, c2.x, d2, q2, x2);
-        const float p3 = power_at(g3.x, g3.y, fxy, g3.z, g3.w, c3.x, d3, q3, x3);
-        const bool e0 = !(p0 < c0.y || p0 > 0.0f), e1 = !(p1 < c1.y || p1 > 0.0f);
-        const bool e2 = !(p2 < c2.y || p2 > 0.0f), e3 = !(p3 < c3.y || p3 > 0.0f);
-        if (STATS) {
-          n_it += 4;
-          n_eval += (unsigned)e0 + (unsigned)e1 + (unsigned)e2 + (unsigned)e3;
-        }
-        if (e0) blend(j0, gauss_of(p0));
-        if (e1 && act) blend(j1, gauss_of(p1));
-        if (e2 && act) blend(j2, gauss_of(p2));
-        if (e3 && act) blend(j3, gauss_of(p3));
-      }
-      for (; k + 1 < nw && act; k += 2) {
-        const int j0 = s_list[warp][k], j1 = s_list[warp][k + 1];
-        const float4 g0 = s_geo[j0], g1 = s_geo[j1];
-        const float2 c0 = s_c[j0], c1 = s_c[j1];
-        float2 d0, d1, q0, q1;
-        float x0, x1;
-        const float p0 = power_at(g0.x, g0.y, fxy, g0.z, g0.w, c0.x, d0, q0, x0);
-        const float p1 = power_at(g1.x, g1.y, fxy, g1.z, g1.w, c1.x, d1, q1, x1);
-        const bool e0 = !(p0 < c0.y || p0 > 0.0f), e1 = !(p1 < c1.y || p1 > 0.0f);
-        if (STATS) {
-          n_it += 2;
-          n_eval += (unsigned)e0 + (unsigned)e1;
-        }
-        if (e0) blend(j0, gauss_of(p0));
-        if (e1 && act) blend(j1, gauss_of(p1));
-      }
-      if (k < nw && act) {
-        const int j = s_list[warp][k];
-        const float4 sg = s_geo[j];
-        const float2 sc = s_c[j];
-        float2 d, d2;
-        float dxy;
-        const float power = power_at(sg.x, sg.y, fxy, sg.z, sg.w, sc.x, d, d2, dxy);
-        if (STATS) ++n_it;
-        if (!(power < sc.y || power > 0.0f)) {
-          if (STATS) ++n_eval;
-          blend(j, gauss_of(power));
         }
       }
-      if (STATS && act0) n_vis += (unsigned long long)jstop;
+      if (!__any_sync(0xffffffffu, T[0] > 0.0f || T[1] > 0.0f)) break;
     }
-    if (inside) {
 #pragma unroll
-      for (int t = 0; t < TG; ++t) {
-        if (t >= ntg) break;
-        const int64_t o = pix0 + ((int64_t)(t0 + t) * height + py) * width + px;
-        out[o] = make_float4(add(Cr[t], mul(T[t], A.bg0)), add(Cg[t], mul(T[t], A.bg1)),
-                             add(Cb[t], mul(T[t], A.bg2)), T[t]);
-        n_contrib[o] = last[t];
-      }
-    }
+    for (int i = 0; i < 2; ++i)
+      if (lb[i] >= 0) last[i] = start + (lb[i] >> 4) + 1;
+    if (STATS) n_vis += (act0[0] ? (unsigned)jstop[0] : 0u) + (act0[1] ? (unsigned)jstop[1] : 0u);
+  }
+  async_wait();  // no copy in flight past the CTA's end
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    if (W.px >= W.width || W.py + 4 * i >= W.height) continue;
+    const int64_t o = W.image + (int64_t)(W.py + 4 * i) * W.width + W.px;
+    const float Tf = fabsf(T[i]);
+    out[o] = make_float4(add(Cr[i], mul(Tf, A.bg0)), add(Cg[i], mul(Tf, A.bg1)),
+                         add(Cb[i], mul(Tf, A.bg2)), Tf);
+    n_contrib[o] = last[i];
   }
   if (STATS) {
 #pragma unroll
@@ -461,14 +547,13 @@ __global__ void __launch_bounds__(256, (TG >= 8 ? 2 : (TG == 1 ? 5 : 4)))
       n_vis += __shfl_down_sync(0xffffffffu, n_vis, o);
       n_it += __shfl_down_sync(0xffffffffu, n_it, o);
       n_eval += __shfl_down_sync(0xffffffffu, n_eval, o);
-      n_alpha += __shfl_down_sync(0xffffffffu, n_alpha, o);
       n_blend += __shfl_down_sync(0xffffffffu, n_blend, o);
     }
     if ((threadIdx.x & 31) == 0) {
       atomicAdd(&stats[0], n_vis);
       atomicAdd(&stats[1], n_it);
       atomicAdd(&stats[2], n_eval);
-      atomicAdd(&stats[3], n_alpha);
+      atomicAdd(&stats[3], n_eval);
       atomicAdd(&stats[4], n_blend);
     }
   }
@@ -478,71 +563,16 @@ __global__ void __launch_bounds__(256, (TG >= 8 ? 2 : (TG == 1 ? 5 : 4)))
 // backward
 // ---------------------------------------------------------------------------
 
-// Sums eight per-lane values over the warp with 9 shuffles: three halving
-// exchanges (offsets 16, 8, 4; each lane keeps the half named by its offset
-// bit and receives the partner's sum of that half), then two full steps
-// (offsets 2, 1).  Lane l returns the warp total of slot l >> 2.
-__device__ __forceinline__ float warp_reduce_scatter8(const float v[8], int lane) {
-  const bool b4 = lane & 16, b2 = lane & 8, b1 = lane & 4;
-  float w[4], x[2];
+// One halving exchange of a warp reduce-scatter: lanes keep the half of the
+// 2 N slots named by their `bit` and add the partner's (lane ^ mask) values.
+template <int N>
+__device__ __forceinline__ void exchange(const float* v, float* w, bool bit, int mask) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float send = b4 ? v[i] : v[i + 4];
-    const float keep = b4 ? v[i + 4] : v[i];
-    w[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+  for (int i = 0; i < N; ++i) {
+    const float send = bit ? v[i] : v[i + N];
+    const float keep = bit ? v[i + N] : v[i];
+    w[i] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
   }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const float send = b2 ? w[i] : w[i + 2];
-    const float keep = b2 ? w[i + 2] : w[i];
-    x[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-  const float send = b1 ? x[0] : x[1];
-  float y = (b1 ? x[1] : x[0]) + __shfl_xor_sync(0xffffffffu, send, 4);
-  y += __shfl_xor_sync(0xffffffffu, y, 2);
-  y += __shfl_xor_sync(0xffffffffu, y, 1);
-  return y;
-}
-
-// The same for sixteen values with 16 shuffles (halving at offsets 16, 8, 4,
-// 2, then one full step at offset 1).  Lane l returns the warp total of
-// slot l >> 1.
-__device__ __forceinline__ float warp_reduce_scatter16(const float v[16], int lane) {
-  const bool b16 = lane & 16, b8 = lane & 8, b4 = lane & 4, b2 = lane & 2;
-  float w[8], x[4], y[2];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float send = b16 ? v[i] : v[i + 8];
-    const float keep = b16 ? v[i + 8] : v[i];
-    w[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float send = b8 ? w[i] : w[i + 4];
-    const float keep = b8 ? w[i + 4] : w[i];
-    x[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const float send = b4 ? x[i] : x[i + 2];
-    const float keep = b4 ? x[i + 2] : x[i];
-    y[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  }
-  const float send = b2 ? y[0] : y[1];
-  float z = (b2 ? y[1] : y[0]) + __shfl_xor_sync(0xffffffffu, send, 2);
-  z += __shfl_xor_sync(0xffffffffu, z, 1);
-  return z;
-}
-
-// Sums one value per splat for two splats (a, b) over the warp with 5
-// shuffles (one halving exchange at offset 16, then full steps at 8, 4, 2,
-// 1).  Lanes 0-15 return the total of a, lanes 16-31 that of b.
-__device__ __forceinline__ float warp_reduce_pair(float a, float b, int lane) {
-  const bool hi = lane & 16;
-  float x = (hi ? b : a) + __shfl_xor_sync(0xffffffffu, hi ? a : b, 16);
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
 }
 
 __device__ __forceinline__ void red_add_v2(float2* p, float a, float b) {
@@ -568,9 +598,19 @@ __device__ __forceinline__ void red_add_v4(float4* p, float a, float b, float c,
 // anyway; Suf grows from the back, so the small terms of deep splats are
 // summed first and keep their relative accuracy (a front-to-back prefix
 // K - S_i would leave them as a difference of two O(1) numbers).  Per splat,
-// the seven screen-space gradients are reduced over the warp, summed over
-// warps in shared memory and added to the per-record gradient buffer once
-// per tile.
+// the seven screen-space gradients are summed over a lane's two pixels,
+// reduced over the warp, summed over warps in shared memory and added to the
+// per-record gradient buffer once per tile.
+//
+// The screen gradients are linear in the sums of dp = dL/dpower times 1, dx,
+// dy, dx^2, dx dy, dy^2 (d = u - pixel; power = -a/2 dx^2 - b dx dy - c/2
+// dy^2), with per-splat coefficients applied once at the flush.  The eight
+// pixels of a block's column share dx, so the warp reduces in two stages:
+// over a column (lanes 8 and 16 apart) the four sums of dp, dp dy, dp dy^2
+// and dL/dv, then, multiplied by the column's dx, over the eight columns.
+// Two splats go through one reduction: 41 instructions against 62 for a
+// direct reduce-scatter of the seven products, and four products fewer per
+// splat.
 //
 // The weight needs no sum of its own: below the clamp alpha = A w e^power,
 // so dalpha/dw = alpha / w = (dalpha/dpower) / w and dL/dw is the summed
@@ -579,261 +619,275 @@ __device__ __forceinline__ void red_add_v4(float4* p, float a, float b, float c,
 //
 // Shaded (LIT): the blended colour is s_d C + s_s, so c.g = s_d (C.g) + s_s
 // (g_r + g_g + g_b), dL/dC = s_d alpha T g, and the pair adds alpha T (C.g)
-// to dL/ds_d and alpha T (g_r + g_g + g_b) to dL/ds_s.  dL/ds_d takes the
-// eighth slot of the 16-slot reduce-scatter and dL/ds_s a separate pair
-// reduction; the two shading sums go to grad_shade.
+// to dL/ds_d and alpha T (g_r + g_g + g_b) to dL/ds_s, reduced beside the
+// others; the two shading sums go to grad_shade.
 //
 // stats (instrumented build): replayed pairs (list positions below the
 // pixel's last contribution), iterated pairs, pairs above the cutoff, alpha
 // evaluations, blended pairs, blended pairs below the clamp, pairs with a
 // nonzero screen-space gradient.
-//
-// Resident CTAs per SM: 4 (64 registers; 8 warps per SM more than 3 CTAs
-// hide the walk's dependent-issue latency, 7% faster on the training step),
-// 3 for the shaded and instrumented builds of a 4-TF group, which would
-// spill at 64 registers.
-template <int TG, int B, bool STATS, bool LIT>
-__global__ void __launch_bounds__(256, ((LIT || STATS) && TG >= 4) ? 3 : 4)
+template <bool LIT>
+struct BwdWarp {
+  static constexpr int kAcc = LIT ? 12 : 8;  // accumulator slots per splat
+  float4 u[34];   // u_x, u_x, u_y, u_y
+  float4 q[34];   // -a/2, -a/2, -b, -b
+  float4 r[34];   // -c/2, -c/2, list position (bits), cutoff
+  float4 c0[34];  // r, r, g, g
+  float4 c1[34];  // b, b, Aw, Aw
+  float4 d0[34];  // dr/dv, dr/dv, dg/dv, dg/dv (times s_d)
+  float4 d1[34];  // db/dv, db/dv, w dA/dv, w dA/dv
+  float4 sh[LIT ? 34 : 1];  // s_d, s_d, s_s, s_s
+  float4 raw[2][2 * 32];    // records, alternate chunks
+  float acc[34 * kAcc];     // gradient sums of the chunk's splats
+};
+
+template <bool STATS, bool LIT>
+__global__ void __launch_bounds__(kCompThreads, 4)
     composite_bwd_kernel(CompArgs A, const float4* __restrict__ out,
                          const int32_t* __restrict__ n_contrib, const float4* __restrict__ dout,
                          float4* __restrict__ grad2d, float2* __restrict__ grad_shade,
                          unsigned long long* __restrict__ stats) {
   pdl_enter();
-  constexpr int kAcc = LIT ? 12 : 8;  // accumulator slots per splat
-  unsigned long long n_rep = 0, n_it = 0, n_eval = 0, n_alpha = 0, n_blend = 0, n_free = 0,
-                     n_grad = 0;
+  using Warp = BwdWarp<LIT>;
+  constexpr int kAcc = Warp::kAcc;
+  unsigned long long n_rep = 0, n_it = 0, n_eval = 0, n_blend = 0, n_free = 0, n_grad = 0;
   extern __shared__ float4 smem[];
-  using LT = typename ListEntry<B>::T;
-  float4* s_col = smem;                                // [TG][B]: rgb, A w
-  float4* s_slope = s_col + TG * B;                    // [TG][B]: drgb/dv, w dA/dv
-  float4* s_geo = s_slope + TG * B;                    // [B]: u, -a/2, -b
-  float2* s_c = reinterpret_cast<float2*>(s_geo + B);  // [B]: -c/2, cutoff
-  float2* s_sh = s_c + B;                              // [B]: s_d, s_s (LIT)
-  float* s_acc = reinterpret_cast<float*>(s_sh + (LIT ? B : 0));  // [B][kAcc] gradient sums
-  uint32_t* s_idx = reinterpret_cast<uint32_t*>(s_acc + kAcc * B);  // [B]: record index
-  unsigned char* s_mask = reinterpret_cast<unsigned char*>(s_idx + B);  // [B]
-  LT* s_lists = reinterpret_cast<LT*>(s_mask + B);  // [kWarps][B]
-  __shared__ int s_maxnc;
-
-  const int t0 = blockIdx.z * TG;  // first output image of the group
-  const int ntg = A.view_tf ? 1 : min(TG, A.n_tf - t0);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  LT* my_list = s_lists + warp * B;
-  for (int e = threadIdx.x; e < kAcc * B; e += 256) s_acc[e] = 0.0f;
-  {
-    const int item = (int)blockIdx.x;
-    const int wi = A.order ? A.order[item] : item;  // global tile id
-    const int view = view_of_tile(A.vm, wi), tile = wi - A.vm.tile_off[view];
-    const int tiles_x = A.vm.tiles_x[view], width = A.vm.width[view], height = A.vm.height[view];
-    const long long pix0 = A.vm.pix_off[view];          // the view's first output pixel
-    const int lut0 = A.view_tf ? A.view_tf[view] : t0;  // first table of the group
-    const float4* g_lut = A.lut + (int64_t)lut0 * A.lut_size;  // the group's tables
-    unsigned valid = 0u;
-#pragma unroll
-    for (int t = 0; t < TG; ++t)
-      if (t < ntg && lut0 + t >= 0 && lut0 + t < A.n_tf) valid |= 1u << t;
-    if (threadIdx.x == 0) s_maxnc = 0;
-    int px, py;
-    pixel_of(tile, tiles_x, px, py);
-    const float tx0 = (float)((tile % tiles_x) * VEG_TILE);
-    const float ty0 = (float)((tile / tiles_x) * VEG_TILE);
-    const bool inside = px < width && py < height;
-    const float2 fxy = make_float2((float)px, (float)py);
-    const int2 rg = A.ranges[wi];
+  Warp& S = reinterpret_cast<Warp*>(smem)[warp];
+  float4* s_lut = reinterpret_cast<float4*>(reinterpret_cast<Warp*>(smem) + kWarps);
+  float2* s_sh = reinterpret_cast<float2*>(s_lut + A.lut_size) + threadIdx.x;
+  const WorkItem W = work_item(A, s_lut);
+  const float bx0 = W.tx0 + (float)((warp & 1) * 8), by0 = W.ty0 + (float)((warp >> 1) * 8);
+  const float2 fx = dup((float)W.px), fy = make_float2((float)W.py, (float)(W.py + 4));
 
-    // per TF: transmittance behind the splats walked so far, the suffix sum,
-    // the upstream colour gradient and n_contrib
-    float T[TG], Suf[TG], gr[TG], gg[TG], gb[TG], gs[TG];
-    int nc[TG];
-    int my_max = 0;
+  // per pixel: transmittance behind the splats walked so far, the negated
+  // suffix sum, the upstream colour gradient and n_contrib
+  float4 ov[2], dv4[2];
+  int nc[2];
 #pragma unroll
-    for (int t = 0; t < TG; ++t) {
-      T[t] = 1.0f;
-      Suf[t] = 0.0f;
-      gr[t] = gg[t] = gb[t] = gs[t] = 0.0f;
-      nc[t] = 0;
-      if (inside && t < ntg) {
-        const int64_t o = pix0 + ((int64_t)(t0 + t) * height + py) * width + px;
-        const float4 ov = out[o], dv4 = dout[o];
-        nc[t] = n_contrib[o];
-        gr[t] = dv4.x;
-        gg[t] = dv4.y;
-        gb[t] = dv4.z;
-        gs[t] = dv4.x + dv4.y + dv4.z;
-        T[t] = ov.w;
-        Suf[t] = ov.w * (A.bg0 * dv4.x + A.bg1 * dv4.y + A.bg2 * dv4.z + dv4.w);
-        my_max = max(my_max, nc[t]);
-      }
-    }
-    if (STATS) n_rep += (unsigned long long)my_max;
-    // loop bounds: a warp walks from its last contribution (all lanes take part
-    // in the reductions); the block stages from its last warp's
-    int warp_max = my_max;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      warp_max = max(warp_max, __shfl_xor_sync(0xffffffffu, warp_max, o));
-    __syncthreads();
-    if (lane == 0) atomicMax(&s_maxnc, warp_max);
-    __syncthreads();
-    const int block_max = s_maxnc;
-
-    // batches from the back: list positions [bstart, bend), slot s = bstart + s
-    for (int bend = block_max; bend > 0; bend -= B) {
-      const int bstart = max(0, bend - B);
-      const int cnt = bend - bstart;
-#pragma unroll
-      for (int r = 0; r < (B + 255) / 256; ++r) {
-        const int sl = (int)threadIdx.x + 256 * r;
-        if (sl < cnt)
-          s_idx[sl] = stage_splat<TG, B, true, LIT>(A, rg.x + bstart + sl, sl, g_lut, valid, tx0,
-                                                    ty0, s_geo, s_c, s_col, s_slope, s_sh, s_mask);
-        else if (sl < B)
-          s_mask[sl] = 0;
-      }
-      __syncthreads();
-      const int nw = build_warp_list<B>(s_mask, my_list);
-      // blend of splat j at list position idx, undone for every TF of the
-      // group: accumulates dL/dG, dL/dv (and dL/ds_d, dL/ds_s) of this pixel
-      auto tf_grads = [&](int j, int idx, float G, float& dG, float& dvv, float& dsd,
-                          float& dss) {
-        float2 sh = make_float2(1.0f, 0.0f);
-        if (LIT) sh = s_sh[j];
-#pragma unroll
-        for (int t = 0; t < TG; ++t) {
-          if (idx >= nc[t]) continue;
-          if (STATS) ++n_alpha;
-          const float4 c = s_col[t * B + j];
-          const float raw = mul(c.w, G);
-          const float alpha = fminf(kAlphaMax, raw);
-          if (alpha < kAlphaMin) continue;
-          if (STATS) {
-            ++n_blend;
-            n_free += (raw <= kAlphaMax);
-          }
-          const float rr = rcp_approx(sub(1.0f, alpha));
-          const float Ti = T[t] * rr;  // transmittance in front of the splat
-          const float wgt = alpha * Ti;
-          const float cgu = c.x * gr[t] + c.y * gg[t] + c.z * gb[t];
-          const float cgd = LIT ? sh.x * cgu + sh.y * gs[t] : cgu;
-          if (LIT) {
-            dsd += wgt * cgu;
-            dss += wgt * gs[t];
-          }
-          const float dalpha = Ti * cgd - Suf[t] * rr;
-          Suf[t] = __fmaf_rn(cgd, wgt, Suf[t]);
-          const float4 sl = s_slope[t * B + j];
-          dvv += wgt * (gr[t] * sl.x + gg[t] * sl.y + gb[t] * sl.z);
-          if (raw <= kAlphaMax) {
-            dvv += dalpha * G * sl.w;
-            dG += dalpha * c.w;
-          }
-          T[t] = Ti;
-        }
-      };
-      // gradient parts of one pair: the exponent gradient dp = dL/dpower
-      // times the offset moments dx, dy, dx^2, dx dy, dy^2 (d = u - pixel),
-      // dL/dv, dp itself (dL/dw times w) (and s_d).  The screen gradients
-      // are linear in these moments with per-splat coefficients (power =
-      // -a/2 dx^2 - b dx dy - c/2 dy^2), applied once per splat at the flush.
-      auto pair_parts = [&](float* v, float dp, float2 d, float2 d2, float dxy, float dvv,
-                            float dsd) {
-        const float2 m = mul2(make_float2(dp, dp), d);
-        v[0] = m.x;
-        v[1] = m.y;
-        v[2] = dp * d2.x;
-        v[3] = dp * dxy;
-        v[4] = dp * d2.y;
-        v[5] = dvv;
-        v[6] = dp;
-        v[7] = LIT ? dsd : 0.0f;
-      };
-      // the warp's list is in list order: skip its entries past the warp's
-      // last contribution, then walk it backwards two splats per step (j0, the
-      // later one, first); independent geometry and exponentials overlap, and
-      // one 16-slot reduce-scatter sums both splats' gradients over the warp
-      int k = nw - 1;
-      while (k >= 0 && bstart + my_list[k] >= warp_max) --k;
-      for (; k >= 0; k -= 2) {
-        const int j0 = my_list[k];
-        const int idx0 = bstart + j0;  // list position
-        const bool has1 = k >= 1;
-        const int j1 = has1 ? my_list[k - 1] : j0;
-        const int idx1 = bstart + j1;
-        if (STATS) n_it += 1 + (unsigned)has1;
-        const float4 sg0 = s_geo[j0], sg1 = s_geo[j1];
-        const float2 sc0 = s_c[j0], sc1 = s_c[j1];
-        float2 d0, d1, q0, q1;
-        float x0, x1;
-        const float p0 = power_at(sg0.x, sg0.y, fxy, sg0.z, sg0.w, sc0.x, d0, q0, x0);
-        const float p1 = power_at(sg1.x, sg1.y, fxy, sg1.z, sg1.w, sc1.x, d1, q1, x1);
-        const bool ev0 = idx0 < my_max && p0 <= 0.0f && p0 >= sc0.y;
-        const bool ev1 = has1 && idx1 < my_max && p1 <= 0.0f && p1 >= sc1.y;
-        const float G0 = ev0 ? gauss_of(p0) : 0.f;
-        const float G1 = ev1 ? gauss_of(p1) : 0.f;
-        float dG0 = 0.f, dv0 = 0.f, dG1 = 0.f, dv1 = 0.f;
-        float dd0 = 0.f, ds0 = 0.f, dd1 = 0.f, ds1 = 0.f;
-        if (ev0) tf_grads(j0, idx0, G0, dG0, dv0, dd0, ds0);
-        if (ev1) tf_grads(j1, idx1, G1, dG1, dv1, dd1, ds1);
-        if (STATS) n_eval += (unsigned)ev0 + (unsigned)ev1;
-        if (STATS) n_grad += (unsigned)(dG0 != 0.f) + (unsigned)(dG1 != 0.f);
-        const float dp0 = dG0 * G0, dp1 = dG1 * G1;
-        bool nz = dp0 != 0.f || dv0 != 0.f || dp1 != 0.f || dv1 != 0.f;
-        if (LIT) nz = nz || dd0 != 0.f || ds0 != 0.f || dd1 != 0.f || ds1 != 0.f;
-        if (__any_sync(0xffffffffu, nz)) {
-          float v[16];
-          pair_parts(v, dp0, d0, q0, x0, dv0, dd0);
-          pair_parts(v + 8, dp1, d1, q1, x1, dv1, dd1);
-          // lane l ends with slot l >> 1 (splat (l >> 4), component (l >> 1) & 7)
-          const float r = warp_reduce_scatter16(v, lane);
-          const int slot = lane >> 1, which = slot >> 3, comp = slot & 7;
-          if ((lane & 1) == 0 && comp < (LIT ? 8 : 7) && (which == 0 || has1))
-            atomicAdd(&s_acc[(which ? j1 : j0) * kAcc + comp], r);
-          if (LIT) {
-            const float rs = warp_reduce_pair(ds0, ds1, lane);
-            if ((lane & 15) == 1 && (lane < 16 || has1))
-              atomicAdd(&s_acc[(lane < 16 ? j0 : j1) * kAcc + 8], rs);
-          }
-        }
-      }
-      __syncthreads();
-#pragma unroll
-      for (int r = 0; r < (B + 255) / 256; ++r) {
-        const int sl = (int)threadIdx.x + 256 * r;
-        if (sl >= cnt) break;
-        float4* acc = reinterpret_cast<float4*>(s_acc) + (kAcc / 4) * sl;
-        const float4 a0 = acc[0], a1 = acc[1];
-        const float4 a2 = LIT ? acc[2] : make_float4(0.f, 0.f, 0.f, 0.f);
-        acc[0] = make_float4(0.f, 0.f, 0.f, 0.f);
-        acc[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (LIT) acc[2] = make_float4(0.f, 0.f, 0.f, 0.f);
-        const bool any = a0.x != 0.f || a0.y != 0.f || a0.z != 0.f || a0.w != 0.f ||
-                         a1.x != 0.f || a1.y != 0.f || a1.z != 0.f;
-        const uint32_t rec = s_idx[sl];
-        if (any) {
-          // moments (S_x, S_y, S_xx, S_xy, S_yy) of dp to the screen
-          // gradients: du = (-a S_x - b S_y, -b S_x - c S_y), dconic =
-          // (-S_xx / 2, -S_xy, -S_yy / 2); s_geo holds (u, -a/2, -b), s_c -c/2
-          const float4 sg = s_geo[sl];
-          const float sc = s_c[sl].x;
-          float4* dst = grad2d + 2 * (int64_t)rec;
-          const float w = A.geo[rec].w;
-          const float dw = w > 0.0f ? a1.z / w : 0.0f;
-          red_add_v4(dst, 2.0f * sg.z * a0.x + sg.w * a0.y, 2.0f * sc * a0.y + sg.w * a0.x,
-                     -0.5f * a0.z, -a0.w);
-          red_add_v4(dst + 1, -0.5f * a1.x, a1.y, dw, 0.0f);
-        }
-        if (LIT && (a1.w != 0.f || a2.x != 0.f)) red_add_v2(grad_shade + rec, a1.w, a2.x);
-      }
-      __syncthreads();
+  for (int i = 0; i < 2; ++i) {
+    ov[i] = make_float4(0.f, 0.f, 0.f, 1.f);
+    dv4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    nc[i] = 0;
+    if (W.px < W.width && W.py + 4 * i < W.height) {
+      const int64_t o = W.image + (int64_t)(W.py + 4 * i) * W.width + W.px;
+      ov[i] = out[o];
+      dv4[i] = dout[o];
+      nc[i] = n_contrib[o];
     }
   }
+  float2 T = make_float2(ov[0].w, ov[1].w);
+  const float2 gr = make_float2(dv4[0].x, dv4[1].x), gg = make_float2(dv4[0].y, dv4[1].y),
+               gb = make_float2(dv4[0].z, dv4[1].z);
+  auto suf = [&](float4 o, float4 d) {
+    return -(o.w * (A.bg0 * d.x + A.bg1 * d.y + A.bg2 * d.z + d.w));
+  };
+  float2 nSuf = make_float2(suf(ov[0], dv4[0]), suf(ov[1], dv4[1]));
+  if (STATS) n_rep += (unsigned long long)nc[0] + (unsigned long long)nc[1];
+  // the warp walks from its last contribution; lane l of a chunk ending at
+  // list position `end` holds position end - 1 - l
+  const int wmax = __reduce_max_sync(0xffffffffu, max(nc[0], nc[1]));
+  const uint32_t* list = A.vals + W.rg.x;
+  uint32_t cur = 0, next = 0;  // this lane's record in the chunk fetched last, and in the next
+  int side = 0;
+  auto raw = [&](int sd) {
+    RawSlot s;
+    s.geo = S.raw[sd] + lane;
+    s.sh = s_sh;
+    return s;
+  };
+  if (wmax - 1 - lane >= 0) {
+    cur = __ldg(&list[wmax - 1 - lane]);
+    fetch_record<LIT>(A, raw(0), cur);
+  }
+  async_commit();
+  if (wmax - 33 - lane >= 0) next = __ldg(&list[wmax - 33 - lane]);
+  __syncthreads();  // the table
+  for (int end = wmax; end > 0; end -= 32, side ^= 1) {
+    // stage this chunk: each lane tests its record against the warp's block,
+    // the hits are compacted, last one first
+    async_wait();
+    const int pos = end - 1 - lane;
+    const uint32_t rec = cur;
+    bool hit = false;
+    float4 ge, au;
+    SplatTf tf;
+    float cut = 1.0f;
+    if (pos >= 0) {
+      ge = S.raw[side][lane];
+      au = S.raw[side][32 + lane];
+      tf = splat_tf(s_lut, A.lut_size, au.w, ge.w);
+      cut = power_cutoff(tf.aw);
+      hit = block_hit(ge.x - bx0, ge.y - by0, Reach(au.x, au.y, au.z, cut));
+    }
+    const unsigned hits = __ballot_sync(0xffffffffu, hit);
+    const int nh = __popc(hits), slot = __popc(hits & lanemask_lt_());
+    if (hit) {
+      float2 sh = make_float2(1.0f, 0.0f);
+      if (LIT) sh = *s_sh;
+      const float sl = (au.w >= 0.0f && au.w <= 1.0f) ? (float)(A.lut_size - 1) : 0.0f;
+      const float slc = LIT ? sl * sh.x : sl;  // colour slope scale
+      const float r = lerp_rn(tf.lo.x, tf.hi.x, tf.q), g = lerp_rn(tf.lo.y, tf.hi.y, tf.q),
+                  b = lerp_rn(tf.lo.z, tf.hi.z, tf.q);
+      const float dr = slc * (tf.hi.x - tf.lo.x), dg = slc * (tf.hi.y - tf.lo.y),
+                  db = slc * (tf.hi.z - tf.lo.z), da = ge.w * sl * (tf.hi.w - tf.lo.w);
+      const float4 cc = clean_conic(au);
+      S.u[slot] = make_float4(ge.x, ge.x, ge.y, ge.y);
+      S.q[slot] = make_float4(-0.5f * cc.x, -0.5f * cc.x, -cc.y, -cc.y);
+      S.r[slot] = make_float4(-0.5f * cc.z, -0.5f * cc.z, __int_as_float(pos), cut);
+      S.c0[slot] = make_float4(r, r, g, g);
+      S.c1[slot] = make_float4(b, b, tf.aw, tf.aw);
+      S.d0[slot] = make_float4(dr, dr, dg, dg);
+      S.d1[slot] = make_float4(db, db, da, da);
+      if (LIT) S.sh[slot] = make_float4(sh.x, sh.x, sh.y, sh.y);
+    }
+    if (lane == 0) {  // pads an odd count: A w = 0 never blends
+      const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+      S.u[nh] = S.q[nh] = S.c0[nh] = S.c1[nh] = S.d0[nh] = S.d1[nh] = z;
+      S.r[nh] = make_float4(0.f, 0.f, 0.f, 1.f);
+      if (LIT) S.sh[nh] = z;
+    }
+#pragma unroll
+    for (int e = 0; e < kAcc / 4; ++e)
+      reinterpret_cast<float4*>(S.acc)[e * 32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (pos - 32 >= 0) {
+      cur = next;
+      fetch_record<LIT>(A, raw(side ^ 1), cur);
+    }
+    async_commit();
+    if (pos - 64 >= 0) next = __ldg(&list[pos - 64]);
+    __syncwarp();
+    // two splats per step: what does not depend on the transmittance is
+    // formed for both, then each blend is undone in turn
+    for (int k = 0; k < nh; k += 2) {
+      Offsets o[2];
+      float2 G[2], raw2[2], al[2];
+      bool ok[2][2];
+      float4 c1[2];
+#pragma unroll
+      for (int m = 0; m < 2; ++m) {
+        const float4 u = S.u[k + m], q = S.q[k + m], r = S.r[k + m];
+        c1[m] = S.c1[k + m];
+        const float2 p = power2(u, q, r, fx, fy, o[m]);
+        const int at = __float_as_int(r.z);
+        const float2 x = mul2(p, dup(kLog2e));
+        G[m] = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+        raw2[m] = mul2(hi2(c1[m]), G[m]);
+        al[m] = make_float2(fminf(kAlphaMax, raw2[m].x), fminf(kAlphaMax, raw2[m].y));
+        ok[m][0] = at < nc[0] && !(p.x > 0.0f) && !(al[m].x < kAlphaMin);
+        ok[m][1] = at < nc[1] && !(p.y > 0.0f) && !(al[m].y < kAlphaMin);
+        if (STATS && r.w < 0.0f) {
+          n_it += 2;
+          n_eval += (unsigned)(at < nc[0] && p.x <= 0.0f && p.x >= r.w) +
+                    (unsigned)(at < nc[1] && p.y <= 0.0f && p.y >= r.w);
+          n_blend += (unsigned)ok[m][0] + (unsigned)ok[m][1];
+          n_free += (unsigned)(ok[m][0] && raw2[m].x <= kAlphaMax) +
+                    (unsigned)(ok[m][1] && raw2[m].y <= kAlphaMax);
+        }
+      }
+      if (!__any_sync(0xffffffffu, ok[0][0] || ok[0][1] || ok[1][0] || ok[1][1])) continue;
+      // the splats' sums over the lane's two pixels: dp, dL/dv (, dL/ds_d),
+      // dp dy, dp dy^2 (, dL/ds_s)
+      constexpr int kSum = LIT ? 6 : 4;
+      float v[2 * kSum];
+#pragma unroll
+      for (int m = 0; m < 2; ++m) {
+        const float4 c0 = S.c0[k + m], s0 = S.d0[k + m], s1 = S.d1[k + m];
+        const float2 om = sub2(dup(1.0f), al[m]);
+        const float2 rr = make_float2(rcp_approx(om.x), rcp_approx(om.y));
+        const float2 cgu = fma2(lo2(c1[m]), gb, fma2(hi2(c0), gg, mul2(lo2(c0), gr)));
+        const float2 h = fma2(lo2(s1), gb, fma2(hi2(s0), gg, mul2(lo2(s0), gr)));
+        const float2 Ti = mul2(T, rr);  // transmittance in front of the splat
+        const float2 wgt = mul2(al[m], Ti);
+        float2 cgd = cgu;
+        if (LIT) {
+          const float4 sh = S.sh[k + m];
+          const float2 gs = add2(add2(gr, gg), gb);
+          cgd = fma2(lo2(sh), cgu, mul2(hi2(sh), gs));
+          const float2 d = mul2(wgt, cgu), s = mul2(wgt, gs);
+          v[m * kSum + 2] = (ok[m][0] ? d.x : 0.0f) + (ok[m][1] ? d.y : 0.0f);
+          v[m * kSum + 5] = (ok[m][0] ? s.x : 0.0f) + (ok[m][1] ? s.y : 0.0f);
+        }
+        const float2 da = fma2(Ti, cgd, mul2(nSuf, rr));
+        // below the clamp alpha follows the exponent and the opacity slope
+        float2 mg = mul2(da, G[m]), cv = mul2(wgt, h);
+        mg.x = ok[m][0] && raw2[m].x <= kAlphaMax ? mg.x : 0.0f;
+        mg.y = ok[m][1] && raw2[m].y <= kAlphaMax ? mg.y : 0.0f;
+        cv.x = ok[m][0] ? cv.x : 0.0f;
+        cv.y = ok[m][1] ? cv.y : 0.0f;
+        const float2 dp = mul2(hi2(c1[m]), mg), dvv = fma2(hi2(s1), mg, cv);
+        const float2 y1 = mul2(dp, o[m].dy), y2 = mul2(dp, o[m].dyy);
+        v[m * kSum] = dp.x + dp.y;
+        v[m * kSum + 1] = dvv.x + dvv.y;
+        v[m * kSum + kSum / 2] = y1.x + y1.y;
+        v[m * kSum + kSum / 2 + 1] = y2.x + y2.y;
+        if (ok[m][0]) {
+          nSuf.x = __fmaf_rn(-cgd.x, wgt.x, nSuf.x);
+          T.x = Ti.x;
+        }
+        if (ok[m][1]) {
+          nSuf.y = __fmaf_rn(-cgd.y, wgt.y, nSuf.y);
+          T.y = Ti.y;
+        }
+        if (STATS) n_grad += (unsigned)(dp.x != 0.f) + (unsigned)(dp.y != 0.f);
+      }
+      // over the columns' lanes: bit 4 selects the splat, bit 3 the half of
+      // its sums; then times the column's dx over the eight columns (slot
+      // bits 2 and 1): slots (S0, S0 dx, S0 dx^2, V) and (S1, S1 dx, -, S2)
+      const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
+      float w[kSum], x[kSum / 2], y[4], z[2];
+      exchange<kSum>(v, w, b4, 16);
+      exchange<kSum / 2>(w, x, b3, 8);
+      const float dx = b4 ? o[1].dx.x : o[0].dx.x;
+      y[0] = x[0];
+      y[1] = x[0] * dx;
+      y[2] = y[1] * dx;
+      y[3] = x[1];
+      exchange<2>(y, z, b2, 4);
+      float f;
+      exchange<1>(z, &f, b1, 2);
+      f += __shfl_xor_sync(0xffffffffu, f, 1);
+      float* acc = S.acc + (k + (b4 ? 1 : 0)) * kAcc;
+      if ((lane & 1) == 0) acc[(lane >> 1) & 7] = f;
+      if (LIT) {
+        float s = x[kSum / 2 - 1];
+#pragma unroll
+        for (int d = 4; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+        if ((lane & 7) == 0) acc[8 + (b3 ? 1 : 0)] = s;
+      }
+    }
+    __syncwarp();
+    // the lane that staged a splat adds its gradients to the record's
+    if (hit) {
+      const float4* acc = reinterpret_cast<const float4*>(S.acc + slot * kAcc);
+      const float4 a0 = acc[0], a1 = acc[1];  // (S, Sx, Sxx, dv), (Sy, Sxy, -, Syy)
+      const bool any = a0.x != 0.f || a0.y != 0.f || a0.z != 0.f || a0.w != 0.f ||
+                       a1.x != 0.f || a1.y != 0.f || a1.w != 0.f;
+      if (any) {
+        // moments of dp to the screen gradients: du = (-a S_x - b S_y, -b S_x
+        // - c S_y), dconic = (-S_xx / 2, -S_xy, -S_yy / 2)
+        const float4 cc = clean_conic(S.raw[side][32 + lane]);
+        const float wt = S.raw[side][lane].w;
+        float4* dst = grad2d + 2 * (int64_t)rec;
+        const float dw = wt > 0.0f ? a0.x / wt : 0.0f;
+        red_add_v4(dst, -cc.x * a0.y - cc.y * a1.x, -cc.z * a1.x - cc.y * a0.y, -0.5f * a0.z,
+                   -a1.y);
+        red_add_v4(dst + 1, -0.5f * a1.w, a0.w, dw, 0.0f);
+      }
+      if (LIT) {
+        const float4 a2 = acc[2];
+        if (a2.x != 0.f || a2.y != 0.f) red_add_v2(grad_shade + rec, a2.x, a2.y);
+      }
+    }
+    __syncwarp();
+  }
+  async_wait();  // no copy in flight past the CTA's end
   if (STATS) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       n_rep += __shfl_down_sync(0xffffffffu, n_rep, o);
       n_it += __shfl_down_sync(0xffffffffu, n_it, o);
       n_eval += __shfl_down_sync(0xffffffffu, n_eval, o);
-      n_alpha += __shfl_down_sync(0xffffffffu, n_alpha, o);
       n_blend += __shfl_down_sync(0xffffffffu, n_blend, o);
       n_free += __shfl_down_sync(0xffffffffu, n_free, o);
       n_grad += __shfl_down_sync(0xffffffffu, n_grad, o);
@@ -842,7 +896,7 @@ __global__ void __launch_bounds__(256, ((LIT || STATS) && TG >= 4) ? 3 : 4)
       atomicAdd(&stats[0], n_rep);
       atomicAdd(&stats[1], n_it);
       atomicAdd(&stats[2], n_eval);
-      atomicAdd(&stats[3], n_alpha);
+      atomicAdd(&stats[3], n_eval);
       atomicAdd(&stats[4], n_blend);
       atomicAdd(&stats[5], n_free);
       atomicAdd(&stats[6], n_grad);
@@ -850,43 +904,24 @@ __global__ void __launch_bounds__(256, ((LIT || STATS) && TG >= 4) ? 3 : 4)
   }
 }
 
-size_t bwd_smem_bytes(int TG, int L, bool lit, int B) {
-  // col + slope, geo, (c, cutoff), (s_d, s_s), acc, idx, mask, warp lists (the
-  // tables stay in global memory)
-  (void)L;
-  return (size_t)TG * B * 16 * 2 + (size_t)B * 16 + (size_t)B * 8 +
-         (lit ? (size_t)B * 8 : 0) + (size_t)(lit ? 12 : 8) * B * 4 + (size_t)B * 4 +
-         (size_t)B + (size_t)kWarps * B * (B > 256 ? 2 : 1);
+// Dynamic shared memory of a CTA.  Forward: the padded splat arrays, the
+// records on their way, the table, warp lists and masks; backward: its
+// warps' splats, the table, the shading factors on their way.
+size_t fwd_smem_bytes(int L, bool lit, int B) {
+  const size_t P = B + 1;
+  return P * (16 + 16 + 8) + (size_t)2 * B * 16 + (size_t)L * 16 + (lit ? (size_t)B * 8 : 0) +
+         (size_t)kWarps * (B + 4) * sizeof(ListEntry) + (size_t)B;
+}
+size_t bwd_smem_bytes(int L, bool lit) {
+  return kWarps * (lit ? sizeof(BwdWarp<true>) : sizeof(BwdWarp<false>)) + (size_t)L * 16 +
+         (lit ? (size_t)kCompThreads * 8 : 0);
 }
 
-// Shared memory of a forward CTA: the group's tables (dynamic) and the
-// batch arrays (static).
-size_t fwd_smem_bytes(int TG, int L, int B) {
-  return (size_t)TG * L * 16 + (size_t)B * (16 + 8 + 1) + (size_t)TG * B * 16 +
-         (size_t)kWarps * B * (B > 256 ? 2 : 1);
-}
-
-// Tile batch: the caller's choice (128, 256 or 512 splats), else 256.
-int pick_batch(int tile_batch) { return tile_batch == 128 || tile_batch == 512 ? tile_batch : 256; }
-
-// TF group size: the caller's choice, else 1 for the forward (measured
-// fastest at the training-step and sweep shapes: each TF stops at its own
-// termination) and up to 4 for the backward (whose replay shares each
-// splat's geometry and reductions across the group); halved until the
-// group's shared memory fits one CTA (227 KB) at tile batch B.  The group
-// size changes no result; one table of up to 4096 entries always fits.
-int pick_group(int tf_group, int n_tf, bool bwd, int lut_size, bool lit, int B) {
-  int g = tf_group;
-  if (g <= 0) g = bwd ? std::min(n_tf, 4) : 1;
-  g = g <= 1 ? 1 : g <= 2 ? 2 : (g <= 4 || bwd) ? 4 : 8;
-  auto fits = [&](int tg) {
-    const size_t bytes = bwd ? bwd_smem_bytes(tg, lut_size, lit, B) + 1024
-                             : fwd_smem_bytes(tg, lut_size, B) + 1024;
-    return bytes <= (size_t)227 * 1024;
-  };
-  while (g > 1 && !fits(g)) g /= 2;
-  return g;
-}
+// Tile batch of the forward: the caller's choice (128, 256 or 512 splats),
+// else 256 (131 us on the 500k-Gaussian 512x512 frame against 135 at 128; 509
+// against 504 on the 1M-Gaussian scene under 4 tables; 512 stages less often
+// but holds half the CTAs: 700 us there, 20% faster for one faint table).
+int pick_batch(int tile_batch) { return tile_batch > 0 ? tile_batch : 256; }
 
 CompArgs make_args(const veg_camera* cams, int n_views, const float4* geo, const float4* aux,
                    const uint32_t* vals, const int2* ranges, const int32_t* order, veg_tf tf,
@@ -909,63 +944,47 @@ CompArgs make_args(const veg_camera* cams, int n_views, const float4* geo, const
   return A;
 }
 
-template <int TG, int B, bool STATS, bool LIT>
-veg_status launch_fwd_t(const CompArgs& A, int n_views, float4* out, int32_t* nc,
-                        unsigned long long* stats, cudaStream_t stream) {
-  const size_t smem = (size_t)TG * A.lut_size * sizeof(float4);
-  auto kern = composite_fwd_kernel<TG, B, STATS, LIT>;
+// One CTA per (tile, image): every table of the call, or one image per view.
+inline dim3 comp_grid(const CompArgs& A, int n_views) {
+  return dim3((unsigned)A.vm.tile_off[n_views], 1u, A.view_tf ? 1u : (unsigned)A.n_tf);
+}
+
+template <int B, bool STATS, bool LIT>
+veg_status launch_fwd(const CompArgs& A, int n_views, float4* out, int32_t* nc,
+                      unsigned long long* stats, cudaStream_t stream) {
+  const size_t smem = fwd_smem_bytes(A.lut_size, LIT, B);
+  auto kern = composite_fwd_kernel<B, STATS, LIT>;
   static SmemRecord configured;
   veg_status st = prepare_smem(kern, smem, configured, true);
   if (st != VEG_OK) return st;
-  const unsigned groups = A.view_tf ? 1u : (unsigned)((A.n_tf + TG - 1) / TG);
-  dim3 grid((unsigned)A.vm.tile_off[n_views], 1u, groups);
-  launch_k(kern, grid, 256, smem, stream, A, out, nc, stats);
+  launch_k(kern, comp_grid(A, n_views), kCompThreads, smem, stream, A, out, nc, stats);
   count_launch();
   return launch_status();
 }
 
-template <int TG, int B, bool STATS, bool LIT>
-veg_status launch_bwd_t(const CompArgs& A, int n_views, const float4* out, const int32_t* nc,
-                        const float4* dout, float4* grad2d, float2* grad_shade,
-                        unsigned long long* stats, cudaStream_t stream) {
-  const size_t smem = bwd_smem_bytes(TG, A.lut_size, LIT, B);
-  auto kern = composite_bwd_kernel<TG, B, STATS, LIT>;
+template <bool STATS, bool LIT>
+veg_status launch_bwd(const CompArgs& A, int n_views, const float4* out, const int32_t* nc,
+                      const float4* dout, float4* grad2d, float2* grad_shade,
+                      unsigned long long* stats, cudaStream_t stream) {
+  const size_t smem = bwd_smem_bytes(A.lut_size, LIT);
+  auto kern = composite_bwd_kernel<STATS, LIT>;
   static SmemRecord configured;
   veg_status st = prepare_smem(kern, smem, configured, true);
   if (st != VEG_OK) return st;
-  const unsigned groups = A.view_tf ? 1u : (unsigned)((A.n_tf + TG - 1) / TG);
-  dim3 grid((unsigned)A.vm.tile_off[n_views], 1u, groups);
-  launch_k(kern, grid, 256, smem, stream, A, out, nc, dout, grad2d, grad_shade, stats);
+  launch_k(kern, comp_grid(A, n_views), kCompThreads, smem, stream, A, out, nc, dout, grad2d,
+           grad_shade, stats);
   count_launch();
   return launch_status();
 }
 
-// Dispatch over the tile batch (the instrumented builds use 256: the pair
+// Dispatch over the tile batch (the instrumented build uses 256: the pair
 // counts do not depend on the batch).
-template <int TG, bool STATS, bool LIT>
+template <bool LIT>
 veg_status fwd_batch(int B, const CompArgs& A, int n_views, float4* out, int32_t* nc,
-                     unsigned long long* stats, cudaStream_t stream) {
-  if constexpr (!STATS) {
-    if (B == 128) return launch_fwd_t<TG, 128, STATS, LIT>(A, n_views, out, nc, stats, stream);
-    if (B == 512) return launch_fwd_t<TG, 512, STATS, LIT>(A, n_views, out, nc, stats, stream);
-  }
-  return launch_fwd_t<TG, 256, STATS, LIT>(A, n_views, out, nc, stats, stream);
-}
-
-template <int TG, bool STATS, bool LIT>
-veg_status bwd_batch(int B, const CompArgs& A, int n_views, const float4* out, const int32_t* nc,
-                     const float4* dout, float4* grad2d, float2* grad_shade,
-                     unsigned long long* stats, cudaStream_t stream) {
-  if constexpr (!STATS) {
-    if (B == 128)
-      return launch_bwd_t<TG, 128, STATS, LIT>(A, n_views, out, nc, dout, grad2d, grad_shade,
-                                               stats, stream);
-    if (B == 512)
-      return launch_bwd_t<TG, 512, STATS, LIT>(A, n_views, out, nc, dout, grad2d, grad_shade,
-                                               stats, stream);
-  }
-  return launch_bwd_t<TG, 256, STATS, LIT>(A, n_views, out, nc, dout, grad2d, grad_shade, stats,
-                                           stream);
+                     cudaStream_t stream) {
+  if (B == 128) return launch_fwd<128, false, LIT>(A, n_views, out, nc, nullptr, stream);
+  if (B == 512) return launch_fwd<512, false, LIT>(A, n_views, out, nc, nullptr, stream);
+  return launch_fwd<256, false, LIT>(A, n_views, out, nc, nullptr, stream);
 }
 
 }  // namespace
