@@ -109,7 +109,10 @@ struct WsHeader {
   unsigned int pad0;
   unsigned long long n_visible;    // records that touch a tile (last binning)
   unsigned int key_min, key_max;   // range of the depth sort's keys (last binning)
-  unsigned int pad[56];
+  unsigned long long n_cells;      // (record, cell) pairs of the cell binning
+  unsigned int cut_rec;            // record whose instances the capacity cuts (cell binning)
+  unsigned int cut_tiles;          // ... and how many of them stay
+  unsigned int pad[52];
 };
 static_assert(sizeof(WsHeader) == 256, "header must be 256 bytes");
 constexpr unsigned int FLAG_CAPACITY = 1u;
