@@ -1564,23 +1564,38 @@ __global__ void __launch_bounds__(kCellChunk)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int total = cstart[n_cells];
   const uint32_t cut_rec = P.hdr->cut_rec, cut_tiles = P.hdr->cut_tiles;
-  for (int k = (int)blockIdx.x; k < total; k += (int)gridDim.x) {
-    const int4 d = desc[k];
-    const int i = d.x + tid;
-    const bool in = i < d.y;
-    const uint32_t g = in ? __ldg(P.words + i) & P.rec_mask : 0u;
-    // the first output position of this chunk's instances of tile `tid`
-    uint32_t dst = 0;
-    if (tid < kCellTiles) {
+  const int step = (int)gridDim.x;
+  // the reads of the next chunk (its descriptor, then its pair and the output
+  // position of tile `tid`, then the pair's rectangle) are in flight while
+  // the current chunk is staged and written
+  auto chunk = [&](int k) { return k < total ? __ldg(desc + k) : make_int4(0, 0, 0, 0); };
+  auto pair_of = [&](int4 d) {
+    return d.x + tid < d.y ? __ldg(P.words + d.x + tid) & P.rec_mask : 0u;
+  };
+  auto rect_of = [&](int4 d, uint32_t g) {
+    return d.x + tid < d.y ? __ldg(P.rect + g) : make_short4(0, 0, 0, 0);
+  };
+  auto start_of = [&](int4 d, int k) {
+    uint32_t at = 0;
+    if (tid < kCellTiles && k < total) {
       const int tx = (d.z & 0xffff) + (tid & 7), ty = (d.z >> 16) + (tid >> 3);
       const int tile = vm.tile_off[d.w] + ty * vm.tiles_x[d.w] + tx;
       if (tx < vm.tiles_x[d.w] && tile < vm.tile_off[d.w + 1])
-        dst = (uint32_t)ranges[tile].x + table[(int64_t)k * kCellTiles + tid];
+        at = (uint32_t)__ldg(&ranges[tile].x) + __ldg(&table[(int64_t)k * kCellTiles + tid]);
     }
-    const unsigned long long m =
-        in ? cell_tiles_of(__ldg(P.rect + g), d.z, g, cut_rec, cut_tiles) : 0ull;
+    return at;
+  };
+  int k = (int)blockIdx.x;
+  int4 d = chunk(k), d1 = chunk(k + step);
+  uint32_t g = pair_of(d), dst = start_of(d, k);
+  short4 rc = rect_of(d, g);
+  for (; k < total; k += step) {
+    const unsigned long long m = cell_tiles_of(rc, d.z, g, cut_rec, cut_tiles);
     uint32_t lo = warp_transpose((uint32_t)m), hi = warp_transpose((uint32_t)(m >> 32));
     s_rec[tid] = g;
+    const uint32_t dst0 = dst;
+    g = pair_of(d1);
+    dst = start_of(d1, k + step);
     s_cnt[warp][lane] = __popc(lo);
     s_cnt[warp][lane + 32] = __popc(hi);
     __syncthreads();
@@ -1611,7 +1626,7 @@ __global__ void __launch_bounds__(kCellChunk)
       }
     }
     __syncthreads();
-    if (tid < kCellTiles) s_base[tid] = dst - s_base[tid];
+    if (tid < kCellTiles) s_base[tid] = dst0 - s_base[tid];
     uint32_t at = s_cnt[warp][lane];
     uint32_t code = ((uint32_t)lane << 8) | (uint32_t)(warp << 5);
     while (lo) {
@@ -1624,6 +1639,9 @@ __global__ void __launch_bounds__(kCellChunk)
       s_stage[at++] = (uint16_t)(code | (uint32_t)(__ffs((int)hi) - 1));
       hi &= hi - 1;
     }
+    rc = rect_of(d1, g);
+    d = d1;
+    d1 = chunk(k + 2 * step);
     __syncthreads();
     const uint32_t n = s_total;
     for (uint32_t p = (uint32_t)tid; p < n; p += kCellChunk) {
