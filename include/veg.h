@@ -260,6 +260,16 @@ veg_status veg_radix_lookback_check(void* workspace, size_t workspace_bytes, int
  */
 veg_status veg_sync_status(const void* workspace, cudaStream_t stream, int64_t* n_instances);
 
+/* The same without waiting: veg_status_fetch enqueues a copy of the status
+ * header into host_status (host, 256 bytes, page-locked for the copy to be
+ * asynchronous); once the stream has passed the copy, veg_status_read turns
+ * it into veg_sync_status's result.  Work enqueued in between (a compositing
+ * pass, say) does not delay the answer.  The lists of a binning that timed
+ * out are empty, those of one that overflowed hold the instances that fit.
+ */
+veg_status veg_status_fetch(const void* workspace, void* host_status, cudaStream_t stream);
+veg_status veg_status_read(const void* host_status, int64_t* n_instances);
+
 /*
  * veg_composite_fwd -- Eq. 1 per pixel, for n_tf transfer functions at once.
  *

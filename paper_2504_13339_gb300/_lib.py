@@ -98,6 +98,8 @@ _SIGS = {
     "veg_bin_sort_static": (ctypes.c_int, [_CAMS, _I32, _I64, _P, _P, _P, _I64, _P, _P, _P, _P,
                                            _P]),
     "veg_sync_status": (ctypes.c_int, [_P, _P, ctypes.POINTER(_I64)]),
+    "veg_status_fetch": (ctypes.c_int, [_P, _P, _P]),
+    "veg_status_read": (ctypes.c_int, [_P, ctypes.POINTER(_I64)]),
     "veg_composite_fwd": (ctypes.c_int, [_CAMS, _I32, _I64, _P, _P, _P, _P, _P, _P, veg_tf, _P,
                                          _I32, _I32, _P, _P, _P, _P]),
     "veg_composite_bwd_workspace_size": (ctypes.c_int, [_I64, _I32, ctypes.POINTER(_SZ)]),
@@ -274,6 +276,21 @@ def veg_sync_status(workspace, stream=None):
     st = load().veg_sync_status(_ptr(workspace), _stream(stream), ctypes.byref(n))
     if st not in (VEG_OK, VEG_ERR_CAPACITY, VEG_ERR_TIMEOUT):
         raise VegError("veg_sync_status", st)
+    return st, n.value
+
+
+def veg_status_fetch(workspace, host_status, stream=None):
+    """host_status: 256-byte pinned uint8 tensor."""
+    _check("veg_status_fetch",
+           load().veg_status_fetch(_ptr(workspace), host_status.data_ptr(), _stream(stream)))
+
+
+def veg_status_read(host_status):
+    """(status, n_instances) of a fetched header, like veg_sync_status."""
+    n = _I64()
+    st = load().veg_status_read(host_status.data_ptr(), ctypes.byref(n))
+    if st not in (VEG_OK, VEG_ERR_CAPACITY, VEG_ERR_TIMEOUT):
+        raise VegError("veg_status_read", st)
     return st, n.value
 
 

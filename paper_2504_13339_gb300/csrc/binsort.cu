@@ -23,6 +23,7 @@
 // workspace header, so no host round trip is needed and no block works past
 // them.
 #include <algorithm>
+#include <cstring>
 
 #include "veg_internal.cuh"
 
@@ -822,8 +823,9 @@ __global__ void zero_ranges_kernel(int2* __restrict__ ranges, int64_t count,
 // marks "no neighbour".
 __global__ void ranges_kernel(const uint32_t* __restrict__ keys, Count cnt,
                               int2* __restrict__ ranges, int key_shift,
-                              uint32_t* __restrict__ vals) {
+                              uint32_t* __restrict__ vals, const WsHeader* hdr) {
   pdl_enter();
+  if (hdr->flags & FLAG_TIMEOUT) return;  // void lists: every range stays empty
   const int64_t n = cnt.get();
   // a bounded grid strides over the items: their count is far below the
   // capacity that the host knows
@@ -2026,7 +2028,7 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
     uint32_t* table = kbuf[(passes & 1) ^ 1];
     uint32_t* totals = table + kCellTiles * max_chunks;
     launch_k(ranges_kernel, pass_grid((int)grid_for(capacity, 1024), 8), 256, 0, stream, ckeys, cc, cranges,
-             rec_bits, (uint32_t*)nullptr);
+             rec_bits, (uint32_t*)nullptr, (const WsHeader*)L.hdr);
     launch_k(cell_map_kernel, 1, kCellScanThreads, 0, stream, (const int2*)cranges, (int)n_cells,
              cm, (int)max_chunks, cstart, desc);
     CellPairs P;
@@ -2073,7 +2075,7 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
   // 4. per-tile ranges (and the records, from packed words) and optional
   //    64-bit keys
   launch_k(ranges_kernel, pass_grid((int)grid_for(capacity, 1024), 8), 256, 0, stream, fkeys, ci, ranges, rec_bits,
-           packed ? vals : (uint32_t*)nullptr);
+           packed ? vals : (uint32_t*)nullptr, (const WsHeader*)L.hdr);
   count_launch();
   if (keys) {
     launch_k(keys64_kernel, grid_for(capacity, 256), 256, 0, stream, fkeys, vals, ci, geo, vm,
@@ -2192,6 +2194,16 @@ extern "C" veg_status veg_bin_sort(const veg_camera* cams, int32_t n_views, int6
                         keys, vals, reinterpret_cast<int2*>(tile_ranges), stream);
 }
 
+namespace {
+
+veg_status status_of(const veg::WsHeader& h, int64_t* n_instances) {
+  if (n_instances) *n_instances = (int64_t)h.n_instances;
+  if (h.flags & veg::FLAG_TIMEOUT) return VEG_ERR_TIMEOUT;
+  return (h.flags & veg::FLAG_CAPACITY) ? VEG_ERR_CAPACITY : VEG_OK;
+}
+
+}  // namespace
+
 extern "C" veg_status veg_sync_status(const void* workspace, cudaStream_t stream,
                                       int64_t* n_instances) {
   if (!workspace) return VEG_ERR_INVALID_ARGUMENT;
@@ -2199,9 +2211,23 @@ extern "C" veg_status veg_sync_status(const void* workspace, cudaStream_t stream
   if (cudaMemcpyAsync(&h, workspace, sizeof(h), cudaMemcpyDeviceToHost, stream) != cudaSuccess)
     return VEG_ERR_CUDA;
   if (cudaStreamSynchronize(stream) != cudaSuccess) return VEG_ERR_CUDA;
-  if (n_instances) *n_instances = (int64_t)h.n_instances;
-  if (h.flags & veg::FLAG_TIMEOUT) return VEG_ERR_TIMEOUT;
-  return (h.flags & veg::FLAG_CAPACITY) ? VEG_ERR_CAPACITY : VEG_OK;
+  return status_of(h, n_instances);
+}
+
+extern "C" veg_status veg_status_fetch(const void* workspace, void* host_status,
+                                       cudaStream_t stream) {
+  if (!workspace || !host_status) return VEG_ERR_INVALID_ARGUMENT;
+  return cudaMemcpyAsync(host_status, workspace, sizeof(veg::WsHeader), cudaMemcpyDeviceToHost,
+                         stream) == cudaSuccess
+             ? VEG_OK
+             : VEG_ERR_CUDA;
+}
+
+extern "C" veg_status veg_status_read(const void* host_status, int64_t* n_instances) {
+  if (!host_status) return VEG_ERR_INVALID_ARGUMENT;
+  veg::WsHeader h;
+  std::memcpy(&h, host_status, sizeof(h));
+  return status_of(h, n_instances);
 }
 
 // ---------------------------------------------------------------------------

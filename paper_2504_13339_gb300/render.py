@@ -71,6 +71,7 @@ class SplatPipeline:
                                    device=dev)
         self.keys = None
         self._lit = None  # (mean_v, normal_beta, k_ads, light_dirs) when shaded
+        self._status_host = self._status_ready = None  # of `render`
         self.generation = 0  # composites so far: a backward must follow its own forward
         self.set_capacity(capacity if capacity is not None else max(1 << 16, 8 * nrec))
 
@@ -244,15 +245,33 @@ class SplatPipeline:
     # -- whole passes --------------------------------------------------------
     def render(self, mean_v, logscale_w, quat, luts, bg=(0.0, 0.0, 0.0), cull=True,
                stream=None):
-        """Project + bin + composite; grows the instance capacity (one host
-        sync) when the binning overflowed."""
+        """Project + bin + composite; waits for the binning's status, and on
+        overflow grows the instance capacity and bins and composites again.
+        The compositing is enqueued before the wait (its lists are valid
+        whatever the status: those that fit, or empty ones), so the GPU does
+        not idle over the host's round trip: 298 -> 269 us for a 512x512
+        frame of 500k Gaussians, 90 -> 74 for a 4096-Gaussian thumbnail."""
+        if self._status_host is None:
+            self._status_host = torch.empty(256, dtype=torch.uint8, pin_memory=True)
+            self._status_ready = torch.cuda.Event()
         self.project(mean_v, logscale_w, quat, luts if cull else None, stream)
         self.bin_sort(stream=stream)
-        st, m = self.status(stream)
+        on = torch.cuda.current_stream() if stream is None else stream
+        if not isinstance(on, torch.cuda.Stream):
+            on = torch.cuda.ExternalStream(on.cuda_stream)
+        _lib.veg_status_fetch(self.ws, self._status_host, on)
+        self._status_ready.record(on)
+        out = self.composite(luts, bg, stream=stream)
+        self._status_ready.synchronize()
+        st, m = _lib.veg_status_read(self._status_host)
+        if st == _lib.VEG_ERR_TIMEOUT:
+            raise _lib.VegError("veg_bin_sort", st)
         if st != _lib.VEG_OK:
+            on.synchronize()  # the compositing reads the buffers that are replaced
             self.set_capacity(int(m * 1.25) + 1024)
             self.bin_sort(stream=stream)
-        return self.composite(luts, bg, stream=stream)
+            return self.composite(luts, bg, stream=stream)
+        return out
 
     def train_step(self, mean_v, logscale_w, quat, luts, target, grads, bg=(0.0, 0.0, 0.0),
                    lighting=None, stream=None, project_grads=True):
