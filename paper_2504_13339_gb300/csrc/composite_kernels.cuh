@@ -223,9 +223,10 @@ __device__ __forceinline__ int build_warp_list(const unsigned char* s_mask, List
   return total;
 }
 
-// The lane's first pixel; its second is four rows below.
-__device__ __forceinline__ void pixel_of(int tile, int tiles_x, int& px, int& py) {
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+// The lane's first pixel in 8x8 block w of a tile; its second is four rows
+// below.
+__device__ __forceinline__ void pixel_of(int tile, int tiles_x, int w, int& px, int& py) {
+  const int l = threadIdx.x & 31;
   px = (tile % tiles_x) * VEG_TILE + (w & 1) * 8 + (l & 7);
   py = (tile / tiles_x) * VEG_TILE + (w >> 1) * 8 + (l >> 3);
 }
@@ -244,7 +245,7 @@ struct CompArgs {
   float bg0, bg1, bg2;
 };
 
-// The work item of a CTA: its tile, output image and table.
+// A work item: its tile, output image and table.
 struct WorkItem {
   int px, py;           // the lane's first pixel
   int width, height;
@@ -252,9 +253,9 @@ struct WorkItem {
   long long image;      // first pixel of the output image
   int2 rg;              // the tile's list
 };
-__device__ __forceinline__ WorkItem work_item(const CompArgs& A, float4* s_lut) {
+__device__ __forceinline__ WorkItem work_item(const CompArgs& A, float4* s_lut, int item,
+                                              int block) {
   WorkItem w;
-  const int item = (int)blockIdx.x;
   const int wi = A.order ? A.order[item] : item;  // global tile id
   const int view = view_of_tile(A.vm, wi), tile = wi - A.vm.tile_off[view];
   const int tiles_x = A.vm.tiles_x[view], t = (int)blockIdx.z;
@@ -262,14 +263,14 @@ __device__ __forceinline__ WorkItem work_item(const CompArgs& A, float4* s_lut) 
   w.height = A.vm.height[view];
   w.rg = A.ranges[wi];
   w.image = A.vm.pix_off[view] + (long long)t * w.width * w.height;
-  pixel_of(tile, tiles_x, w.px, w.py);
+  pixel_of(tile, tiles_x, block, w.px, w.py);
   w.tx0 = (float)((tile % tiles_x) * VEG_TILE);
   w.ty0 = (float)((tile / tiles_x) * VEG_TILE);
   // the table into shared memory; an index outside [0, n_tf) reads as fully
   // transparent
   const int ti = A.view_tf ? A.view_tf[view] : t;
   const bool ok = ti >= 0 && ti < A.n_tf;
-  for (int e = threadIdx.x; e < A.lut_size; e += kCompThreads)
+  for (int e = threadIdx.x; e < A.lut_size; e += blockDim.x)
     s_lut[e] = ok ? __ldg(&A.lut[(int64_t)ti * A.lut_size + e]) : make_float4(0.f, 0.f, 0.f, 0.f);
   return w;
 }
@@ -393,6 +394,20 @@ __device__ __forceinline__ float2 at16(const float2* a, unsigned off) {
 // forward
 // ---------------------------------------------------------------------------
 
+// Exponents and alphas of a splat at a lane's two pixels (x, y) and (x, y'):
+// g = (u_x, u_y, -a/2, -b), h = (-c/2, A w).
+__device__ __forceinline__ float2 pair_alpha(float4 g, float2 h, float x, float2 y, float2& p) {
+  const float dx = sub(g.x, x);
+  const float2 dy = make_float2(sub(g.y, y.x), sub(g.y, y.y));
+  const float dxx = mul(dx, dx);
+  const float2 dyy = mul2(dy, dy);
+  p = make_float2(__fmaf_rn(g.z, dxx, __fmaf_rn(h.x, dyy.x, mul(g.w, mul(dx, dy.x)))),
+                  __fmaf_rn(g.z, dxx, __fmaf_rn(h.x, dyy.y, mul(g.w, mul(dx, dy.y)))));
+  const float2 e = mul2(p, dup(kLog2e));
+  return make_float2(fminf(kAlphaMax, mul(h.y, ex2_approx(e.x))),
+                     fminf(kAlphaMax, mul(h.y, ex2_approx(e.y))));
+}
+
 // stats (instrumented build): visited pairs (every pair reached before the
 // pixel's termination, the method's own count), iterated pairs (walked by
 // the warp lists), pairs above the cutoff, alpha evaluations, blended pairs.
@@ -419,7 +434,7 @@ __global__ void __launch_bounds__(kCompThreads, 7)
   const int warp = threadIdx.x >> 5;
   ListEntry* my_list = s_list + warp * (B + 4);
   unsigned long long n_vis = 0, n_it = 0, n_eval = 0, n_blend = 0;
-  const WorkItem W = work_item(A, s_lut);
+  const WorkItem W = work_item(A, s_lut, (int)blockIdx.x, (int)(threadIdx.x >> 5));
   if (threadIdx.x == 0) {  // the padding slot: A w = 0 never blends
     s_geo[B] = s_col[B] = make_float4(0.f, 0.f, 0.f, 0.f);
     s_ca[B] = make_float2(0.f, 0.f);
@@ -479,16 +494,8 @@ __global__ void __launch_bounds__(kCompThreads, 7)
         col[m] = at16(s_col, off[m]);
         const float4 g = at16(s_geo, off[m]);
         const float2 h = at16(s_ca, off[m]);
-        const float dx = sub(g.x, fx.x);
-        const float2 dy = make_float2(sub(g.y, fy.x), sub(g.y, fy.y));
-        const float dxx = mul(dx, dx);
-        const float2 dyy = mul2(dy, dy);
-        const float2 p = make_float2(
-            __fmaf_rn(g.z, dxx, __fmaf_rn(h.x, dyy.x, mul(g.w, mul(dx, dy.x)))),
-            __fmaf_rn(g.z, dxx, __fmaf_rn(h.x, dyy.y, mul(g.w, mul(dx, dy.y)))));
-        const float2 x = mul2(p, dup(kLog2e));
-        al[m] = make_float2(fminf(kAlphaMax, mul(h.y, ex2_approx(x.x))),
-                            fminf(kAlphaMax, mul(h.y, ex2_approx(x.y))));
+        float2 p;
+        al[m] = pair_alpha(g, h, fx.x, fy, p);
         ok[m][0] = !(p.x > 0.0f) && !(al[m].x < kAlphaMin);
         ok[m][1] = !(p.y > 0.0f) && !(al[m].y < kAlphaMin);
         if (STATS && k + m < nw) {
@@ -557,6 +564,217 @@ __global__ void __launch_bounds__(kCompThreads, 7)
       atomicAdd(&stats[4], n_blend);
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// forward of few work items
+// ---------------------------------------------------------------------------
+
+// With a few CTAs per SM in all, a launch lasts as long as its longest list:
+// a warp blends it splat after splat, and most of that chain (a list entry,
+// the shared reads, the exponent) does not depend on the transmittance.  Here
+// a CTA holds one 8x8 block; four producer warps take every fourth chunk of
+// 32 list entries, stage it and form the alphas of its splats at the 64
+// pixels; two consumer warps, a pixel per lane, only blend.  The alphas pass
+// through shared memory, a slot per producer, full and empty barriers per
+// slot.  Decisions and images are those of composite_fwd_kernel bit for bit
+// (the alphas come from the same operations, a pair that does not blend
+// passes as 0).  It issues more instructions per pair, so the large launches
+// stay with the other kernel (48.6M warp instructions against 26.5M on the
+// 512x512 frame of 500k Gaussians, most of the difference the staging, which
+// each of a tile's blocks does by itself; there it takes 100 us against 148,
+// the SMs' busy share rising from 45% to 70%).
+//
+// Ending early: a consumer warp whose pixels have all left notes the chunk at
+// which they did.  A chunk's producer ends the list when both did by the
+// chunk that was in its slot before, which both have handed back: so the
+// first chunk to end is kProducers after the later of the two notes, whatever
+// the warps' timing, the next kProducers - 1 end too, and the consumers take
+// all their marks before they leave.  Every barrier is met by all that take
+// part in it.
+constexpr int kProducers = 4;
+constexpr int kDeepThreads = 32 * (2 + kProducers);
+
+template <int ID0>
+__device__ __forceinline__ void slot_sync(int slot) {
+  __syncwarp();
+  asm volatile("bar.sync %0, 96;" ::"r"(ID0 + slot) : "memory");
+}
+template <int ID0>
+__device__ __forceinline__ void slot_arrive(int slot) {
+  __threadfence_block();
+  __syncwarp();
+  asm volatile("bar.arrive %0, 96;" ::"r"(ID0 + slot) : "memory");
+}
+constexpr int kFull = 1, kEmpty = 1 + kProducers;  // named barriers; 0 is __syncthreads
+
+template <bool LIT>
+struct DeepSmem {
+  struct Producer {
+    float4 raw[2][2 * 32];        // records, alternate chunks
+    float2 raw_sh[LIT ? 64 : 1];  // their shading factors
+    float4 geo[32];               // the chunk's splats that reach the block
+    float2 ca[32];
+  } prod[kProducers];
+  float alpha[kProducers][32 * 64];  // [splat][pixel], 0: does not blend
+  float4 col[kProducers][32];
+  int pos[kProducers][32];           // list position of each splat
+  volatile int cnt[kProducers];      // splats in the slot, -1: the end
+  volatile int gone[2];              // chunk at which a consumer's last pixel left
+};
+
+template <bool LIT>
+__global__ void __launch_bounds__(kDeepThreads, 4)
+    composite_fwd_deep_kernel(CompArgs A, float4* __restrict__ out,
+                              int32_t* __restrict__ n_contrib) {
+  pdl_enter();
+  extern __shared__ float4 smem[];
+  DeepSmem<LIT>& S = *reinterpret_cast<DeepSmem<LIT>*>(smem);
+  float4* s_lut = reinterpret_cast<float4*>(&S + 1);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int block = (int)blockIdx.x & 3;
+  const WorkItem W = work_item(A, s_lut, (int)blockIdx.x >> 2, block);
+  const int n = W.rg.y - W.rg.x;
+  const int chunks = (n + 31) / 32;
+
+  if (warp < 2) {
+    const int py = W.py + 4 * warp;
+    const bool inside = W.px < W.width && py < W.height;
+    float T = inside ? 1.0f : -1.0f, Cr = 0.0f, Cg = 0.0f, Cb = 0.0f;
+    int last = 0;
+    bool gone = !__any_sync(0xffffffffu, inside);
+    if (lane == 0) S.gone[warp] = gone ? 0 : 0x7fffffff;
+    __syncthreads();
+    for (int c = 0; c < chunks; ++c) {
+      const int slot = c % kProducers;
+      slot_sync<kFull>(slot);
+      const int cnt = S.cnt[slot];
+      if (cnt < 0) {
+        for (int k = c + 1; k < c + kProducers && k < chunks; ++k) slot_sync<kFull>(k % kProducers);
+        break;
+      }
+      if (!gone) {
+        const float* al = S.alpha[slot] + warp * 32 + lane;
+        int lb = -1;
+        // eight splats per step: their reads overlap, then they blend in
+        // order (the products of a whole step as one chain, with the stop
+        // tested once, measured the same: the producers are the bound)
+        for (int j = 0; j < cnt; j += 8) {
+          float a[8];
+          float4 col[8];
+#pragma unroll
+          for (int m = 0; m < 8; ++m) {
+            a[m] = al[(j + m) * 64];
+            col[m] = S.col[slot][j + m];
+          }
+#pragma unroll
+          for (int m = 0; m < 8; ++m) {
+            const float test = mul(T, sub(1.0f, a[m])), wgt = mul(a[m], T);
+            const bool ok = a[m] > 0.0f, stop = test < kTMin;
+            if (ok && stop) T = -fabsf(T);
+            if (ok && !stop) {
+              Cr = __fmaf_rn(col[m].x, wgt, Cr);
+              Cg = __fmaf_rn(col[m].y, wgt, Cg);
+              Cb = __fmaf_rn(col[m].z, wgt, Cb);
+              T = test;
+              lb = j + m;
+            }
+          }
+        }
+        if (lb >= 0) last = S.pos[slot][lb] + 1;
+        gone = !__any_sync(0xffffffffu, T > 0.0f);
+        if (gone && lane == 0) S.gone[warp] = c;
+      }
+      if (c + kProducers < chunks) slot_arrive<kEmpty>(slot);
+    }
+    if (inside) {
+      const int64_t o = W.image + (int64_t)py * W.width + W.px;
+      const float Tf = fabsf(T);
+      out[o] = make_float4(add(Cr, mul(Tf, A.bg0)), add(Cg, mul(Tf, A.bg1)),
+                           add(Cb, mul(Tf, A.bg2)), Tf);
+      n_contrib[o] = last;
+    }
+    return;
+  }
+
+  const int me = warp - 2;
+  auto& P = S.prod[me];
+  const float bx0 = W.tx0 + (float)((block & 1) * 8), by0 = W.ty0 + (float)((block >> 1) * 8);
+  const float fx = (float)W.px;
+  const float2 fy = make_float2((float)W.py, (float)(W.py + 4));
+  const uint32_t* list = A.vals + W.rg.x;
+  constexpr int kStride = 32 * kProducers;
+  auto raw = [&](int side) {
+    RawSlot r;
+    r.geo = P.raw[side] + lane;
+    r.sh = P.raw_sh + (LIT ? side * 32 + lane : 0);
+    return r;
+  };
+  int at = me * 32 + lane;  // this lane's list position
+  uint32_t next = 0;
+  if (at < n) fetch_record<LIT>(A, raw(0), __ldg(&list[at]));
+  async_commit();
+  if (at + kStride < n) next = __ldg(&list[at + kStride]);
+  __syncthreads();  // the table, the consumers' marks
+  int side = 0;
+  for (int c = me; c < chunks; c += kProducers, at += kStride, side ^= 1) {
+    async_wait();
+    bool hit = false;
+    float4 ge, au;
+    SplatTf tf;
+    float cut = 1.0f;
+    if (at < n) {
+      ge = P.raw[side][lane];
+      au = P.raw[side][32 + lane];
+      tf = splat_tf(s_lut, A.lut_size, au.w, ge.w);
+      cut = power_cutoff(tf.aw);
+      hit = block_hit(ge.x - bx0, ge.y - by0, Reach(au.x, au.y, au.z, cut));
+    }
+    const unsigned hits = __ballot_sync(0xffffffffu, hit);
+    const int nh = __popc(hits), place = __popc(hits & lanemask_lt_());
+    float4 col = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (hit) {
+      col = make_float4(lerp_rn(tf.lo.x, tf.hi.x, tf.q), lerp_rn(tf.lo.y, tf.hi.y, tf.q),
+                        lerp_rn(tf.lo.z, tf.hi.z, tf.q), 0.0f);
+      if (LIT) {
+        const float2 sh = P.raw_sh[side * 32 + lane];
+        col.x = __fmaf_rn(sh.x, col.x, sh.y);
+        col.y = __fmaf_rn(sh.x, col.y, sh.y);
+        col.z = __fmaf_rn(sh.x, col.z, sh.y);
+      }
+      const float4 cc = clean_conic(au);
+      P.geo[place] = make_float4(ge.x, ge.y, -0.5f * cc.x, -cc.y);
+      P.ca[place] = make_float2(-0.5f * cc.z, tf.aw);
+    }
+    if (at + kStride < n) fetch_record<LIT>(A, raw(side ^ 1), next);
+    async_commit();
+    if (at + 2 * kStride < n) next = __ldg(&list[at + 2 * kStride]);
+    if (c >= kProducers) {
+      slot_sync<kEmpty>(me);
+      if (max(S.gone[0], S.gone[1]) <= c - kProducers) {
+        if (lane == 0) S.cnt[me] = -1;
+        slot_arrive<kFull>(me);
+        break;
+      }
+    }
+    if (hit) {
+      S.col[me][place] = col;
+      S.pos[me][place] = at;
+    }
+    if (lane == 0) S.cnt[me] = nh;
+    __syncwarp();
+    float* al = S.alpha[me] + lane;
+#pragma unroll 4
+    for (int j = 0; j < nh; ++j) {
+      float2 p;
+      const float2 a = pair_alpha(P.geo[j], P.ca[j], fx, fy, p);
+      al[j * 64] = !(p.x > 0.0f) && !(a.x < kAlphaMin) ? a.x : 0.0f;
+      al[j * 64 + 32] = !(p.y > 0.0f) && !(a.y < kAlphaMin) ? a.y : 0.0f;
+    }
+    for (int j = nh; j < ((nh + 7) & ~7); ++j) al[j * 64] = al[j * 64 + 32] = 0.0f;
+    slot_arrive<kFull>(me);
+  }
+  async_wait();  // no copy in flight past the CTA's end
 }
 
 // ---------------------------------------------------------------------------
@@ -656,7 +874,7 @@ __global__ void __launch_bounds__(kCompThreads, 4)
   Warp& S = reinterpret_cast<Warp*>(smem)[warp];
   float4* s_lut = reinterpret_cast<float4*>(reinterpret_cast<Warp*>(smem) + kWarps);
   float2* s_sh = reinterpret_cast<float2*>(s_lut + A.lut_size) + threadIdx.x;
-  const WorkItem W = work_item(A, s_lut);
+  const WorkItem W = work_item(A, s_lut, (int)blockIdx.x, (int)(threadIdx.x >> 5));
   const float bx0 = W.tx0 + (float)((warp & 1) * 8), by0 = W.ty0 + (float)((warp >> 1) * 8);
   const float2 fx = dup((float)W.px), fy = make_float2((float)W.py, (float)(W.py + 4));
 
@@ -977,11 +1195,37 @@ veg_status launch_bwd(const CompArgs& A, int n_views, const float4* out, const i
   return launch_status();
 }
 
+// The launches that take composite_fwd_deep_kernel: fewer work items than
+// kDeepItems.  Forward with it against one warp per block, by (tile, table)
+// items: 64 items 52 against 107 us (20k Gaussians), 1024 items 100 and 148,
+// 1105 items (five views) 144 and 232, 2500 items 128 and 144; 3072 items 182
+// and 152 (100k), 544 and 559 (1M), 3690 items 226 and 196.
+constexpr int64_t kDeepItems = 2048;
+
+template <bool LIT>
+veg_status launch_fwd_deep(const CompArgs& A, int n_views, float4* out, int32_t* nc,
+                           cudaStream_t stream) {
+  const size_t smem = sizeof(DeepSmem<LIT>) + (size_t)A.lut_size * 16;
+  auto kern = composite_fwd_deep_kernel<LIT>;
+  static SmemRecord configured;
+  veg_status st = prepare_smem(kern, smem, configured, true);
+  if (st != VEG_OK) return st;
+  dim3 grid = comp_grid(A, n_views);
+  grid.x *= 4;
+  launch_k(kern, grid, kDeepThreads, smem, stream, A, out, nc);
+  count_launch();
+  return launch_status();
+}
+
 // Dispatch over the tile batch (the instrumented build uses 256: the pair
 // counts do not depend on the batch).
 template <bool LIT>
 veg_status fwd_batch(int B, const CompArgs& A, int n_views, float4* out, int32_t* nc,
                      cudaStream_t stream) {
+  const dim3 items = comp_grid(A, n_views);
+  if ((int64_t)items.x * items.z < kDeepItems &&
+      sizeof(DeepSmem<LIT>) + (size_t)A.lut_size * 16 <= 100 * 1024)
+    return launch_fwd_deep<LIT>(A, n_views, out, nc, stream);
   if (B == 128) return launch_fwd<128, false, LIT>(A, n_views, out, nc, nullptr, stream);
   if (B == 512) return launch_fwd<512, false, LIT>(A, n_views, out, nc, nullptr, stream);
   return launch_fwd<256, false, LIT>(A, n_views, out, nc, nullptr, stream);
