@@ -316,14 +316,11 @@ __global__ void __launch_bounds__(256, 3)
       if (on == 0u) continue;
       float sd = 1.0f, ss = 0.0f;
       if (A.shade) {
-        // normal = -gradient / |gradient|; scaled first by the power of two
-        // that brings the largest component to [1, 4), exactly, so that
-        // tiny gradients cannot underflow
+        // normal = -gradient / |gradient|; scaled by the largest component
+        // first so that tiny gradients cannot underflow
         sd = A.ka;
         if (m > 0.0f) {
-          const int e = __float_as_int(m) & 0x7f800000;
-          const float by = __int_as_float(max(0x7f000000 - e, 0x00800000));
-          const float gx = sx * by, gy = sy_ * by, gz = sz_ * by;
+          const float gx = sx / m, gy = sy_ / m, gz = sz_ / m;
           const float ig = rsqrtf(gx * gx + gy * gy + gz * gz);
           const float nl = fabsf((gx * V.light[0] + gy * V.light[1] + gz * V.light[2]) * ig);
           const float nh = fabsf((gx * hv[0] + gy * hv[1] + gz * hv[2]) * ig);
