@@ -99,6 +99,7 @@ _SIGS = {
                                            _P]),
     "veg_sync_status": (ctypes.c_int, [_P, _P, ctypes.POINTER(_I64)]),
     "veg_status_fetch": (ctypes.c_int, [_P, _P, _P]),
+    "veg_zero_buffers": (ctypes.c_int, [ctypes.POINTER(_P), ctypes.POINTER(_I64), _I32, _P]),
     "veg_status_read": (ctypes.c_int, [_P, ctypes.POINTER(_I64)]),
     "veg_composite_fwd": (ctypes.c_int, [_CAMS, _I32, _I64, _P, _P, _P, _P, _P, _P, veg_tf, _P,
                                          _I32, _I32, _P, _P, _P, _P]),
@@ -283,6 +284,15 @@ def veg_status_fetch(workspace, host_status, stream=None):
     """host_status: 256-byte pinned uint8 tensor."""
     _check("veg_status_fetch",
            load().veg_status_fetch(_ptr(workspace), host_status.data_ptr(), _stream(stream)))
+
+
+def veg_zero_buffers(tensors, stream=None):
+    """Zeroes up to eight contiguous tensors."""
+    k = len(tensors)
+    _check("veg_zero_buffers",
+           load().veg_zero_buffers((_P * k)(*[t.data_ptr() for t in tensors]),
+                                   (_I64 * k)(*[t.numel() * t.element_size() for t in tensors]),
+                                   k, _stream(stream)))
 
 
 def veg_status_read(host_status):

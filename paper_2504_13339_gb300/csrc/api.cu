@@ -129,11 +129,60 @@ RenderLayout carve_render(void* ws, int64_t n, int n_views, int64_t capacity,
   return R;
 }
 
+// Block row y zeroes buffer y: 16 bytes per step, the unaligned ends bytewise.
+__global__ void __launch_bounds__(256) zero_kernel(const ZeroBuffers z) {
+  pdl_enter();
+  char* p = static_cast<char*>(z.ptr[blockIdx.y]);
+  const int64_t n = z.bytes[blockIdx.y];
+  const int64_t head = min(n, (int64_t)(-reinterpret_cast<intptr_t>(p) & 15));
+  const int64_t vec = (n - head) / 16, tail = head + vec * 16;
+  float4* v = reinterpret_cast<float4*>(p + head);
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+#pragma unroll 4
+  for (int64_t i = i0; i < vec; i += step) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (i0 < head) p[i0] = 0;
+  if (tail + i0 < n) p[tail + i0] = 0;
+}
+
 }  // namespace
+
+veg_status zero_launch(const ZeroBuffers& z, cudaStream_t stream) {
+  ZeroBuffers used = {};
+  int rows = 0;
+  int64_t most = 0;
+  for (int k = 0; k < kZeroBuffers; ++k)
+    if (z.ptr[k] && z.bytes[k] > 0) {
+      used.ptr[rows] = z.ptr[k];
+      used.bytes[rows++] = z.bytes[k];
+      most = z.bytes[k] > most ? z.bytes[k] : most;
+    }
+  if (rows == 0) return VEG_OK;
+  // 16 bytes per thread, at most about eight CTAs per SM over all buffers (a
+  // full grid for each took 24 us for five of 8 MB)
+  const int64_t blocks = (most + 4095) / 4096, cap = 1216 / rows;
+  launch_k(zero_kernel, dim3((unsigned)(blocks < cap ? blocks : cap), (unsigned)rows), 256, 0,
+           stream, used);
+  count_launch();
+  return launch_status();
+}
 
 }  // namespace veg
 
 using namespace veg;
+
+extern "C" veg_status veg_zero_buffers(void* const* buffers, const int64_t* bytes, int32_t count,
+                                       cudaStream_t stream) {
+  if (count < 0 || count > kZeroBuffers || (count > 0 && (!buffers || !bytes)))
+    return VEG_ERR_INVALID_ARGUMENT;
+  ZeroBuffers z = {};
+  for (int k = 0; k < count; ++k) {
+    if (bytes[k] < 0 || (bytes[k] > 0 && !buffers[k])) return VEG_ERR_INVALID_ARGUMENT;
+    z.ptr[k] = buffers[k];
+    z.bytes[k] = bytes[k];
+  }
+  return zero_launch(z, stream);
+}
 
 extern "C" const char* veg_status_string(veg_status status) {
   switch (status) {

@@ -123,12 +123,12 @@ extern "C" veg_status veg_composite_bwd(const veg_camera* cams, int32_t n_views,
     g2 = reinterpret_cast<float4*>(workspace);
   }
   const int64_t nrec2 = 2 * g.n * n_views;
-  if (nrec2 > 0 && cudaMemsetAsync(g2, 0, (size_t)nrec2 * sizeof(float4), stream) != cudaSuccess)
-    return VEG_ERR_CUDA;
   float2* gsh = reinterpret_cast<float2*>(grad_shade);
-  if (lit && nrec2 > 0 &&
-      cudaMemsetAsync(gsh, 0, (size_t)(nrec2 / 2) * sizeof(float2), stream) != cudaSuccess)
-    return VEG_ERR_CUDA;
+  const ZeroBuffers zero = {{g2, lit ? gsh : nullptr},
+                            {nrec2 * (int64_t)sizeof(float4),
+                             nrec2 / 2 * (int64_t)sizeof(float2)}};
+  st = zero_launch(zero, stream);
+  if (st != VEG_OK) return st;
   CompArgs A = make_args(cams, n_views, reinterpret_cast<const float4*>(splat_geo),
                          reinterpret_cast<const float4*>(splat_aux), vals,
                          reinterpret_cast<const int2*>(tile_ranges), tile_order, tf, bg,

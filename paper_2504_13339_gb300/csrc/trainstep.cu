@@ -50,10 +50,12 @@ extern "C" veg_status veg_train_step(const veg_train_args* a, int32_t view, int3
   const float* target = a->targets + ((int64_t)view * a->n_maps + map) * img;
   VEG_TRY(veg_l1_ssim_loss(a->out, target, 1, H, W, a->lambda, a->loss_grad, a->loss,
                            a->loss_ws, a->loss_ws_bytes, stream));
-  for (int k = 0; k < 5; ++k)
-    if (a->grad[k] && a->n > 0 &&
-        cudaMemsetAsync(a->grad[k], 0, (size_t)a->n * 16, stream) != cudaSuccess)
-      return VEG_ERR_CUDA;
+  veg::ZeroBuffers zero = {};
+  for (int k = 0; k < 5; ++k) {
+    zero.ptr[k] = a->grad[k];
+    zero.bytes[k] = a->n * 16;
+  }
+  VEG_TRY(veg::zero_launch(zero, stream));
   VEG_TRY(veg_composite_bwd(cam, 1, g, a->splat_geo, a->splat_aux, shade, a->tiles_touched,
                             a->vals, a->tile_ranges, a->tile_order, tf, a->bg, a->tf_group, 0,
                             a->out, a->n_contrib, a->loss_grad, nullptr, 0, a->grad[0],

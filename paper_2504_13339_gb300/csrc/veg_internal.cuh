@@ -207,6 +207,15 @@ struct ViewModels {
   int64_t n[VEG_MAX_VIEWS];
 };
 
+// Zeroes up to kZeroBuffers buffers (null or empty ones are passed over) in
+// one launch: a memset each ends the chain of early launches and costs 4 us
+// beyond its bytes.
+constexpr int kZeroBuffers = 8;
+struct ZeroBuffers {
+  void* ptr[kZeroBuffers];
+  int64_t bytes[kZeroBuffers];
+};
+veg_status zero_launch(const ZeroBuffers& z, cudaStream_t stream);
 veg_status project_launch(const CamSet& cs, int n_views, veg_gaussians g, const veg_tf* cull_tf,
                           float4* geo, float4* aux, int32_t* tiles, short4* rect,
                           cudaStream_t stream);

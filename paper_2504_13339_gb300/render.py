@@ -281,8 +281,7 @@ class SplatPipeline:
         buffers, zeroed first; lighting = (normal_beta, k_ads, light_dirs).
         With project_grads=False the projection backward is left to the
         caller (e.g. a bucketed one overlapping the gradient all-reduce)."""
-        for gbuf in grads:
-            gbuf.zero_()
+        _lib.veg_zero_buffers(grads, stream)
         self.project(mean_v, logscale_w, quat, luts, stream)
         if lighting is not None:
             self.shade(mean_v, *lighting, stream=stream)
