@@ -1103,8 +1103,13 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
   for (int j = 0; j < kCellRows; ++j) {
     const bool in = cell_item(j) < nrec;
-    t[j] = in ? (uint32_t)__ldg(&tiles[g[j]]) : 0u;
     rc[j] = in ? __ldg(&rect[g[j]]) : make_short4(0, 0, 0, 0);
+    // all records of a compacted order touch a tile: the rectangle's area
+    // then saves a second gather
+    if (tiles)
+      t[j] = in ? (uint32_t)__ldg(&tiles[g[j]]) : 0u;
+    else
+      t[j] = (uint32_t)((rc[j].z - rc[j].x) * (rc[j].w - rc[j].y));
   }
   unsigned long long e = 0, c = 0;
 #pragma unroll
@@ -1347,8 +1352,8 @@ __global__ void __launch_bounds__(256)
 }
 
 // One chunk: pairs [start, end) of a cell, the cell's first tile, its view.
-// (x, y, ox | oy << 16, view); in one CTA: the chunks before each cell
-// (cstart [n_cells + 1]), then each cell's chunks by a warp.
+// (x, y, ox | oy << 16, view).  Every CTA scans the cells' chunks (block 0
+// writes cstart [n_cells + 1]) and describes its share of the cells.
 __global__ void __launch_bounds__(kCellScanThreads)
     cell_map_kernel(const int2* __restrict__ cranges, int n_cells,
                     const __grid_constant__ CellMap cm, int max_chunks,
@@ -1387,10 +1392,11 @@ __global__ void __launch_bounds__(kCellScanThreads)
     __syncthreads();
     s_first[threadIdx.x] = carry + s_warp[warp] + inc - nch;
     s_range[threadIdx.x] = r;
-    if (c < n_cells) cstart[c] = min(s_first[threadIdx.x], max_chunks);
+    if (blockIdx.x == 0 && c < n_cells) cstart[c] = min(s_first[threadIdx.x], max_chunks);
     __syncthreads();
     // cell after cell by warp, its chunks over the lanes
-    for (int j = warp; j < kCellScanThreads && base + j < n_cells; j += 32) {
+    for (int j = warp * (int)gridDim.x + (int)blockIdx.x;
+         j < kCellScanThreads && base + j < n_cells; j += 32 * (int)gridDim.x) {
       const int f = s_first[j], cc = base + j;
       const int2 q = s_range[j];
       const int n = (q.y - q.x + kCellChunk - 1) / kCellChunk;
@@ -1405,7 +1411,7 @@ __global__ void __launch_bounds__(kCellScanThreads)
     carry += s_total;
     __syncthreads();
   }
-  if (threadIdx.x == 0) cstart[n_cells] = min(carry, max_chunks);
+  if (blockIdx.x == 0 && threadIdx.x == 0) cstart[n_cells] = min(carry, max_chunks);
 }
 
 // The tiles of the cell at `origin` that record g covers, bit ty * 8 + tx.
@@ -2007,7 +2013,8 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
     int2* cranges = reinterpret_cast<int2*>(L.dk1);
     int* cstart = reinterpret_cast<int*>(L.dk1) + 2 * n_cells;
     int4* desc = reinterpret_cast<int4*>(L.hist);
-    launch_k(cell_reduce_kernel, nb, 256, 0, stream, tiles, rect, order, cr, L.esum, csum, L.dk0);
+    launch_k(cell_reduce_kernel, nb, 256, 0, stream,
+             nrec <= kSmallRecords ? tiles : (const int32_t*)nullptr, rect, order, cr, L.esum, csum, L.dk0);
     launch_k(cell_top_kernel, 1, kCellScanThreads, 0, stream, L.esum, csum, nb, L.hdr, capacity,
              cranges, (int)n_cells);
     // sorted records end in iv0 (unpacked) or in the packed words' buffer
@@ -2029,7 +2036,7 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
     uint32_t* totals = table + kCellTiles * max_chunks;
     launch_k(ranges_kernel, pass_grid((int)grid_for(capacity, 1024), 8), 256, 0, stream, ckeys, cc, cranges,
              rec_bits, (uint32_t*)nullptr, (const WsHeader*)L.hdr);
-    launch_k(cell_map_kernel, 1, kCellScanThreads, 0, stream, (const int2*)cranges, (int)n_cells,
+    launch_k(cell_map_kernel, 16, kCellScanThreads, 0, stream, (const int2*)cranges, (int)n_cells,
              cm, (int)max_chunks, cstart, desc);
     CellPairs P;
     P.words = rec_bits ? ckeys : L.iv0;
