@@ -18,7 +18,9 @@
 // one hand-written LSD radix sort of 8-bit digits in three forms by size:
 // the whole binning in one CTA (at most 4096 records and 256 lists), one
 // look-back kernel per pass (at most 64 chunks of 2048 items), or per-chunk
-// counts, their scan and a stable scatter per pass.  The visible and
+// counts, their scan and a stable scatter per pass.  The lists of large
+// inputs are made by cells of 8x8 tiles instead of stage 2 (cell binning,
+// below): the same lists from a sixth of the sorted items.  The visible and
 // instance counts live only on the device; later kernels read them from the
 // workspace header, so no host round trip is needed and no block works past
 // them.

@@ -14,6 +14,9 @@
 // provably cannot blend cost nothing.  A pixel leaves once it has terminated
 // (T (1 - alpha) < 1e-4); a work item ends once all its pixels have left.
 //
+// Launches of few work items take a second forward kernel, whose CTA holds one
+// 8x8 block and divides staging and blending between warps (below).
+//
 // One table per work item: a splat that a table maps to no opacity never
 // enters that item's lists, and each table stops at its own termination.
 // Walking a group of 2 or 4 tables at once shares a splat's geometry but
