@@ -298,7 +298,8 @@ veg_status veg_zero_buffers(void* const* buffers, const int64_t* bytes, int32_t 
  * it.
  * tile_batch: splats of a tile's list staged per pass through shared memory
  * (128, 256 or 512; 0 = 256; the autotuner of the Python package picks per
- * shape); results do not depend on it.  The instrumented build (stats)
+ * shape); results do not depend on it, and launches of few work items do
+ * not use it.  The instrumented build (stats)
  * stages 256.
  * splat_shade: optional device float [V][n][2] of Blinn-Phong factors
  * (s_d, s_s) from veg_shade (8-byte aligned); when given, each splat is

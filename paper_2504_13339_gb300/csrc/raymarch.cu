@@ -58,6 +58,7 @@ struct MarchArgs {
   int width, height, tiles_x, tiles_per_view;
   bool shade;
   float ka, kd, ks, beta;
+  bool leave_out;  // tables without opacity (every factor of them is finite)
   float bg0, bg1, bg2;
   // empty-space skipping: per-macrocell table masks (veg_raymarch_cells)
   // over macrocells of 2^cell_shift vertex cells per axis, or null
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(256, 3)
   const float4* lut = A.lut + (known ? (int64_t)lut0 * L : 0);
   // A table is left out between entries k and k + 1 where it adds exactly
   // nothing: neither opacity is positive (the interpolated one clamps to 0)
-  // and the colours are finite (0 times them is 0).
+  // and the colours are far from infinite (0 times them, shaded, is 0).
   for (int k = threadIdx.x; k < L; k += blockDim.x) {
     unsigned m = 0u;
     for (int t = 0; known && t < ntg; ++t) {
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(256, 3)
       const float big = fmaxf(fmaxf(fmaxf(fabsf(lo.x), fabsf(lo.y)), fmaxf(fabsf(lo.z), fabsf(hi.x))),
                               fmaxf(fabsf(hi.y), fabsf(hi.z)));
       const float sum = lo.x + lo.y + lo.z + hi.x + hi.y + hi.z;  // NaN of any entry stays
-      if (lo.w > 0.0f || hi.w > 0.0f || !(big <= 3.0e37f) || sum != sum) m |= 1u << t;
+      if (lo.w > 0.0f || hi.w > 0.0f || !(big <= 1.0e30f) || sum != sum) m |= 1u << t;
     }
     s_any[k] = m;
   }
@@ -312,7 +313,7 @@ __global__ void __launch_bounds__(256, 3)
       // a NaN colour under any table, so no table is left out
       const float m = fmaxf(fmaxf(fabsf(sx), fabsf(sy_)), fabsf(sz_));
       const float chk = sx * 0.0f + sy_ * 0.0f + sz_ * 0.0f;
-      const unsigned on = chk == 0.0f ? s_any[q.k] & live : live;
+      const unsigned on = A.leave_out && chk == 0.0f ? s_any[q.k] & live : live;
       if (on == 0u) continue;
       float sd = 1.0f, ss = 0.0f;
       if (A.shade) {
@@ -483,6 +484,9 @@ extern "C" veg_status veg_raymarch_masked(const veg_camera* cams, int32_t n_view
   A.kd = material ? material->kd : 0.f;
   A.ks = material ? material->ks : 0.f;
   A.beta = material ? material->beta : 0.f;
+  // a negative shininess or huge coefficients can shade to infinity
+  A.leave_out = std::fabs(A.ka) <= 1e6f && std::fabs(A.kd) <= 1e6f && std::fabs(A.ks) <= 1e6f &&
+                A.beta >= 0.0f;
   A.bg0 = bg ? bg[0] : 0.f;
   A.bg1 = bg ? bg[1] : 0.f;
   A.bg2 = bg ? bg[2] : 0.f;
