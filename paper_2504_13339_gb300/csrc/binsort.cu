@@ -1710,11 +1710,12 @@ __global__ void __launch_bounds__(kCellChunk)
 // chunk starts), the radix histograms (chunk descriptors), and the instance buffer
 // that the cell sort does not end in (the chunk counts, the tiles' totals).
 // Taken when the tile sort would need more than one pass and the capacity is
-// at least 2^21 instances: a frame of 1.4M instances takes 316 us with it and
-// 312 with the tile sort, five views of 1.7M instances 430 and 437.  Small
-// images keep the one-pass tile sort, and calls that ask for the 64-bit keys
-// the sort that has them.
-constexpr int64_t kCellMinCapacity = (int64_t)1 << 21;
+// at least 1.3M instances.  Projection and binning with the cells and with
+// the tile sort, by capacity (1.25 times the instances): 0.56M 82 and 77 us
+// (100k Gaussians), 1.07M 106 and 103 (300k), 1.21M 98 and 104 (60k), 1.54M
+// 91 and 95 (100k), 1.95M 116 and 120 (500k).  Small images keep the one-pass
+// tile sort, and calls that ask for the 64-bit keys the sort that has them.
+constexpr int64_t kCellMinCapacity = (int64_t)5 << 18;
 bool cell_binning_fits(int64_t nrec, int64_t nranges, int64_t n_cells, int64_t capacity,
                        const Layout& L, int64_t* max_chunks) {
   *max_chunks = (capacity + kCellChunk - 1) / kCellChunk + n_cells;

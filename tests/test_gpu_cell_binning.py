@@ -3,7 +3,7 @@
 A call that asks for the 64-bit keys takes the sort of all instances by tile
 (itself checked against the oracle in test_gpu_parity.py); the same call
 without keys takes the cell binning when the views have more than 256 tiles
-and the capacity is at least 2^21 instances.  Records are random: depths
+and the capacity is at least 5 * 2^18 instances.  Records are random: depths
 with many ties, rectangles from one tile to the whole image, empty ones, and
 both sides of the cells' edges.
 """
