@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "raymarch_step.h"
 #include "veg_internal.cuh"
 
 namespace veg {
@@ -256,39 +257,31 @@ __global__ void __launch_bounds__(256, 3)
     const int R = A.R;
     // the group's tables occupy bits lut0 .. lut0 + ntg - 1 of a cell mask
     const bool skip_empty = A.cell_mask != nullptr && lut0 >= 0 && lut0 + ntg <= 32;
-    // samples per vertex cell along each axis
-    float rate[3];
+    MarchRay ray;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) rate[c] = 1.0f / (d[c] * A.inv_h * A.step);
+    for (int c = 0; c < 3; ++c) {
+      ray.eye[c] = V.eye[c];
+      ray.d[c] = d[c];
+    }
+    ray.ta = ta;
+    ray.step = A.step;
+    ray.inv_h = A.inv_h;
+    ray.R = R;
+    float rate[3];
+    march_rates(ray, rate);
     for (int k = 0; live; ++k) {
       float g[3];
       int ic[3];
       // the next sample that a table still compositing can see
       for (; k < n;) {
-        const float t = fmaf((float)k + 0.5f, A.step, ta);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          g[c] = (fmaf(t, d[c], V.eye[c]) + 1.0f) * A.inv_h;
-          ic[c] = min(max((int)floorf(g[c]), 0), R - 2);
-        }
+        const float t = march_place(ray, k, g, ic);
         if (!skip_empty) break;
         const int m[3] = {ic[0] >> A.cell_shift, ic[1] >> A.cell_shift, ic[2] >> A.cell_shift};
         const int mc = (m[2] * A.cells + m[1]) * A.cells + m[0];
         if (((__ldg(&A.cell_mask[mc]) >> lut0) & live) != 0u) break;
         // Every table still compositing has zero opacity in this macrocell:
-        // its samples would leave colour and transmittance unchanged.  A
-        // sample's macrocell index is monotone in k on each axis, so all
-        // samples up to one that lies inside are inside; that one is taken
-        // 1/64 vertex cell short of the macrocell's far faces, far beyond
-        // the float32 error of the positions (2e-3 at R = 2048).
-        float s = 1.0e6f;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const float face = (float)((rate[c] > 0.0f ? m[c] + 1 : m[c]) << A.cell_shift);
-          const float ahead = (face - g[c]) * rate[c] - fabsf(rate[c]) * 0.015625f;
-          if (d[c] != 0.0f) s = fminf(s, ahead);
-        }
-        const int next = min(k + 1 + (int)fmaxf(s, 0.0f), n);
+        // its samples would leave colour and transmittance unchanged.
+        const int next = march_next(ray, k, n, t, g, m, A.cell_shift, rate);
         if (STATS) n_skip += (unsigned)(next - k);
         k = next;
       }

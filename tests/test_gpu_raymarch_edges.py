@@ -1,0 +1,38 @@
+"""The march at the edges of its inputs: distant eyes."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2504_13339_gb300 import scenes as S
+from test_gpu_raymarch import MAT, march, prepared
+from test_gpu_raymarch_groups import masked
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+@pytest.mark.parametrize("R,cell,distance", [(65, 4, 5e4), (130, 8, 2e4), (65, 2, 1e5)])
+def test_steps_over_empty_space_from_far_away(R, cell, distance):
+    """Beyond 2^13 or so a distance's rounding is a fair part of a vertex cell:
+    the masked image must still be the plain one, bit for bit."""
+    vol = np.zeros((R, R, R), np.float32)
+    rng = np.random.default_rng(R)
+    at = rng.integers(0, R, (R * R // 2, 3))
+    vol[tuple(at.T)] = rng.uniform(0.3, 1, len(at))  # a dust of single vertices
+    luts = np.zeros((2, 1024, 4), np.float32)  # opaque from a few thousandths on
+    luts[..., :3] = rng.uniform(0, 1, (2, 1024, 3))
+    luts[0, 4:, 3] = 0.2
+    luts[1, 40:, 3] = 0.3
+    fov = math.degrees(2 * math.atan(1.5 / distance))
+    cams = [S.orbit_camera(a, b, distance, 150, 140, fov_deg=fov) for a, b in ((20, 10), (77, -40))]
+    step, v4 = 2.0 / (R - 1) * 0.5, prepared(vol)
+    plain = march(cams, v4, luts, step, MAT)
+    assert (plain[..., 3] < 1).mean() > 0.05  # the dust is seen
+    assert np.array_equal(masked(cams, v4, luts, step, cell, MAT), plain)
