@@ -277,8 +277,7 @@ __global__ void __launch_bounds__(256, 3)
         const float t = march_place(ray, k, g, ic);
         if (!skip_empty) break;
         const int m[3] = {ic[0] >> A.cell_shift, ic[1] >> A.cell_shift, ic[2] >> A.cell_shift};
-        const int mc = (m[2] * A.cells + m[1]) * A.cells + m[0];
-        if (((__ldg(&A.cell_mask[mc]) >> lut0) & live) != 0u) break;
+        if (((__ldg(&A.cell_mask[march_macrocell(m, A.cells)]) >> lut0) & live) != 0u) break;
         // Every table still compositing has zero opacity in this macrocell:
         // its samples would leave colour and transmittance unchanged.
         const int next = march_next(ray, k, n, t, g, m, A.cell_shift, rate);

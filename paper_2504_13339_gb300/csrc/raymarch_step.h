@@ -36,6 +36,12 @@ VEG_HD float march_place(const MarchRay& r, int k, float g[3], int ic[3]) {
   return t;
 }
 
+// A macrocell's place in the mask (2047^3 of them at the largest volume's
+// single cells).
+VEG_HD int64_t march_macrocell(const int m[3], int cells) {
+  return ((int64_t)m[2] * cells + m[1]) * cells + m[0];
+}
+
 // How far, in vertex cells, a sample may lie from where its distance to the
 // one at t says.  Both distances, at most |t| and the volume's diagonal, are
 // rounded to 2^-24 of that, the points to 2^-24 of at most 1 and their sums

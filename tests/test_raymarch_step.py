@@ -39,6 +39,10 @@ extern "C" void walk(const float* eye, const float* d, float ta, float tb, float
     k = next;
   }
 }
+extern "C" long long macrocell(int x, int y, int z, int cells) {
+  const int m[3] = {x, y, z};
+  return march_macrocell(m, cells);
+}
 """
 
 
@@ -85,3 +89,12 @@ def test_no_step_leaves_its_macrocell(lib, R, cell, distance, per):
     assert samples.value > 0 and wrong.value == 0
     if distance == 4.0:  # near eyes: still a few steps per macrocell
         assert steps.value * cell / per < 4.0 * samples.value
+
+
+@pytest.mark.parametrize("cells", [1, 32, 1290, 1291, 2047])
+def test_macrocell_numbers_beyond_31_bits(lib, cells):
+    """1291^3 macrocells and more (vertex cells of 1292^3 vertices) number past
+    2^31 - 1."""
+    lib.macrocell.restype = ctypes.c_longlong
+    for x, y, z in ((0, 0, 0), (cells - 1, 0, cells - 1), (cells - 1,) * 3):
+        assert lib.macrocell(x, y, z, cells) == x + cells * (y + cells * z)
