@@ -476,9 +476,12 @@ extern "C" veg_status veg_raymarch_masked(const veg_camera* cams, int32_t n_view
   A.kd = material ? material->kd : 0.f;
   A.ks = material ? material->ks : 0.f;
   A.beta = material ? material->beta : 0.f;
-  // a negative shininess or huge coefficients can shade to infinity
+  // what a sample's shade must be for zero opacity times it to be zero under
+  // every table that leaves it out (colours up to 1e30): no huge coefficient or
+  // light, and no shininess that is negative or lifts a cosine rounded up
+  // from 1 beyond the floats
   A.leave_out = std::fabs(A.ka) <= 1e6f && std::fabs(A.kd) <= 1e6f && std::fabs(A.ks) <= 1e6f &&
-                A.beta >= 0.0f;
+                A.beta >= 0.0f && A.beta <= 1e6f;
   A.bg0 = bg ? bg[0] : 0.f;
   A.bg1 = bg ? bg[1] : 0.f;
   A.bg2 = bg ? bg[2] : 0.f;
@@ -491,6 +494,7 @@ extern "C" veg_status veg_raymarch_masked(const veg_camera* cams, int32_t n_view
     for (int c = 0; c < 3; ++c) {
       V.eye[c] = -(w[0 * 4 + c] * w[3] + w[1 * 4 + c] * w[7] + w[2 * 4 + c] * w[11]);
       V.light[c] = -w[2 * 4 + c];
+      A.leave_out = A.leave_out && std::fabs(V.light[c]) <= 2.0f;
     }
     V.fx = cams[v].fx;
     V.fy = cams[v].fy;

@@ -1,5 +1,6 @@
-"""The march at the edges of its inputs: distant eyes."""
+"""The march at the edges of its inputs: distant eyes, shades without bound."""
 import math
+from dataclasses import replace
 
 import numpy as np
 import pytest
@@ -36,3 +37,24 @@ def test_steps_over_empty_space_from_far_away(R, cell, distance):
     plain = march(cams, v4, luts, step, MAT)
     assert (plain[..., 3] < 1).mean() > 0.05  # the dust is seen
     assert np.array_equal(masked(cams, v4, luts, step, cell, MAT), plain)
+
+
+@pytest.mark.parametrize("beta,scale,colour", [(1e10, 1.0, 0.5), (12.0, 1e15, 1e28)])
+def test_a_sample_shaded_to_infinity_reaches_the_image(beta, scale, colour):
+    """A shininess that lifts a cosine of 1 + 1e-7 to infinity, or a camera whose
+    rows (and headlight) are not unit: zero opacity times such a shade is NaN,
+    as it is under an opacity too small to count."""
+    R, eye = 24, np.array([1.0, 2.0, 3.0])
+    cam = S.look_at_camera(eye, 64, 64, fov_deg=0.05)  # normals within 1e-3 of the half vectors
+    x = np.linspace(-1, 1, R)
+    vol = 0.5 + 0.1 * np.einsum("c,cijk->ijk", eye, np.stack(np.meshgrid(x, x, x, indexing="ij"))[::-1])
+    vol = vol.astype(np.float32)
+    w = np.array(cam.world_to_cam, np.float32)
+    w[:, :3] *= scale
+    w[:, 3] /= scale
+    cam = replace(cam, world_to_cam=w)
+    luts = np.full((2, 16, 4), colour, np.float32)
+    luts[0, :, 3], luts[1, :, 3] = 0.0, 1e-30
+    out = march([cam], prepared(vol), luts, 1.0 / (R - 1), (0.3, 0.6, 0.25, beta))
+    assert np.isnan(out[0, 1]).any()
+    assert np.array_equal(out[0, 0], out[0, 1], equal_nan=True)
