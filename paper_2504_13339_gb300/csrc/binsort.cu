@@ -38,12 +38,17 @@ constexpr int kItems = 8;
 constexpr int kTileItems = kThreads * kItems;  // 2048 items per radix block
 constexpr int64_t kSmallRecords = 1 << 16;      // below: no compaction before the sort
 
-// Number of items to process: a fixed count, or min(*dev, cap).
+// Number of items to process: a fixed count, or min(*dev, cap).  With `after`
+// none once a sort before this kernel has timed out: the items that it did not
+// move are whatever the buffer held.  (The look-back passes do not take it:
+// they set the flag, and their threads must agree on the count.)
 struct Count {
   int64_t fixed;
   const unsigned long long* dev;
   int64_t cap;
+  const WsHeader* after;
   __device__ __forceinline__ int64_t get() const {
+    if (after && (after->flags & FLAG_TIMEOUT)) return 0;
     if (dev == nullptr) return fixed;
     unsigned long long m = *dev;
     return (int64_t)(m < (unsigned long long)cap ? m : (unsigned long long)cap);
@@ -363,7 +368,8 @@ __device__ __forceinline__ unsigned digit_peers(uint32_t d, bool valid) {
 // stride over the chunks) or found by look-back (blocks loop over tickets,
 // so a chunk's predecessors belong to blocks that are already running; a
 // look-back not answered within `spins` polls sets FLAG_TIMEOUT in the
-// header and stops waiting: the output is then void).  dtot: the digit
+// header and stops waiting: the output is then void, and since later passes
+// read places that nothing was written to, look-back passes check theirs).  dtot: the digit
 // totals of the pass.
 template <bool TABLE, int ITEMS>
 __global__ void __launch_bounds__(kThreads, ITEMS == 4 ? 6 : 4)
@@ -511,6 +517,7 @@ __global__ void __launch_bounds__(kThreads, ITEMS == 4 ? 6 : 4)
       uint32_t key = s_keys[p];
       uint32_t d = ((key - kb) >> shift) & mask;
       uint32_t g = s_dbase[d] + (uint32_t)p;
+      if (!TABLE && (int64_t)g >= n) continue;  // only after a timeout
       kout[g] = key;
       if (vout) vout[g] = s_vals[p];  // keys-only sorts carry no values
     }
@@ -825,9 +832,8 @@ __global__ void zero_ranges_kernel(int2* __restrict__ ranges, int64_t count,
 // marks "no neighbour".
 __global__ void ranges_kernel(const uint32_t* __restrict__ keys, Count cnt,
                               int2* __restrict__ ranges, int key_shift,
-                              uint32_t* __restrict__ vals, const WsHeader* hdr) {
+                              uint32_t* __restrict__ vals) {
   pdl_enter();
-  if (hdr->flags & FLAG_TIMEOUT) return;  // void lists: every range stays empty
   const int64_t n = cnt.get();
   // a bounded grid strides over the items: their count is far below the
   // capacity that the host knows
@@ -2010,12 +2016,12 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
   // 1. the visible records (touching a tile) in index order, then their
   //    depth sort; small inputs sort every record with culled ones last
   //    (same order, fewer launches)
-  Count cr{0, &L.hdr->n_visible, nrec};
+  Count cr{0, &L.hdr->n_visible, nrec, nullptr};
   if (nrec <= kSmallRecords) {
     launch_k(depth_keys_kernel, grid_for(nrec, 256), 256, 0, stream, geo, tiles, nrec, L.dk0, L.dv0,
              L.hdr);
     count_launch();
-    cr = Count{nrec, nullptr, 0};
+    cr = Count{nrec, nullptr, 0, nullptr};
   } else {
     launch_k(visible_count_kernel, L.nb_rec, kThreads, 0, stream, tiles, nrec, L.bsum);
     launch_k(chunk_scan_kernel, 1, 1024, 0, stream, L.bsum, L.nb_rec, &L.hdr->n_visible);
@@ -2027,11 +2033,12 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
   uint32_t* const dk[2] = {L.dk0, L.dk1};
   uint32_t* const dv[2] = {L.dv0, L.dv1};
   const SortedVals order = radix_sort(dk, dv, cr, 32, L.nb_rec, L, 0, L.hdr, stream);
+  cr.after = L.hdr;
   const CellMap cm = make_cellmap(cams, n_views);
   const int64_t n_cells = cm.cell_off[n_views];
   int rec_bits = 1;
   while (((int64_t)1 << rec_bits) < nrec) ++rec_bits;
-  Count ci{0, &L.hdr->n_instances, capacity};
+  Count ci{0, &L.hdr->n_instances, capacity, nullptr};
   const int nb_inst = (int)std::max<int64_t>(1, (capacity + kTileItems - 1) / kTileItems);
   int64_t max_chunks = 0;
   if (!keys && cell_binning_fits(nrec, nranges, n_cells, capacity, L, &max_chunks)) {
@@ -2059,13 +2066,13 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
              (const unsigned long long*)L.esum, (const unsigned long long*)csum, cr, n, cm,
              capacity, rec_bits, kbuf[0], vbuf[0], L.hdr);
     count_launch(3);
-    Count cc{0, &L.hdr->n_cells, capacity};
+    const Count cc{0, &L.hdr->n_cells, capacity, nullptr};
     radix_sort(kbuf, vbuf, cc, bits, nb_inst, L, 1, nullptr, stream, kLookbackSpins, rec_bits);
     const uint32_t* ckeys = kbuf[passes & 1];
     uint32_t* table = kbuf[(passes & 1) ^ 1];
     uint32_t* totals = table + kCellTiles * max_chunks;
     launch_k(ranges_kernel, pass_grid((int)grid_for(capacity, 1024), 8), 256, 0, stream, ckeys, cc, cranges,
-             rec_bits, (uint32_t*)nullptr, (const WsHeader*)L.hdr);
+             rec_bits, (uint32_t*)nullptr);
     launch_k(cell_map_kernel, 16, kCellScanThreads, 0, stream, (const int2*)cranges, (int)n_cells,
              cm, (int)max_chunks, cstart, desc);
     CellPairs P;
@@ -2109,10 +2116,11 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
   count_launch();
   radix_sort(kbuf, vbuf, ci, bits, nb_inst, L, 1, nullptr, stream, kLookbackSpins, rec_bits);
   const uint32_t* fkeys = kbuf[passes & 1];
+  ci.after = L.hdr;
   // 4. per-tile ranges (and the records, from packed words) and optional
   //    64-bit keys
   launch_k(ranges_kernel, pass_grid((int)grid_for(capacity, 1024), 8), 256, 0, stream, fkeys, ci, ranges, rec_bits,
-           packed ? vals : (uint32_t*)nullptr, (const WsHeader*)L.hdr);
+           packed ? vals : (uint32_t*)nullptr);
   count_launch();
   if (keys) {
     launch_k(keys64_kernel, grid_for(capacity, 256), 256, 0, stream, fkeys, vals, ci, geo, vm,
@@ -2309,7 +2317,7 @@ extern "C" veg_status veg_radix_lookback_check(void* workspace, size_t workspace
   count_launch();
   uint32_t* const dk[2] = {L.dk0, L.dk1};
   uint32_t* const dv[2] = {L.dv0, L.dv1};
-  radix_sort(dk, dv, Count{n, nullptr, 0}, 32, L.nb_rec, L, 0, nullptr, stream,
+  radix_sort(dk, dv, Count{n, nullptr, 0, nullptr}, 32, L.nb_rec, L, 0, nullptr, stream,
              spins);  // 4 passes: into dk0, dv0
   if (cudaMemcpyAsync(keys_out, L.dk0, (size_t)n * 4, cudaMemcpyDeviceToDevice, stream) !=
           cudaSuccess ||
