@@ -1386,9 +1386,13 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// One chunk: pairs [start, end) of a cell, the cell's first tile, its view.
-// (x, y, ox | oy << 16, view).  Every CTA scans the cells' chunks (block 0
-// writes cstart [n_cells + 1]) and describes its share of the cells.
+// One chunk: its first pair and their number (an end could pass 2^31), the
+// cell's first tile, its view: (first, pairs, ox | oy << 16, view).  Every CTA
+// scans the cells' chunks (block 0 writes cstart [n_cells + 1]) and describes
+// its share of the cells.
+__device__ __forceinline__ int cell_chunks(int2 r) {
+  return (int)(((unsigned)(r.y - r.x) + kCellChunk - 1) / kCellChunk);
+}
 __global__ void __launch_bounds__(kCellScanThreads)
     cell_map_kernel(const int2* __restrict__ cranges, int n_cells,
                     const __grid_constant__ CellMap cm, int max_chunks,
@@ -1404,7 +1408,7 @@ __global__ void __launch_bounds__(kCellScanThreads)
     const int c = base + (int)threadIdx.x;
     int2 r = make_int2(0, 0);
     if (c < n_cells) r = cranges[c];
-    const int nch = (r.y - r.x + kCellChunk - 1) / kCellChunk;
+    const int nch = cell_chunks(r);
     int inc = nch;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1434,13 +1438,13 @@ __global__ void __launch_bounds__(kCellScanThreads)
          j < kCellScanThreads && base + j < n_cells; j += 32 * (int)gridDim.x) {
       const int f = s_first[j], cc = base + j;
       const int2 q = s_range[j];
-      const int n = (q.y - q.x + kCellChunk - 1) / kCellChunk;
+      const int n = cell_chunks(q);
       int view = 0;
       while (view + 1 < cm.n_views && cm.cell_off[view + 1] <= cc) ++view;
       const int cell = cc - cm.cell_off[view], cx = cm.cells_x[view];
       const int origin = ((cell % cx) << kCellShift) | (((cell / cx) << kCellShift) << 16);
       for (int k = lane; k < n && f + k < max_chunks; k += 32)
-        desc[f + k] = make_int4(q.x + k * kCellChunk, min(q.x + (k + 1) * kCellChunk, q.y),
+        desc[f + k] = make_int4(q.x + k * kCellChunk, min(kCellChunk, q.y - q.x - k * kCellChunk),
                                 origin, view);
     }
     carry += s_total;
@@ -1504,13 +1508,11 @@ __global__ void __launch_bounds__(256)
     uint32_t g[8];
     short4 rc[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int i = d.x + j * 32 + lane;
-      g[j] = i < d.y ? __ldg(P.words + i) & P.rec_mask : 0u;
-    }
+    for (int j = 0; j < 8; ++j)
+      g[j] = j * 32 + lane < d.y ? __ldg(P.words + d.x + j * 32 + lane) & P.rec_mask : 0u;
 #pragma unroll
     for (int j = 0; j < 8; ++j)
-      rc[j] = d.x + j * 32 + lane < d.y ? __ldg(P.rect + g[j]) : make_short4(0, 0, 0, 0);
+      rc[j] = j * 32 + lane < d.y ? __ldg(P.rect + g[j]) : make_short4(0, 0, 0, 0);
     uint32_t lo = 0, hi = 0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -1628,10 +1630,10 @@ __global__ void __launch_bounds__(kCellChunk)
   // the current chunk is staged and written
   auto chunk = [&](int k) { return k < total ? __ldg(desc + k) : make_int4(0, 0, 0, 0); };
   auto pair_of = [&](int4 d) {
-    return d.x + tid < d.y ? __ldg(P.words + d.x + tid) & P.rec_mask : 0u;
+    return tid < d.y ? __ldg(P.words + d.x + tid) & P.rec_mask : 0u;
   };
   auto rect_of = [&](int4 d, uint32_t g) {
-    return d.x + tid < d.y ? __ldg(P.rect + g) : make_short4(0, 0, 0, 0);
+    return tid < d.y ? __ldg(P.rect + g) : make_short4(0, 0, 0, 0);
   };
   auto start_of = [&](int4 d, int k) {
     uint32_t at = 0;
