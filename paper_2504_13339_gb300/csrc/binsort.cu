@@ -38,22 +38,26 @@ constexpr int kItems = 8;
 constexpr int kTileItems = kThreads * kItems;  // 2048 items per radix block
 constexpr int64_t kSmallRecords = 1 << 16;      // below: no compaction before the sort
 
-// Number of items to process: a fixed count, or min(*dev, cap).  With `after`
-// none once a sort before this kernel has timed out: the items that it did not
-// move are whatever the buffer held.  (The look-back passes do not take it:
-// they set the flag, and their threads must agree on the count.)
+// Number of items to process: a fixed count, or min(*dev, cap).
 struct Count {
   int64_t fixed;
   const unsigned long long* dev;
   int64_t cap;
-  const WsHeader* after;
   __device__ __forceinline__ int64_t get() const {
-    if (after && (after->flags & FLAG_TIMEOUT)) return 0;
     if (dev == nullptr) return fixed;
     unsigned long long m = *dev;
     return (int64_t)(m < (unsigned long long)cap ? m : (unsigned long long)cap);
   }
 };
+
+// The items of a kernel behind a sort that may have timed out (`after`, the
+// status header; null for sorts that wait for nothing): none if it did, since
+// the places that it did not write hold whatever the buffer held.  (The
+// look-back passes themselves set the flag, and their threads must agree on
+// the count: they check their places instead.)
+__device__ __forceinline__ int64_t count_after(const Count& c, const WsHeader* after) {
+  return after && (after->flags & FLAG_TIMEOUT) ? 0 : c.get();
+}
 
 __device__ __forceinline__ float rcp_approx_f(float x) {
   float y;
@@ -664,11 +668,11 @@ __global__ void __launch_bounds__(1024)
 // blocks of the emission kernel).
 __global__ void __launch_bounds__(256)
     count_reduce_kernel(const int32_t* __restrict__ tiles, SortedVals sorted, Count cnt,
-                        unsigned long long* __restrict__ bsum) {
+                        const WsHeader* after, unsigned long long* __restrict__ bsum) {
   pdl_enter();
   const uint32_t* __restrict__ order = sorted.get();
   __shared__ unsigned long long s_warp[8];
-  const int64_t nrec = cnt.get();
+  const int64_t nrec = count_after(cnt, after);
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   unsigned long long acc = i < nrec ? (unsigned)tiles[order[i]] : 0u;
 #pragma unroll
@@ -737,13 +741,13 @@ __global__ void __launch_bounds__(1024)
 __global__ void __launch_bounds__(256)
     emit_kernel(const int32_t* __restrict__ tiles, const short4* __restrict__ rect,
                 SortedVals sorted, const unsigned long long* __restrict__ bsum, Count visible,
-                int64_t n_per_view, ViewMap vm, int64_t capacity, int rec_bits,
-                uint32_t* __restrict__ ikeys, uint32_t* __restrict__ ivals) {
+                const WsHeader* after, int64_t n_per_view, ViewMap vm, int64_t capacity,
+                int rec_bits, uint32_t* __restrict__ ikeys, uint32_t* __restrict__ ivals) {
   pdl_enter();
   __shared__ unsigned long long s_warp[8];
   const uint32_t* __restrict__ order = sorted.get();
   const int lane = threadIdx.x & 31;
-  const int64_t nrec = visible.get();
+  const int64_t nrec = count_after(visible, after);
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t g = 0, cnt = 0;
   short4 rc = make_short4(0, 0, 0, 0);
@@ -830,11 +834,11 @@ __global__ void zero_ranges_kernel(int2* __restrict__ ranges, int64_t count,
 // aligned): a run starts where the key differs from its predecessor and
 // ends where it differs from its successor.  Keys are < 2^31, so 0xffffffff
 // marks "no neighbour".
-__global__ void ranges_kernel(const uint32_t* __restrict__ keys, Count cnt,
+__global__ void ranges_kernel(const uint32_t* __restrict__ keys, Count cnt, const WsHeader* after,
                               int2* __restrict__ ranges, int key_shift,
                               uint32_t* __restrict__ vals) {
   pdl_enter();
-  const int64_t n = cnt.get();
+  const int64_t n = count_after(cnt, after);
   // a bounded grid strides over the items: their count is far below the
   // capacity that the host knows
   for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i0 < n;
@@ -874,10 +878,10 @@ __global__ void ranges_kernel(const uint32_t* __restrict__ keys, Count cnt,
 // key = (view << (tb + 32)) | (tile of the view << 32) | depth bits, with tb
 // the tile bits of the largest view.
 __global__ void keys64_kernel(const uint32_t* __restrict__ tkeys, const uint32_t* __restrict__ vals,
-                              Count cnt, const float4* __restrict__ geo, ViewMap vm, int tb,
-                              int key_shift, uint64_t* __restrict__ keys64) {
+                              Count cnt, const WsHeader* after, const float4* __restrict__ geo,
+                              ViewMap vm, int tb, int key_shift, uint64_t* __restrict__ keys64) {
   pdl_enter();
-  const int64_t n = cnt.get();
+  const int64_t n = count_after(cnt, after);
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   uint32_t tk = tkeys[i] >> key_shift;
@@ -1094,12 +1098,12 @@ __device__ __forceinline__ int64_t cell_item(int j) {
 constexpr uint32_t kNoCells = 0x0000ffffu;  // first cell beyond the last
 __global__ void __launch_bounds__(256)
     cell_reduce_kernel(const int32_t* __restrict__ tiles, const short4* __restrict__ rect,
-                       SortedVals sorted, Count cnt, unsigned long long* __restrict__ esum,
-                       unsigned long long* __restrict__ csum, uint32_t* __restrict__ cells) {
+                       SortedVals sorted, Count cnt, const WsHeader* after,
+                       unsigned long long* __restrict__ esum, unsigned long long* __restrict__ csum, uint32_t* __restrict__ cells) {
   pdl_enter();
   const uint32_t* __restrict__ order = sorted.get();
   __shared__ unsigned long long s_e[8], s_c[8];
-  const int64_t nrec = cnt.get();
+  const int64_t nrec = count_after(cnt, after);
   if ((int64_t)blockIdx.x * kCellBlock >= nrec) {  // block-uniform
     if (threadIdx.x == 0) esum[blockIdx.x] = csum[blockIdx.x] = 0ull;
     return;
@@ -1250,14 +1254,14 @@ __global__ void __launch_bounds__(256)
     cell_emit_kernel(const int32_t* __restrict__ tiles, const uint32_t* __restrict__ cells,
                      SortedVals sorted, const unsigned long long* __restrict__ esum,
                      const unsigned long long* __restrict__ csum, Count visible,
-                     int64_t n_per_view, const __grid_constant__ CellMap cm, int64_t capacity,
-                     int rec_bits, uint32_t* __restrict__ ckeys, uint32_t* __restrict__ cvals,
+                     const WsHeader* after, int64_t n_per_view,
+                     const __grid_constant__ CellMap cm, int64_t capacity, int rec_bits, uint32_t* __restrict__ ckeys, uint32_t* __restrict__ cvals,
                      WsHeader* __restrict__ hdr) {
   pdl_enter();
   __shared__ unsigned long long s_e[8], s_c[8];
   const uint32_t* __restrict__ order = sorted.get();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t nrec = visible.get();
+  const int64_t nrec = count_after(visible, after);
   const bool over = (hdr->flags & FLAG_CAPACITY) != 0u;
   if ((int64_t)blockIdx.x * kCellBlock >= nrec) return;  // block-uniform
   uint32_t g[kCellRows], packed[kCellRows];
@@ -2018,12 +2022,12 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
   // 1. the visible records (touching a tile) in index order, then their
   //    depth sort; small inputs sort every record with culled ones last
   //    (same order, fewer launches)
-  Count cr{0, &L.hdr->n_visible, nrec, nullptr};
+  Count cr{0, &L.hdr->n_visible, nrec};
   if (nrec <= kSmallRecords) {
     launch_k(depth_keys_kernel, grid_for(nrec, 256), 256, 0, stream, geo, tiles, nrec, L.dk0, L.dv0,
              L.hdr);
     count_launch();
-    cr = Count{nrec, nullptr, 0, nullptr};
+    cr = Count{nrec, nullptr, 0};
   } else {
     launch_k(visible_count_kernel, L.nb_rec, kThreads, 0, stream, tiles, nrec, L.bsum);
     launch_k(chunk_scan_kernel, 1, 1024, 0, stream, L.bsum, L.nb_rec, &L.hdr->n_visible);
@@ -2035,12 +2039,12 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
   uint32_t* const dk[2] = {L.dk0, L.dk1};
   uint32_t* const dv[2] = {L.dv0, L.dv1};
   const SortedVals order = radix_sort(dk, dv, cr, 32, L.nb_rec, L, 0, L.hdr, stream);
-  cr.after = L.hdr;
+  const WsHeader* const after_depth = L.nb_rec <= kLookbackMaxChunks ? L.hdr : nullptr;
   const CellMap cm = make_cellmap(cams, n_views);
   const int64_t n_cells = cm.cell_off[n_views];
   int rec_bits = 1;
   while (((int64_t)1 << rec_bits) < nrec) ++rec_bits;
-  Count ci{0, &L.hdr->n_instances, capacity, nullptr};
+  Count ci{0, &L.hdr->n_instances, capacity};
   const int nb_inst = (int)std::max<int64_t>(1, (capacity + kTileItems - 1) / kTileItems);
   int64_t max_chunks = 0;
   if (!keys && cell_binning_fits(nrec, nranges, n_cells, capacity, L, &max_chunks)) {
@@ -2053,7 +2057,8 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
     int* cstart = reinterpret_cast<int*>(L.dk1) + 2 * n_cells;
     int4* desc = reinterpret_cast<int4*>(L.hist);
     launch_k(cell_reduce_kernel, nb, 256, 0, stream,
-             nrec <= kSmallRecords ? tiles : (const int32_t*)nullptr, rect, order, cr, L.esum, csum, L.dk0);
+             nrec <= kSmallRecords ? tiles : (const int32_t*)nullptr, rect, order, cr, after_depth,
+             L.esum, csum, L.dk0);
     launch_k(cell_top_kernel, 1, kCellScanThreads, 0, stream, L.esum, csum, nb, L.hdr, capacity,
              cranges, (int)n_cells);
     // sorted records end in iv0 (unpacked) or in the packed words' buffer
@@ -2065,16 +2070,16 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
       vbuf[(passes & 1) ^ 1] = vals;
     }
     launch_k(cell_emit_kernel, nb, 256, 0, stream, tiles, (const uint32_t*)L.dk0, order,
-             (const unsigned long long*)L.esum, (const unsigned long long*)csum, cr, n, cm,
+             (const unsigned long long*)L.esum, (const unsigned long long*)csum, cr, after_depth, n, cm,
              capacity, rec_bits, kbuf[0], vbuf[0], L.hdr);
     count_launch(3);
-    const Count cc{0, &L.hdr->n_cells, capacity, nullptr};
+    const Count cc{0, &L.hdr->n_cells, capacity};
     radix_sort(kbuf, vbuf, cc, bits, nb_inst, L, 1, nullptr, stream, kLookbackSpins, rec_bits);
     const uint32_t* ckeys = kbuf[passes & 1];
     uint32_t* table = kbuf[(passes & 1) ^ 1];
     uint32_t* totals = table + kCellTiles * max_chunks;
-    launch_k(ranges_kernel, pass_grid((int)grid_for(capacity, 1024), 8), 256, 0, stream, ckeys, cc, cranges,
-             rec_bits, (uint32_t*)nullptr);
+    launch_k(ranges_kernel, pass_grid((int)grid_for(capacity, 1024), 8), 256, 0, stream, ckeys, cc,
+             (const WsHeader*)nullptr, cranges, rec_bits, (uint32_t*)nullptr);
     launch_k(cell_map_kernel, 16, kCellScanThreads, 0, stream, (const int2*)cranges, (int)n_cells,
              cm, (int)max_chunks, cstart, desc);
     CellPairs P;
@@ -2095,7 +2100,7 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
     return launch_status();
   }
   // 2. instance offsets in depth order, total into the header
-  launch_k(count_reduce_kernel, L.nb_emit, 256, 0, stream, tiles, order, cr, L.esum);
+  launch_k(count_reduce_kernel, L.nb_emit, 256, 0, stream, tiles, order, cr, after_depth, L.esum);
   launch_k(count_top_kernel, 1, 1024, 0, stream, L.esum, L.nb_emit, L.hdr, capacity);
   count_launch(2);
   // 3. emit (tile key, record) pairs, then stable sort by tile key.  When
@@ -2114,19 +2119,20 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
     vbuf[passes % 2 == 0 ? 1 : 0] = L.iv0;
   }
   launch_k(emit_kernel, L.nb_emit, 256, 0, stream, tiles, rect, order,
-           (const unsigned long long*)L.esum, cr, n, vm, capacity, rec_bits, kbuf[0], vbuf[0]);
+           (const unsigned long long*)L.esum, cr, after_depth, n, vm, capacity, rec_bits, kbuf[0],
+           vbuf[0]);
   count_launch();
   radix_sort(kbuf, vbuf, ci, bits, nb_inst, L, 1, nullptr, stream, kLookbackSpins, rec_bits);
   const uint32_t* fkeys = kbuf[passes & 1];
-  ci.after = L.hdr;
+  const WsHeader* const after_tiles = nb_inst <= kLookbackMaxChunks ? L.hdr : nullptr;
   // 4. per-tile ranges (and the records, from packed words) and optional
   //    64-bit keys
-  launch_k(ranges_kernel, pass_grid((int)grid_for(capacity, 1024), 8), 256, 0, stream, fkeys, ci, ranges, rec_bits,
-           packed ? vals : (uint32_t*)nullptr);
+  launch_k(ranges_kernel, pass_grid((int)grid_for(capacity, 1024), 8), 256, 0, stream, fkeys, ci,
+           after_tiles, ranges, rec_bits, packed ? vals : (uint32_t*)nullptr);
   count_launch();
   if (keys) {
-    launch_k(keys64_kernel, grid_for(capacity, 256), 256, 0, stream, fkeys, vals, ci, geo, vm,
-             tile_bits_of(vm.max_tiles), rec_bits, keys);
+    launch_k(keys64_kernel, grid_for(capacity, 256), 256, 0, stream, fkeys, vals, ci, after_tiles,
+             geo, vm, tile_bits_of(vm.max_tiles), rec_bits, keys);
     count_launch();
   }
   return launch_status();
@@ -2319,7 +2325,7 @@ extern "C" veg_status veg_radix_lookback_check(void* workspace, size_t workspace
   count_launch();
   uint32_t* const dk[2] = {L.dk0, L.dk1};
   uint32_t* const dv[2] = {L.dv0, L.dv1};
-  radix_sort(dk, dv, Count{n, nullptr, 0, nullptr}, 32, L.nb_rec, L, 0, nullptr, stream,
+  radix_sort(dk, dv, Count{n, nullptr, 0}, 32, L.nb_rec, L, 0, nullptr, stream,
              spins);  // 4 passes: into dk0, dv0
   if (cudaMemcpyAsync(keys_out, L.dk0, (size_t)n * 4, cudaMemcpyDeviceToDevice, stream) !=
           cudaSuccess ||
