@@ -1768,7 +1768,6 @@ constexpr int kOneCtaRecords = 4096;                    // 4 per thread, 128 per
 constexpr int kOneCtaLists = 256;
 
 struct OneCtaSmem {
-  uint32_t key[2][kOneCtaRecords];
   uint32_t rec[2][kOneCtaRecords];
   uint32_t off[kOneCtaRecords + 1];            // instance offsets of the sorted records
   uint32_t lbase[kOneCtaRecords];              // list of each sorted record's first tile
@@ -1778,6 +1777,12 @@ struct OneCtaSmem {
   uint32_t ltotal[kOneCtaLists];
   uint32_t scan[kOneCtaWarps];
   uint32_t kmin, kmax, nvis;
+  union {
+    uint32_t key[2][kOneCtaRecords];
+    // once sorted: per 32 lists and round, each lane's word of the lists that
+    // its record touches, then of the records that touch its list
+    uint32_t sets[kOneCtaLists / 32][kOneCtaRecords / kOneCtaThreads][kOneCtaThreads];
+  };
 };
 
 __global__ void __launch_bounds__(kOneCtaThreads, 1)
@@ -1921,33 +1926,38 @@ __global__ void __launch_bounds__(kOneCtaThreads, 1)
     hdr->flags = (int64_t)total > capacity ? FLAG_CAPACITY : 0u;
   }
 
-  // 4. the first m_cap instances sorted by list, 32 lists at a time.  A lane
-  //    holds one record of its warp's round and the set of lists it touches;
-  //    transposed over the warp, lane l has the ordered set of the round's
-  //    records that touch list l, so a warp counts with popcounts, and after
-  //    a prefix over the warps writes each set's records in order (lane
-  //    masks set by shared atomics, list by list, were 22 of the kernel's 59
-  //    thousand cycles on 4096 records over 64 lists; this, the reads of step
-  //    3 together and runs no longer than the visible records need took it
-  //    from 29.0 to 21.3 us).
-  auto touching = [&](int round, int word) {
+  // 4. the first m_cap instances sorted by list.  A lane holds one record of its
+  //    warp's round and sets the bits of the lists it touches, row by row;
+  //    transposed over the warp 32 lists at a time, lane l has the ordered set
+  //    of the round's records that touch list l, so a warp counts with
+  //    popcounts, and after a prefix over the warps writes each set's records
+  //    in order.  The sets are kept between the two: forming them twice, and
+  //    every record's rows for each 32 lists, took 73 us for 4096 records over
+  //    256 lists (lane masks set by shared atomics, list by list: 64; this form
+  //    49), and 36 over 64 lists (45; 34).
+  const int words = (nlists + 31) / 32;
+  for (int round = 0; round < rounds; ++round) {
     const int j = run0 + round * 32 + lane;
-    uint32_t bits = 0u;
+    for (int w = 0; w < words; ++w) S.sets[w][round][tid] = 0u;
     if (j < nvis) {
       const int e0 = (int)min(S.off[j], m_cap), left = (int)min(S.off[j + 1], m_cap) - e0;
       const int wx = max((int)(S.shape[j] & 0xffffu), 1), tx = (int)(S.shape[j] >> 16);
-      int first = (int)S.lbase[j] - 32 * word;  // tiles row-major: first + row * tx + rx
-      for (int t = 0; t < left; t += wx, first += tx) {
-        const int lo = max(first, 0), hi = min(first + min(wx, left - t), 32);
-        if (lo < hi) bits |= (0xffffffffu << lo) & (0xffffffffu >> (32 - hi));
-      }
+      int first = (int)S.lbase[j];  // tiles row-major: first + row * tx + rx
+      for (int t = 0; t < left; t += wx, first += tx)
+        for (int l = first, end = min(first + min(wx, left - t), kOneCtaLists); l < end;) {
+          const int stop = min(end, (l | 31) + 1);  // of the word that holds l
+          S.sets[l >> 5][round][tid] |= (0xffffffffu >> (32 - (stop - l))) << (l & 31);
+          l = stop;
+        }
     }
-    return warp_transpose(bits);
-  };
-  const int words = (nlists + 31) / 32;
+  }
   for (int w = 0; w < words; ++w) {
     uint32_t c = 0;
-    for (int round = 0; round < rounds; ++round) c += __popc(touching(round, w));
+    for (int round = 0; round < rounds; ++round) {
+      const uint32_t bits = warp_transpose(S.sets[w][round][tid]);
+      S.sets[w][round][tid] = bits;
+      c += __popc(bits);
+    }
     S.wcnt[warp][32 * w + lane] = (uint16_t)c;
   }
   __syncthreads();
@@ -1971,7 +1981,7 @@ __global__ void __launch_bounds__(kOneCtaThreads, 1)
     const int l = 32 * w + lane;
     uint32_t q = l < nlists ? S.lstart[l] + S.wcnt[warp][l] : 0u;
     for (int round = 0; round < rounds; ++round) {
-      for (uint32_t bits = touching(round, w); bits; bits &= bits - 1, ++q) {
+      for (uint32_t bits = S.sets[w][round][tid]; bits; bits &= bits - 1, ++q) {
         const uint32_t g = order[run0 + round * 32 + __ffs((int)bits) - 1];
         if (q >= m_cap) continue;  // never, when the counts agree
         vals[q] = g;
