@@ -298,9 +298,9 @@ veg_status veg_zero_buffers(void* const* buffers, const int64_t* bytes, int32_t 
  * it.
  * tile_batch: splats of a tile's list staged per pass through shared memory
  * (128, 256 or 512; 0 = 256; the autotuner of the Python package picks per
- * shape); results do not depend on it, and launches of few work items do
- * not use it.  The instrumented build (stats)
- * stages 256.
+ * shape); results do not depend on it.  Launches of few (tile, table) items
+ * divide a tile between CTAs instead and do not use it:
+ * veg_composite_fwd_batch tells.  The instrumented build (stats) stages 256.
  * splat_shade: optional device float [V][n][2] of Blinn-Phong factors
  * (s_d, s_s) from veg_shade (8-byte aligned); when given, each splat is
  * blended with the colour s_d rgb + s_s of Eq. 2 instead of rgb.  Opacity,
@@ -321,6 +321,13 @@ veg_status veg_composite_fwd(const veg_camera* cams, int32_t n_views, int64_t n,
                              int32_t tf_group, int32_t tile_batch, float* out,
                              int32_t* n_contrib, unsigned long long* stats,
                              cudaStream_t stream);
+
+/* The tile batch that veg_composite_fwd takes for these sizes (tf's lut is not
+ * read, view_tf only tested for NULL): `tile_batch` or its default, or 0 for a
+ * launch that stages no batches.  Host only; batch: host.
+ */
+veg_status veg_composite_fwd_batch(const veg_camera* cams, int32_t n_views, int64_t n, veg_tf tf,
+                                   int32_t tile_batch, int32_t* batch);
 
 /*
  * veg_composite_bwd -- manual gradients of the render (Sec. 3.3, backward

@@ -103,6 +103,8 @@ _SIGS = {
     "veg_status_read": (ctypes.c_int, [_P, ctypes.POINTER(_I64)]),
     "veg_composite_fwd": (ctypes.c_int, [_CAMS, _I32, _I64, _P, _P, _P, _P, _P, _P, veg_tf, _P,
                                          _I32, _I32, _P, _P, _P, _P]),
+    "veg_composite_fwd_batch": (ctypes.c_int, [_CAMS, _I32, _I64, veg_tf, _I32,
+                                               ctypes.POINTER(_I32)]),
     "veg_composite_bwd_workspace_size": (ctypes.c_int, [_I64, _I32, ctypes.POINTER(_SZ)]),
     "veg_composite_bwd": (ctypes.c_int, [_CAMS, _I32, veg_gaussians, _P, _P, _P, _P, _P, _P, _P,
                                          veg_tf, _P, _I32, _I32, _P, _P, _P, _P, _SZ, _P, _P, _P,
@@ -318,6 +320,15 @@ def veg_composite_fwd(cams, n, splat_geo, splat_aux, vals, tile_ranges, tf, bg, 
                                     _ptr(splat_shade), _ptr(vals), _ptr(tile_ranges), _ptr(tile_order), tf,
                                     ctypes.cast(bgc, ctypes.c_void_p), tf_group, tile_batch,
                                     _ptr(out), _ptr(n_contrib), _ptr(stats), _stream(stream)))
+
+
+def veg_composite_fwd_batch(cams, n, tf, tile_batch=0) -> int:
+    """Splats per staged batch of a forward of these sizes, 0 if it stages none."""
+    out = _I32()
+    _check("veg_composite_fwd_batch",
+           load().veg_composite_fwd_batch(cams, len(cams), int(n), tf, int(tile_batch),
+                                          ctypes.byref(out)))
+    return out.value
 
 
 def veg_composite_bwd_workspace_size(n, n_views) -> int:

@@ -17,14 +17,13 @@ veg_status composite_fwd_launch(const veg_camera* cams, int n_views, int64_t n,
                                 int tile_batch, float4* out, int32_t* n_contrib,
                                 unsigned long long* stats, cudaStream_t stream) {
   CompArgs A = make_args(cams, n_views, geo, aux, vals, ranges, order, tf, bg, shade);
-  (void)n;
   (void)tf_group;  // every pass composites one table
   const int B = pick_batch(tile_batch);
   if (stats)
     return shade ? VEG_ERR_UNSUPPORTED
                  : launch_fwd<256, true, false>(A, n_views, out, n_contrib, stats, stream);
-  return shade ? fwd_batch<true>(B, A, n_views, out, n_contrib, stream)
-               : fwd_batch<false>(B, A, n_views, out, n_contrib, stream);
+  return shade ? fwd_batch<true>(B, A, n_views, n, out, n_contrib, stream)
+               : fwd_batch<false>(B, A, n_views, n, out, n_contrib, stream);
 }
 
 size_t composite_bwd_ws_bytes(int64_t n, int n_views) {
@@ -73,6 +72,17 @@ extern "C" veg_status veg_composite_fwd(const veg_camera* cams, int32_t n_views,
                               reinterpret_cast<const int2*>(tile_ranges), tile_order, tf, bg,
                               splat_shade, tf_group, tile_batch, reinterpret_cast<float4*>(out),
                               n_contrib, stats, stream);
+}
+
+extern "C" veg_status veg_composite_fwd_batch(const veg_camera* cams, int32_t n_views, int64_t n,
+                                              veg_tf tf, int32_t tile_batch, int32_t* batch) {
+  veg_status st = check_cameras(cams, n_views);
+  if (st != VEG_OK) return st;
+  if (!batch || n < 0 || tf.lut_size < 2 || tf.n_tf < 1 || tf.n_tf > 4096 || !batch_ok(tile_batch))
+    return VEG_ERR_INVALID_ARGUMENT;
+  const int64_t items = total_tiles_of(cams, n_views) * (tf.view_tf ? 1 : tf.n_tf);
+  *batch = takes_deep(n, items, tf.lut_size) ? 0 : pick_batch(tile_batch);
+  return VEG_OK;
 }
 
 extern "C" veg_status veg_composite_bwd_workspace_size(int64_t n, int32_t n_views,

@@ -1200,12 +1200,21 @@ veg_status launch_bwd(const CompArgs& A, int n_views, const float4* out, const i
   return launch_status();
 }
 
-// The launches that take composite_fwd_deep_kernel: fewer work items than
-// kDeepItems.  Forward with it against one warp per block, by (tile, table)
-// items: 64 items 52 against 107 us (20k Gaussians), 1024 items 100 and 148,
-// 1105 items (five views) 144 and 232, 2500 items 128 and 144; 3072 items 182
-// and 152 (100k), 544 and 559 (1M), 3690 items 226 and 196.
-constexpr int64_t kDeepItems = 2048;
+// The launches that take composite_fwd_deep_kernel.  Its time per (tile, table)
+// item is mostly fixed (four CTAs that each read a table and stage a list), the
+// other kernel's is its longest lists until the SMs are full, so the line
+// rises with the lists' length, for which the records stand: forward with
+// it against without, L = 256, 500 records at 576 items 18 and 18 us, 1024 24
+// and 17; 5,000 at 1024 38 and 47, 1296 46 and 47, 1600 56 and 46; 100,000 at
+// 1296 68 and 82, 1600 80 and 81, 2025 96 and 75; 400,000 at 1600 103 and 111,
+// 2025 121 and 104; 1,500,000 at 1764 165 and 178, 2025 178 and 174.  It falls
+// as tables take CTAs from the SMs (four at 256 entries, two at 2048) and
+// time: 100,000 records, 1024 items 72 and 81 us at 1024 entries, 108 and 67 at
+// 2048; 256 items 48 and 76 at 2048, 50 and 85 at 4096.
+bool takes_deep(int64_t n, int64_t items, int lut_size) {
+  const int64_t line = n < 4096 ? 640 : n < 65536 ? 1280 : 1536;
+  return items * (lut_size + 768) < line * 1024;
+}
 
 template <bool LIT>
 veg_status launch_fwd_deep(const CompArgs& A, int n_views, float4* out, int32_t* nc,
@@ -1225,11 +1234,10 @@ veg_status launch_fwd_deep(const CompArgs& A, int n_views, float4* out, int32_t*
 // Dispatch over the tile batch (the instrumented build uses 256: the pair
 // counts do not depend on the batch).
 template <bool LIT>
-veg_status fwd_batch(int B, const CompArgs& A, int n_views, float4* out, int32_t* nc,
+veg_status fwd_batch(int B, const CompArgs& A, int n_views, int64_t n, float4* out, int32_t* nc,
                      cudaStream_t stream) {
   const dim3 items = comp_grid(A, n_views);
-  if ((int64_t)items.x * items.z < kDeepItems &&
-      sizeof(DeepSmem<LIT>) + (size_t)A.lut_size * 16 <= 100 * 1024)
+  if (takes_deep(n, (int64_t)items.x * items.z, A.lut_size))
     return launch_fwd_deep<LIT>(A, n_views, out, nc, stream);
   if (B == 128) return launch_fwd<128, false, LIT>(A, n_views, out, nc, nullptr, stream);
   if (B == 512) return launch_fwd<512, false, LIT>(A, n_views, out, nc, nullptr, stream);
