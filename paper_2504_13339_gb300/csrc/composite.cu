@@ -81,7 +81,7 @@ extern "C" veg_status veg_composite_fwd_batch(const veg_camera* cams, int32_t n_
   if (!batch || n < 0 || tf.lut_size < 2 || tf.n_tf < 1 || tf.n_tf > 4096 || !batch_ok(tile_batch))
     return VEG_ERR_INVALID_ARGUMENT;
   const int64_t items = total_tiles_of(cams, n_views) * (tf.view_tf ? 1 : tf.n_tf);
-  *batch = takes_deep(n, items, tf.lut_size) ? 0 : pick_batch(tile_batch);
+  *batch = takes_deep(n, items) ? 0 : pick_batch(tile_batch);
   return VEG_OK;
 }
 

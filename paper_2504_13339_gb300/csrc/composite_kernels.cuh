@@ -8,7 +8,7 @@
 // chosen by the caller or its autotuner) through shared memory; the
 // backward's warps each stage the chunks of 32 that they walk.  The stager
 // evaluates a splat's colour and opacity under the table (linear
-// interpolation, the table in shared memory), the exponent below which it
+// interpolation, the table read through the L1 cache), the exponent below which it
 // cannot reach alpha = 1/255, and which warp blocks its visible ellipse can
 // touch; each warp walks only the splats that touch its block, so pairs that
 // provably cannot blend cost nothing.  A pixel leaves once it has terminated
@@ -255,9 +255,9 @@ struct WorkItem {
   float tx0, ty0;       // the tile's first pixel
   long long image;      // first pixel of the output image
   int2 rg;              // the tile's list
+  const float4* lut;    // the table, or null
 };
-__device__ __forceinline__ WorkItem work_item(const CompArgs& A, float4* s_lut, int item,
-                                              int block) {
+__device__ __forceinline__ WorkItem work_item(const CompArgs& A, int item, int block) {
   WorkItem w;
   const int wi = A.order ? A.order[item] : item;  // global tile id
   const int view = view_of_tile(A.vm, wi), tile = wi - A.vm.tile_off[view];
@@ -269,12 +269,11 @@ __device__ __forceinline__ WorkItem work_item(const CompArgs& A, float4* s_lut, 
   pixel_of(tile, tiles_x, block, w.px, w.py);
   w.tx0 = (float)((tile % tiles_x) * VEG_TILE);
   w.ty0 = (float)((tile / tiles_x) * VEG_TILE);
-  // the table into shared memory; an index outside [0, n_tf) reads as fully
-  // transparent
+  // an index outside [0, n_tf) reads as fully transparent: no table, an empty list
   const int ti = A.view_tf ? A.view_tf[view] : t;
   const bool ok = ti >= 0 && ti < A.n_tf;
-  for (int e = threadIdx.x; e < A.lut_size; e += blockDim.x)
-    s_lut[e] = ok ? __ldg(&A.lut[(int64_t)ti * A.lut_size + e]) : make_float4(0.f, 0.f, 0.f, 0.f);
+  if (!ok) w.rg = make_int2(0, 0);
+  w.lut = ok ? A.lut + (int64_t)ti * A.lut_size : nullptr;
   return w;
 }
 
@@ -307,7 +306,11 @@ __device__ __forceinline__ void fetch_record(const CompArgs& A, RawSlot s, uint3
 }
 
 // A record's colour and opacity under the item's table: lo and hi are the
-// table entries around its scalar, aw = A w.
+// table entries around its scalar, aw = A w.  The entries come through the L1
+// cache: a copy of the table in shared memory costs each item its time and the
+// SMs their CTAs (1M-Gaussian scene under four tables, forward and backward:
+// 525 and 1086 us at 256 entries, 528 and 1105 at 4096; with the copy 563 and
+// 1125, 1158 and 1958).
 struct SplatTf {
   float4 lo, hi;
   TfPos q;
@@ -316,8 +319,8 @@ struct SplatTf {
 __device__ __forceinline__ SplatTf splat_tf(const float4* lut, int L, float v, float w) {
   SplatTf s;
   s.q = tf_pos(v, L);
-  s.lo = lut[s.q.k];
-  s.hi = lut[s.q.k + 1];
+  s.lo = __ldg(lut + s.q.k);
+  s.hi = __ldg(lut + s.q.k + 1);
   s.aw = mul(lerp_rn(s.lo.w, s.hi.w, s.q), w);
   return s;
 }
@@ -429,15 +432,14 @@ __global__ void __launch_bounds__(kCompThreads, 7)
   float4* s_col = s_geo + P;  // [P]: r, g, b, cutoff
   Prefetch<B, LIT> pre;
   pre.raw = s_col + P;        // [2][B]
-  float4* s_lut = pre.raw + 2 * B;                                 // [L]
-  float2* s_ca = reinterpret_cast<float2*>(s_lut + A.lut_size);    // [P]: -c/2, A w
-  pre.raw_sh = s_ca + P;                                           // [B] (LIT)
+  float2* s_ca = reinterpret_cast<float2*>(pre.raw + 2 * B);  // [P]: -c/2, A w
+  pre.raw_sh = s_ca + P;                                      // [B] (LIT)
   ListEntry* s_list = reinterpret_cast<ListEntry*>(pre.raw_sh + (LIT ? B : 0));  // [kWarps][B + 4]
   unsigned char* s_mask = reinterpret_cast<unsigned char*>(s_list + kWarps * (B + 4));  // [B]
   const int warp = threadIdx.x >> 5;
   ListEntry* my_list = s_list + warp * (B + 4);
   unsigned long long n_vis = 0, n_it = 0, n_eval = 0, n_blend = 0;
-  const WorkItem W = work_item(A, s_lut, (int)blockIdx.x, (int)(threadIdx.x >> 5));
+  const WorkItem W = work_item(A, (int)blockIdx.x, (int)(threadIdx.x >> 5));
   if (threadIdx.x == 0) {  // the padding slot: A w = 0 never blends
     s_geo[B] = s_col[B] = make_float4(0.f, 0.f, 0.f, 0.f);
     s_ca[B] = make_float2(0.f, 0.f);
@@ -465,7 +467,7 @@ __global__ void __launch_bounds__(kCompThreads, 7)
       const int sl = pre.slot(r);
       if (sl < cnt)
         stage_splat<B, LIT>(pre.raw[sl], pre.raw[B + sl],
-                            LIT ? pre.raw_sh[sl] : make_float2(1.f, 0.f), sl, s_lut, A.lut_size,
+                            LIT ? pre.raw_sh[sl] : make_float2(1.f, 0.f), sl, W.lut, A.lut_size,
                             W.tx0, W.ty0, s_geo, s_ca, s_col, s_mask);
       else
         s_mask[sl] = 0;
@@ -633,10 +635,9 @@ __global__ void __launch_bounds__(kDeepThreads, 4)
   pdl_enter();
   extern __shared__ float4 smem[];
   DeepSmem<LIT>& S = *reinterpret_cast<DeepSmem<LIT>*>(smem);
-  float4* s_lut = reinterpret_cast<float4*>(&S + 1);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int block = (int)blockIdx.x & 3;
-  const WorkItem W = work_item(A, s_lut, (int)blockIdx.x >> 2, block);
+  const WorkItem W = work_item(A, (int)blockIdx.x >> 2, block);
   const int n = W.rg.y - W.rg.x;
   const int chunks = (n + 31) / 32;
 
@@ -718,7 +719,7 @@ __global__ void __launch_bounds__(kDeepThreads, 4)
   if (at < n) fetch_record<LIT>(A, raw(0), __ldg(&list[at]));
   async_commit();
   if (at + kStride < n) next = __ldg(&list[at + kStride]);
-  __syncthreads();  // the table, the consumers' marks
+  __syncthreads();  // the consumers' marks
   int side = 0;
   for (int c = me; c < chunks; c += kProducers, at += kStride, side ^= 1) {
     async_wait();
@@ -729,7 +730,7 @@ __global__ void __launch_bounds__(kDeepThreads, 4)
     if (at < n) {
       ge = P.raw[side][lane];
       au = P.raw[side][32 + lane];
-      tf = splat_tf(s_lut, A.lut_size, au.w, ge.w);
+      tf = splat_tf(W.lut, A.lut_size, au.w, ge.w);
       cut = power_cutoff(tf.aw);
       hit = block_hit(ge.x - bx0, ge.y - by0, Reach(au.x, au.y, au.z, cut));
     }
@@ -877,9 +878,8 @@ __global__ void __launch_bounds__(kCompThreads, LIT || STATS ? 4 : 5)
   extern __shared__ float4 smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   Warp& S = reinterpret_cast<Warp*>(smem)[warp];
-  float4* s_lut = reinterpret_cast<float4*>(reinterpret_cast<Warp*>(smem) + kWarps);
-  float2* s_sh = reinterpret_cast<float2*>(s_lut + A.lut_size) + threadIdx.x;
-  const WorkItem W = work_item(A, s_lut, (int)blockIdx.x, (int)(threadIdx.x >> 5));
+  float2* s_sh = reinterpret_cast<float2*>(reinterpret_cast<Warp*>(smem) + kWarps) + threadIdx.x;
+  const WorkItem W = work_item(A, (int)blockIdx.x, (int)(threadIdx.x >> 5));
   const float bx0 = W.tx0 + (float)((warp & 1) * 8), by0 = W.ty0 + (float)((warp >> 1) * 8);
   const float2 fx = dup((float)W.px), fy = make_float2((float)W.py, (float)(W.py + 4));
 
@@ -892,7 +892,7 @@ __global__ void __launch_bounds__(kCompThreads, LIT || STATS ? 4 : 5)
     ov[i] = make_float4(0.f, 0.f, 0.f, 1.f);
     dv4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     nc[i] = 0;
-    if (W.px < W.width && W.py + 4 * i < W.height) {
+    if (W.lut && W.px < W.width && W.py + 4 * i < W.height) {
       const int64_t o = W.image + (int64_t)(W.py + 4 * i) * W.width + W.px;
       ov[i] = out[o];
       dv4[i] = dout[o];
@@ -925,7 +925,6 @@ __global__ void __launch_bounds__(kCompThreads, LIT || STATS ? 4 : 5)
   }
   async_commit();
   if (wmax - 33 - lane >= 0) next = __ldg(&list[wmax - 33 - lane]);
-  __syncthreads();  // the table
   for (int end = wmax; end > 0; end -= 32, side ^= 1) {
     // stage this chunk: each lane tests its record against the warp's block,
     // the hits are compacted, last one first
@@ -939,7 +938,7 @@ __global__ void __launch_bounds__(kCompThreads, LIT || STATS ? 4 : 5)
     if (pos >= 0) {
       ge = S.raw[side][lane];
       au = S.raw[side][32 + lane];
-      tf = splat_tf(s_lut, A.lut_size, au.w, ge.w);
+      tf = splat_tf(W.lut, A.lut_size, au.w, ge.w);
       cut = power_cutoff(tf.aw);
       hit = block_hit(ge.x - bx0, ge.y - by0, Reach(au.x, au.y, au.z, cut));
     }
@@ -1128,15 +1127,15 @@ __global__ void __launch_bounds__(kCompThreads, LIT || STATS ? 4 : 5)
 }
 
 // Dynamic shared memory of a CTA.  Forward: the padded splat arrays, the
-// records on their way, the table, warp lists and masks; backward: its
-// warps' splats, the table, the shading factors on their way.
-size_t fwd_smem_bytes(int L, bool lit, int B) {
+// records on their way, warp lists and masks; backward: its warps' splats, the
+// shading factors on their way.
+size_t fwd_smem_bytes(bool lit, int B) {
   const size_t P = B + 1;
-  return P * (16 + 16 + 8) + (size_t)2 * B * 16 + (size_t)L * 16 + (lit ? (size_t)B * 8 : 0) +
+  return P * (16 + 16 + 8) + (size_t)2 * B * 16 + (lit ? (size_t)B * 8 : 0) +
          (size_t)kWarps * (B + 4) * sizeof(ListEntry) + (size_t)B;
 }
-size_t bwd_smem_bytes(int L, bool lit) {
-  return kWarps * (lit ? sizeof(BwdWarp<true>) : sizeof(BwdWarp<false>)) + (size_t)L * 16 +
+size_t bwd_smem_bytes(bool lit) {
+  return kWarps * (lit ? sizeof(BwdWarp<true>) : sizeof(BwdWarp<false>)) +
          (lit ? (size_t)kCompThreads * 8 : 0);
 }
 
@@ -1175,10 +1174,10 @@ inline dim3 comp_grid(const CompArgs& A, int n_views) {
 template <int B, bool STATS, bool LIT>
 veg_status launch_fwd(const CompArgs& A, int n_views, float4* out, int32_t* nc,
                       unsigned long long* stats, cudaStream_t stream) {
-  const size_t smem = fwd_smem_bytes(A.lut_size, LIT, B);
+  const size_t smem = fwd_smem_bytes(LIT, B);
   auto kern = composite_fwd_kernel<B, STATS, LIT>;
   static SmemRecord configured;
-  veg_status st = prepare_smem(kern, smem, configured, true);
+  veg_status st = prepare_smem(kern, smem, configured, false);
   if (st != VEG_OK) return st;
   launch_k(kern, comp_grid(A, n_views), kCompThreads, smem, stream, A, out, nc, stats);
   count_launch();
@@ -1189,10 +1188,10 @@ template <bool STATS, bool LIT>
 veg_status launch_bwd(const CompArgs& A, int n_views, const float4* out, const int32_t* nc,
                       const float4* dout, float4* grad2d, float2* grad_shade,
                       unsigned long long* stats, cudaStream_t stream) {
-  const size_t smem = bwd_smem_bytes(A.lut_size, LIT);
+  const size_t smem = bwd_smem_bytes(LIT);
   auto kern = composite_bwd_kernel<STATS, LIT>;
   static SmemRecord configured;
-  veg_status st = prepare_smem(kern, smem, configured, true);
+  veg_status st = prepare_smem(kern, smem, configured, false);
   if (st != VEG_OK) return st;
   launch_k(kern, comp_grid(A, n_views), kCompThreads, smem, stream, A, out, nc, dout, grad2d,
            grad_shade, stats);
@@ -1201,28 +1200,24 @@ veg_status launch_bwd(const CompArgs& A, int n_views, const float4* out, const i
 }
 
 // The launches that take composite_fwd_deep_kernel.  Its time per (tile, table)
-// item is mostly fixed (four CTAs that each read a table and stage a list), the
-// other kernel's is its longest lists until the SMs are full, so the line
-// rises with the lists' length, for which the records stand: forward with
-// it against without, L = 256, 500 records at 576 items 18 and 18 us, 1024 24
-// and 17; 5,000 at 1024 38 and 47, 1296 46 and 47, 1600 56 and 46; 100,000 at
-// 1296 68 and 82, 1600 80 and 81, 2025 96 and 75; 400,000 at 1600 103 and 111,
-// 2025 121 and 104; 1,500,000 at 1764 165 and 178, 2025 178 and 174.  It falls
-// as tables take CTAs from the SMs (four at 256 entries, two at 2048) and
-// time: 100,000 records, 1024 items 72 and 81 us at 1024 entries, 108 and 67 at
-// 2048; 256 items 48 and 76 at 2048, 50 and 85 at 4096.
-bool takes_deep(int64_t n, int64_t items, int lut_size) {
-  const int64_t line = n < 4096 ? 640 : n < 65536 ? 1280 : 1536;
-  return items * (lut_size + 768) < line * 1024;
+// item is mostly fixed (four CTAs that each stage a list), the other kernel's
+// is its longest lists until the SMs are full, so the line rises with the
+// lists' length, for which the records stand: forward with it against without,
+// 500 records at 576 items 15 and 17 us, 784 18 and 17, 1024 23 and 17; 5,000 at
+// 1024 36 and 45, 1296 44 and 46, 1600 53 and 46; 100,000 at 1296 65 and 80, 1600
+// 76 and 78, 2025 91 and 72; 400,000 at 1600 100 and 109, 2025 116 and 102;
+// 1,500,000 at 1764 162 and 177, 2025 171 and 171.
+bool takes_deep(int64_t n, int64_t items) {
+  return items < (n < 4096 ? 640 : n < 65536 ? 1280 : 1536);
 }
 
 template <bool LIT>
 veg_status launch_fwd_deep(const CompArgs& A, int n_views, float4* out, int32_t* nc,
                            cudaStream_t stream) {
-  const size_t smem = sizeof(DeepSmem<LIT>) + (size_t)A.lut_size * 16;
+  const size_t smem = sizeof(DeepSmem<LIT>);
   auto kern = composite_fwd_deep_kernel<LIT>;
   static SmemRecord configured;
-  veg_status st = prepare_smem(kern, smem, configured, true);
+  veg_status st = prepare_smem(kern, smem, configured, false);
   if (st != VEG_OK) return st;
   dim3 grid = comp_grid(A, n_views);
   grid.x *= 4;
@@ -1237,7 +1232,7 @@ template <bool LIT>
 veg_status fwd_batch(int B, const CompArgs& A, int n_views, int64_t n, float4* out, int32_t* nc,
                      cudaStream_t stream) {
   const dim3 items = comp_grid(A, n_views);
-  if (takes_deep(n, (int64_t)items.x * items.z, A.lut_size))
+  if (takes_deep(n, (int64_t)items.x * items.z))
     return launch_fwd_deep<LIT>(A, n_views, out, nc, stream);
   if (B == 128) return launch_fwd<128, false, LIT>(A, n_views, out, nc, nullptr, stream);
   if (B == 512) return launch_fwd<512, false, LIT>(A, n_views, out, nc, nullptr, stream);

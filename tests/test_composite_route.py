@@ -1,5 +1,5 @@
 """Which forward kernel a launch takes, asked of the library on the host: both
-sides of the lines by records and by table size."""
+sides of the lines by records."""
 import os
 import shutil
 
@@ -22,10 +22,6 @@ def cams(tiles):
     return c
 
 
-def batch(n, items, L=256, asked=0):
-    return _lib.veg_composite_fwd_batch(cams(items), n, _lib.veg_tf(0, L, 1), asked)
-
-
 @pytest.mark.parametrize("n,line", [(0, 640), (4095, 640), (4096, 1280), (65535, 1280),
                                     (65536, 1536), (10_000_000, 1536)])
 def test_few_items_stage_no_batches(n, line):
@@ -34,11 +30,6 @@ def test_few_items_stage_no_batches(n, line):
         ask = lambda tiles, b: _lib.veg_composite_fwd_batch(cams(tiles), n, tf, b)
         assert ask(line // tables - 1, 128) == 0
         assert [ask(line // tables, b) for b in (0, 128, 512)] == [256, 128, 512]
-
-
-@pytest.mark.parametrize("L,items", [(1024, 731), (2048, 465), (4096, 269)])
-def test_the_line_falls_with_the_table(L, items):
-    assert batch(10_000, items, L) == 0 and batch(10_000, items + 1, L) == 256
 
 
 def test_a_table_per_view_is_one_item_per_tile():

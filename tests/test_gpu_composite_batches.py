@@ -88,6 +88,31 @@ def test_needles_and_extreme_widths(aspect):
 
 @pytest.mark.parametrize("L", [2, 1024, 2048, 4096])
 def test_table_sizes(L):
-    """Both kernels over the tables' range (their shared memory grows with it)."""
+    """Both kernels over the tables' range."""
     g = S.uniform_gaussians(3000, 79, logscale_mean=-2.5)
     check(g, S.orbit_cameras(2, 6, 60, 40), S.bump_tfs(1, 44, size=L), L == 2048)
+
+
+def test_a_table_index_out_of_range_has_no_gradient():
+    """Such a view reads as transparent in the backward too, also after a forward
+    that saw a valid index."""
+    g = S.uniform_gaussians(500, 80, logscale_mean=-2.5)
+    cams = S.orbit_cameras(2, 6, 60, 40)
+    tens = (dev(g.mean_v), dev(g.logscale_w), dev(g.quat))
+    luts = lut_tensor(S.bump_tfs(2, 45))
+    p = SplatPipeline(g.n, cams, n_tf=1)
+    p.project(*tens)
+    p.bin_sort()
+    dout = torch.randn_like(p.out)
+    got = []
+    for view_tf in ([1, 0], [1, 5]):
+        vt = torch.tensor(view_tf, dtype=torch.int32, device="cuda")
+        if not got:
+            _lib.veg_composite_fwd(p.c_cams, p.n, p.geo, p.aux, p.vals, p.ranges,
+                                   _lib.tf_desc(luts, vt), (0.0, 0.0, 0.0), 0, p.out, p.n_contrib)
+        _lib.veg_composite_bwd(p.c_cams, p._g, p.geo, p.aux, p.tiles, p.vals, p.ranges,
+                               _lib.tf_desc(luts, vt), (0.0, 0.0, 0.0), 0, p.out, p.n_contrib,
+                               dout, None, None, None, None, p.grad2d)
+        got.append(p.grad2d.view(2, -1).clone())
+    assert (got[0] != 0).any(1).all() and torch.allclose(got[0][0], got[1][0], rtol=1e-4, atol=1e-6)
+    assert (got[1][1] == 0).all()
