@@ -92,48 +92,66 @@ __global__ void __launch_bounds__(256)
 // and sets the bit when any of them has a positive opacity (interpolating
 // two non-positive entries gives a clamped opacity of 0).  A NaN vertex, or
 // more than 32 tables, sets every bit.
-// One warp per macrocell, lanes over its vertices (x fastest, so that
-// neighbouring lanes read neighbouring vertices), then over the tables: the
-// kernel reads every sector of the volume once: 85 us at 256^3 (268 MB), where a
-// thread per macrocell took 515.
+// G lanes per macrocell, over its vertices (x fastest, so that neighbouring
+// lanes read neighbouring vertices), then over the tables: a lane each where
+// macrocells are small and many, a warp where they are large, eight lanes
+// between.  256^3 vertices (268 MB) under two tables, 1, 8 and 32 lanes: single
+// cells 234, 1394 and 4726 us, 4^3 cells 68, 117 and 158, 8^3 101, 66 and 73, 16^3
+// 621, 157 and 90; 64^3 vertices in 4^3 cells (4096 macrocells) 14, 8 and 8.
+template <int G>
 __global__ void __launch_bounds__(256)
     cell_mask_kernel(const float4* __restrict__ vol, int R, int cell, int cells,
                      const float4* __restrict__ lut, int L, int n_tf, uint32_t* __restrict__ mask) {
   pdl_enter();
-  const int lane = threadIdx.x & 31;
-  const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & (G - 1);
+  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
   const int64_t nc = (int64_t)cells * cells * cells;
-  if (i >= nc) return;  // warp-uniform
-  const int cx = (int)(i % cells), cy = (int)((i / cells) % cells), cz = (int)(i / ((int64_t)cells * cells));
+  if (i >= nc) return;  // uniform over a macrocell's lanes
+  const unsigned mine = G == 32 ? 0xffffffffu
+                                : ((1u << (G & 31)) - 1u) << (threadIdx.x & 31 & ~(G - 1));
+  const int cx = (int)(i % cells), cy = (int)((i / cells) % cells),
+            cz = (int)(i / ((int64_t)cells * cells));
   const int x0 = cx * cell, y0 = cy * cell, z0 = cz * cell;
-  const int nx = min(x0 + cell, R - 1) - x0 + 1, ny = min(y0 + cell, R - 1) - y0 + 1,
-            nz = min(z0 + cell, R - 1) - z0 + 1;
+  const int x1 = min(x0 + cell, R - 1), y1 = min(y0 + cell, R - 1), z1 = min(z0 + cell, R - 1);
   float mn = 3.0e38f, mx = -3.0e38f;
   bool nan = false;
-  const int nv = nx * ny * nz;
-#pragma unroll 8
-  for (int e = lane; e < nv; e += 32) {
-    const int row = e / nx, x = e - row * nx, z = row / ny, y = row - z * ny;
-    const float v = __ldg(&vol[((int64_t)(z0 + z) * R + y0 + y) * R + x0 + x].x);
+  auto see = [&](float v) {
     nan |= v != v;
     mn = fminf(mn, v);
     mx = fmaxf(mx, v);
-  }
-  nan = __any_sync(0xffffffffu, nan);
+  };
+  if (G == 1) {
+    for (int z = z0; z <= z1; ++z)
+      for (int y = y0; y <= y1; ++y)
+        for (int x = x0; x <= x1; ++x) see(__ldg(&vol[((int64_t)z * R + y) * R + x]).x);
+  } else {
+    const int nx = x1 - x0 + 1, ny = y1 - y0 + 1, nv = nx * ny * (z1 - z0 + 1);
+#pragma unroll 8
+    for (int e = lane; e < nv; e += G) {
+      const int row = e / nx, x = e - row * nx, z = row / ny, y = row - z * ny;
+      see(__ldg(&vol[((int64_t)(z0 + z) * R + y0 + y) * R + x0 + x].x));
+    }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    for (int o = G / 2; o > 0; o >>= 1) {
+      nan |= __shfl_xor_sync(mine, (int)nan, o) != 0;
+      mn = fminf(mn, __shfl_xor_sync(mine, mn, o));
+      mx = fmaxf(mx, __shfl_xor_sync(mine, mx, o));
+    }
   }
   uint32_t m = 0xffffffffu;
   if (!nan && n_tf <= 32) {
     const float lo = fminf(fmaxf(mn - 1e-6f, 0.0f), 1.0f) * (float)(L - 1);
     const float hi = fminf(fmaxf(mx + 1e-6f, 0.0f), 1.0f) * (float)(L - 1);
     const int k0 = max((int)floorf(lo) - 1, 0), k1 = min((int)floorf(hi) + 2, L - 1);
-    bool any = false;
-    if (lane < n_tf)
-      for (int k = k0; k <= k1 && !any; ++k) any = __ldg(&lut[(int64_t)lane * L + k].w) > 0.0f;
-    m = __ballot_sync(0xffffffffu, any);
+    m = 0u;
+    for (int t = G == 1 ? 0 : lane; t < n_tf; t += G)
+      for (int k = k0; k <= k1; ++k)
+        if (__ldg(&lut[(int64_t)t * L + k].w) > 0.0f) {
+          m |= 1u << t;
+          break;
+        }
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) m |= __shfl_xor_sync(mine, m, o);
   }
   if (lane == 0) mask[i] = m;
 }
@@ -432,9 +450,13 @@ extern "C" veg_status veg_raymarch_cells(const float* vol4, int32_t resolution, 
     return VEG_ERR_INVALID_ARGUMENT;
   const int c = cells_per_axis(resolution, cell);
   const int64_t nc = (int64_t)c * c * c;
-  launch_k(cell_mask_kernel, (unsigned)((nc + 7) / 8), 256, 0, stream, 
-      reinterpret_cast<const float4*>(vol4), resolution, cell, c,
-      reinterpret_cast<const float4*>(tf.lut), tf.lut_size, tf.n_tf, mask);
+  const int lanes = cell >= 8 ? 32 : nc >= 65536 ? 1 : 8;
+  auto kern = lanes == 1   ? cell_mask_kernel<1>
+              : lanes == 8 ? cell_mask_kernel<8>
+                           : cell_mask_kernel<32>;
+  launch_k(kern, (unsigned)((nc * lanes + 255) / 256), 256, 0, stream,
+           reinterpret_cast<const float4*>(vol4), resolution, cell, c,
+           reinterpret_cast<const float4*>(tf.lut), tf.lut_size, tf.n_tf, mask);
   count_launch();
   return launch_status();
 }

@@ -1,4 +1,5 @@
-"""The march at the edges of its inputs: distant eyes, shades without bound."""
+"""The march at the edges of its inputs: distant eyes, shades without bound, and
+the macrocells' masks from single cells to macrocells wider than the volume."""
 import math
 from dataclasses import replace
 
@@ -6,7 +7,8 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2504_13339_gb300 import scenes as S
+from paper_2504_13339_gb300 import _lib, scenes as S
+from paper_2504_13339_gb300.render import lut_tensor
 from test_gpu_raymarch import MAT, march, prepared
 from test_gpu_raymarch_groups import masked
 
@@ -58,3 +60,38 @@ def test_a_sample_shaded_to_infinity_reaches_the_image(beta, scale, colour):
     out = march([cam], prepared(vol), luts, 1.0 / (R - 1), (0.3, 0.6, 0.25, beta))
     assert np.isnan(out[0, 1]).any()
     assert np.array_equal(out[0, 0], out[0, 1], equal_nan=True)
+
+
+# 65536 macrocells and more take a lane each up to cells of four, fewer eight
+# lanes; cells of eight and more a warp
+@pytest.mark.parametrize("R,cell", [(42, 1), (20, 1), (84, 2), (31, 2), (163, 4), (30, 4), (60, 8),
+                                    (33, 16), (21, 64)])
+@pytest.mark.parametrize("n_tf", [1, 9, 32, 33])
+def test_masks(R, cell, n_tf):
+    rng = np.random.default_rng(R + n_tf)
+    vol = rng.uniform(-0.2, 1.2, (R, R, R)).astype(np.float32) ** 3
+    vol[rng.integers(0, R, 3), 0, 1] = np.nan
+    vol[1, rng.integers(0, R, 3), 2] = np.inf
+    vol[2, 1, rng.integers(0, R, 3)] = -np.inf
+    L = 64
+    op = np.where(rng.random((n_tf, L)) < 0.06, 0.5, -0.1).astype(np.float32)
+    luts = np.zeros((n_tf, L, 4), np.float32)
+    luts[..., 3] = op
+    v4 = prepared(vol)
+    got = torch.empty(_lib.veg_raymarch_cells_count(R, cell), dtype=torch.int32, device="cuda")
+    _lib.veg_raymarch_cells(v4, _lib.tf_desc(lut_tensor(luts)), cell, got)
+    at = [slice(c, min(c + cell, R - 1) + 1) for c in range(0, R - 1, cell)]
+    lo, hi = (np.stack([np.stack([np.stack([f(vol[z, y, x]) for x in at]) for y in at]) for z in at])
+              for f in (np.min, np.max))  # a NaN vertex makes both NaN
+    nan = np.isnan(lo)
+    one = np.float32(1e-6)
+    with np.errstate(invalid="ignore"):
+        k0 = np.floor(np.clip(np.nan_to_num(lo) - one, 0, 1) * np.float32(L - 1)).astype(int) - 1
+        k1 = np.floor(np.clip(np.nan_to_num(hi) + one, 0, 1) * np.float32(L - 1)).astype(int) + 2
+    k0, k1 = np.maximum(k0, 0), np.minimum(k1, L - 1)
+    seen = np.concatenate([np.zeros((n_tf, 1), int), np.cumsum(op > 0, 1)], 1)
+    want = np.zeros(lo.shape, np.uint32)
+    for t in range(min(n_tf, 32)):
+        want |= (seen[t][k1 + 1] > seen[t][k0]).astype(np.uint32) << np.uint32(t)
+    want[nan | (n_tf > 32)] = 0xffffffff
+    assert np.array_equal(got.cpu().numpy().view(np.uint32).reshape(want.shape), want)
