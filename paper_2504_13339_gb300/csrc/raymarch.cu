@@ -285,20 +285,19 @@ __global__ void __launch_bounds__(256, 3)
     ray.step = A.step;
     ray.inv_h = A.inv_h;
     ray.R = R;
-    float rate[3];
-    march_rates(ray, rate);
+    const MarchStep over = march_step(ray, n, A.cell_shift);
     for (int k = 0; live; ++k) {
       float g[3];
       int ic[3];
       // the next sample that a table still compositing can see
       for (; k < n;) {
-        const float t = march_place(ray, k, g, ic);
+        march_place(ray, k, g, ic);
         if (!skip_empty) break;
         const int m[3] = {ic[0] >> A.cell_shift, ic[1] >> A.cell_shift, ic[2] >> A.cell_shift};
         if (((__ldg(&A.cell_mask[march_macrocell(m, A.cells)]) >> lut0) & live) != 0u) break;
         // Every table still compositing has zero opacity in this macrocell:
         // its samples would leave colour and transmittance unchanged.
-        const int next = march_next(ray, k, n, t, g, m, A.cell_shift, rate);
+        const int next = march_next(ray, over, k, n, g, m, A.cell_shift);
         if (STATS) n_skip += (unsigned)(next - k);
         k = next;
       }

@@ -22,14 +22,14 @@ extern "C" void walk(const float* eye, const float* d, float ta, float tb, float
   MarchRay r;
   for (int c = 0; c < 3; ++c) r.eye[c] = eye[c], r.d[c] = d[c];
   r.ta = ta, r.step = step, r.inv_h = inv_h, r.R = R;
-  float rate[3], g[3], q[3];
+  float g[3], q[3];
   int ic[3], jc[3];
-  march_rates(r, rate);
   const int n = (int)floorf((tb - ta) / step);
+  const MarchStep over = march_step(r, n, shift);
   for (int k = 0; k < n; ++*steps) {
-    const float t = march_place(r, k, g, ic);
+    march_place(r, k, g, ic);
     const int m[3] = {ic[0] >> shift, ic[1] >> shift, ic[2] >> shift};
-    const int next = march_next(r, k, n, t, g, m, shift, rate);
+    const int next = march_next(r, over, k, n, g, m, shift);
     for (int j = k + 1; j < next; ++j) {
       march_place(r, j, q, jc);
       for (int c = 0; c < 3; ++c)
