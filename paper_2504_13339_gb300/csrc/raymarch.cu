@@ -57,7 +57,6 @@ struct MarchArgs {
   int group;  // tables per group
   const int32_t* view_tf;
   int width, height, tiles_x, tiles_per_view;
-  bool shade;
   float ka, kd, ks, beta;
   bool leave_out;  // tables without opacity (every factor of them is finite)
   float bg0, bg1, bg2;
@@ -180,12 +179,15 @@ __device__ __forceinline__ Sample load_sample(const float4* p) {
 // held the kernel at two CTAs per SM, and every table was a branch of every
 // sample.  Ten opacity maps over a 256^3 volume, three 800x800 views (with the macrocells' masks): 6300 us
 // in groups of eight with every sample visited and every table evaluated,
-// 4330 with the steps, bits and registers, 3440 so.
+// 4330 with the steps, bits and registers, 3430 so.  Without a material
+// (SHADE false) only the value is read and blended: ten tables over 64^3
+// vertices, one 400x300 view, 357 us (371 in the groups of eight, 409 with the
+// whole blend), one table 99 (194).
 //
 // stats (instrumented build): samples taken (per ray and table group),
 // table evaluations (samples x live tables) and, with a cell mask, samples
 // skipped as empty.
-template <bool MANY, bool STATS>
+template <bool MANY, bool STATS, bool SHADE>
 __global__ void __launch_bounds__(256, 3)
     raymarch_kernel(MarchArgs A, const __grid_constant__ RaySet rs, float4* __restrict__ out,
                     unsigned long long* __restrict__ stats) {
@@ -306,30 +308,28 @@ __global__ void __launch_bounds__(256, 3)
       for (int c = 0; c < 3; ++c) g[c] -= (float)ic[c];
       const float4* base = A.vol + ((int64_t)ic[2] * R + ic[1]) * R + ic[0];
       const int64_t sy = R, sz = (int64_t)R * R;
-      const Sample c00 = lerp_sample(load_sample(base), load_sample(base + 1), g[0]);
-      const Sample c01 = lerp_sample(load_sample(base + sy), load_sample(base + sy + 1), g[0]);
-      const Sample c10 = lerp_sample(load_sample(base + sz), load_sample(base + sz + 1), g[0]);
-      const Sample c11 =
-          lerp_sample(load_sample(base + sz + sy), load_sample(base + sz + sy + 1), g[0]);
-      const Sample sm = lerp_sample(lerp_sample(c00, c01, g[1]), lerp_sample(c10, c11, g[1]), g[2]);
-      const float sx = sm.vx.y, sy_ = sm.yz.x, sz_ = sm.yz.y;
-      const TfPos q = tf_pos(sm.vx.x, L);
-      if (STATS) {
-        ++n_samp;
-        n_tab += (unsigned)__popc(live);
-      }
-      // the largest gradient component; a gradient that is not finite makes
-      // a NaN colour under any table, so no table is left out
-      const float m = fmaxf(fmaxf(fabsf(sx), fabsf(sy_)), fabsf(sz_));
-      const float chk = sx * 0.0f + sy_ * 0.0f + sz_ * 0.0f;
-      const unsigned on = A.leave_out && chk == 0.0f ? s_any[q.k] & live : live;
-      if (on == 0u) continue;
       float sd = 1.0f, ss = 0.0f;
-      if (A.shade) {
+      unsigned on;
+      TfPos q;
+      if (SHADE) {
+        const Sample c00 = lerp_sample(load_sample(base), load_sample(base + 1), g[0]);
+        const Sample c01 = lerp_sample(load_sample(base + sy), load_sample(base + sy + 1), g[0]);
+        const Sample c10 = lerp_sample(load_sample(base + sz), load_sample(base + sz + 1), g[0]);
+        const Sample c11 =
+            lerp_sample(load_sample(base + sz + sy), load_sample(base + sz + sy + 1), g[0]);
+        const Sample sm =
+            lerp_sample(lerp_sample(c00, c01, g[1]), lerp_sample(c10, c11, g[1]), g[2]);
+        const float sx = sm.vx.y, sy_ = sm.yz.x, sz_ = sm.yz.y;
+        q = tf_pos(sm.vx.x, L);
+        // the largest gradient component; a gradient that is not finite makes
+        // a NaN colour under any table, so no table is left out
+        const float m = fmaxf(fmaxf(fabsf(sx), fabsf(sy_)), fabsf(sz_));
+        const float chk = sx * 0.0f + sy_ * 0.0f + sz_ * 0.0f;
+        on = A.leave_out && chk == 0.0f ? s_any[q.k] & live : live;
         // normal = -gradient / |gradient|; scaled by the largest component
         // first so that tiny gradients cannot underflow
         sd = A.ka;
-        if (m > 0.0f) {
+        if (on != 0u && m > 0.0f) {
           const float gx = sx / m, gy = sy_ / m, gz = sz_ / m;
           const float ig = rsqrtf(gx * gx + gy * gy + gz * gz);
           const float nl = fabsf((gx * V.light[0] + gy * V.light[1] + gz * V.light[2]) * ig);
@@ -337,7 +337,22 @@ __global__ void __launch_bounds__(256, 3)
           sd = A.ka + A.kd * nl;
           ss = nl > 0.f ? A.ks * __powf(nh, A.beta) : 0.f;
         }
+      } else {  // the value alone
+        auto along = [&](const float4* p) {
+          const float a = __ldg(&p[0].x), b = __ldg(&p[1].x);
+          return fmaf(g[0], b - a, a);
+        };
+        const float c00 = along(base), c01 = along(base + sy), c10 = along(base + sz),
+                    c11 = along(base + sz + sy);
+        const float c0 = fmaf(g[1], c01 - c00, c00), c1 = fmaf(g[1], c11 - c10, c10);
+        q = tf_pos(fmaf(g[2], c1 - c0, c0), L);
+        on = s_any[q.k] & live;
       }
+      if (STATS) {
+        ++n_samp;
+        n_tab += (unsigned)__popc(live);
+      }
+      if (on == 0u) continue;
       // each lane its own next table: a step serves lanes at different ones
       for (unsigned left = on; left != 0u; left &= left - 1u) {
         const int tt = MANY ? __ffs((int)left) - 1 : 0;
@@ -384,26 +399,27 @@ __global__ void __launch_bounds__(256, 3)
 // shared memory each (three CTAs per SM hold 16).
 constexpr int kMarchTables = 16;
 
-template <bool MANY, bool STATS>
+template <bool MANY, bool STATS, bool SHADE>
 veg_status launch_march(const MarchArgs& A, const RaySet& rs, int n_views, float4* out,
                         unsigned long long* stats, cudaStream_t stream) {
   const size_t smem = (MANY ? (size_t)A.group * 256 * sizeof(float4) : 0) +
                       (size_t)A.lut_size * sizeof(unsigned);
+  auto kern = raymarch_kernel<MANY, STATS, SHADE>;
   static SmemRecord configured;  // default carveout: the volume samples want L1
-  veg_status st = prepare_smem(raymarch_kernel<MANY, STATS>, smem, configured, false);
+  veg_status st = prepare_smem(kern, smem, configured, false);
   if (st != VEG_OK) return st;
   const unsigned groups = A.view_tf ? 1u : (unsigned)((A.n_tf + A.group - 1) / A.group);
   dim3 grid((unsigned)(A.tiles_per_view * n_views), 1u, groups);
-  launch_k(raymarch_kernel<MANY, STATS>, grid, 256, smem, stream, A, rs, out, stats);
+  launch_k(kern, grid, 256, smem, stream, A, rs, out, stats);
   count_launch();
   return launch_status();
 }
 
-template <bool MANY>
+template <bool MANY, bool SHADE>
 veg_status launch_march_s(const MarchArgs& A, const RaySet& rs, int n_views, float4* out,
                           unsigned long long* stats, cudaStream_t stream) {
-  return stats ? launch_march<MANY, true>(A, rs, n_views, out, stats, stream)
-               : launch_march<MANY, false>(A, rs, n_views, out, nullptr, stream);
+  return stats ? launch_march<MANY, true, SHADE>(A, rs, n_views, out, stats, stream)
+               : launch_march<MANY, false, SHADE>(A, rs, n_views, out, nullptr, stream);
 }
 
 }  // namespace
@@ -492,7 +508,6 @@ extern "C" veg_status veg_raymarch_masked(const veg_camera* cams, int32_t n_view
   A.height = cams[0].height;
   A.tiles_x = tiles_x_of(A.width);
   A.tiles_per_view = A.tiles_x * tiles_x_of(A.height);
-  A.shade = material != nullptr;
   A.ka = material ? material->ka : 0.f;
   A.kd = material ? material->kd : 0.f;
   A.ks = material ? material->ks : 0.f;
@@ -527,8 +542,11 @@ extern "C" veg_status veg_raymarch_masked(const veg_camera* cams, int32_t n_view
   // tables per sample pass: the fewest equal groups
   const int all = tf.view_tf ? 1 : tf.n_tf, groups = (all + kMarchTables - 1) / kMarchTables;
   A.group = (all + groups - 1) / groups;
-  return A.group > 1 ? launch_march_s<true>(A, rs, n_views, o, stats, stream)
-                     : launch_march_s<false>(A, rs, n_views, o, stats, stream);
+  if (material)
+    return A.group > 1 ? launch_march_s<true, true>(A, rs, n_views, o, stats, stream)
+                       : launch_march_s<false, true>(A, rs, n_views, o, stats, stream);
+  return A.group > 1 ? launch_march_s<true, false>(A, rs, n_views, o, stats, stream)
+                     : launch_march_s<false, false>(A, rs, n_views, o, stats, stream);
 }
 
 extern "C" veg_status veg_raymarch(const veg_camera* cams, int32_t n_views, const float* vol4,
