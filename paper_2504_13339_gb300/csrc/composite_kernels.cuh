@@ -50,6 +50,7 @@ namespace {
 constexpr int kWarps = 4;
 constexpr int kCompThreads = 32 * kWarps;
 constexpr float kLog2e = 1.44269502162933349609375f;
+constexpr float kHuge = 3.0e38f;
 // Every per-splat shared array of the forward is indexed by the splat's batch
 // slot, which a thread loops over in steps of the block size; slot B is a
 // splat that no pixel blends (it pads the warp lists to whole steps of the
@@ -952,7 +953,8 @@ __global__ void __launch_bounds__(kCompThreads, LIT || STATS ? 4 : 5)
       const float r = lerp_rn(tf.lo.x, tf.hi.x, tf.q), g = lerp_rn(tf.lo.y, tf.hi.y, tf.q),
                   b = lerp_rn(tf.lo.z, tf.hi.z, tf.q);
       const float dr = slc * (tf.hi.x - tf.lo.x), dg = slc * (tf.hi.y - tf.lo.y),
-                  db = slc * (tf.hi.z - tf.lo.z), da = ge.w * sl * (tf.hi.w - tf.lo.w);
+                  db = slc * (tf.hi.z - tf.lo.z),
+                  da = fminf(fmaxf(ge.w * sl * (tf.hi.w - tf.lo.w), -kHuge), kHuge);
       const float4 cc = clean_conic(au);
       S.u[slot] = make_float4(ge.x, ge.x, ge.y, ge.y);
       S.q[slot] = make_float4(-0.5f * cc.x, -0.5f * cc.x, -cc.y, -cc.y);
@@ -1031,13 +1033,19 @@ __global__ void __launch_bounds__(kCompThreads, LIT || STATS ? 4 : 5)
           v[m * kSum + 5] = (ok[m][0] ? s.x : 0.0f) + (ok[m][1] ? s.y : 0.0f);
         }
         const float2 da = fma2(Ti, cgd, mul2(nSuf, rr));
-        // below the clamp alpha follows the exponent and the opacity slope
+        // below the clamp alpha follows the exponent and the opacity slope (the
+        // product is masked, not a factor: A w may be infinite)
         float2 mg = mul2(da, G[m]), cv = mul2(wgt, h);
-        mg.x = ok[m][0] && raw2[m].x <= kAlphaMax ? mg.x : 0.0f;
-        mg.y = ok[m][1] && raw2[m].y <= kAlphaMax ? mg.y : 0.0f;
+        const bool free[2] = {ok[m][0] && raw2[m].x <= kAlphaMax,
+                              ok[m][1] && raw2[m].y <= kAlphaMax};
+        float2 dp = mul2(hi2(c1[m]), mg);
+        dp.x = free[0] ? dp.x : 0.0f;
+        dp.y = free[1] ? dp.y : 0.0f;
+        mg.x = free[0] ? mg.x : 0.0f;
+        mg.y = free[1] ? mg.y : 0.0f;
         cv.x = ok[m][0] ? cv.x : 0.0f;
         cv.y = ok[m][1] ? cv.y : 0.0f;
-        const float2 dp = mul2(hi2(c1[m]), mg), dvv = fma2(hi2(s1), mg, cv);
+        const float2 dvv = fma2(hi2(s1), mg, cv);
         const float2 y1 = mul2(dp, o[m].dy), y2 = mul2(dp, o[m].dyy);
         v[m * kSum] = dp.x + dp.y;
         v[m * kSum + 1] = dvv.x + dvv.y;
