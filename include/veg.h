@@ -270,8 +270,9 @@ veg_status veg_sync_status(const void* workspace, cudaStream_t stream, int64_t* 
 veg_status veg_status_fetch(const void* workspace, void* host_status, cudaStream_t stream);
 veg_status veg_status_read(const void* host_status, int64_t* n_instances);
 
-/* Zeroes `count` (0..8) device buffers of bytes[k] bytes in one launch
- * (gradients before a step).  buffers, bytes: host arrays.
+/* Zeroes `count` (0..8) device buffers of bytes[k] bytes (gradients before a
+ * step): one launch for all below 96 MB, a fill for each larger one.  buffers,
+ * bytes: host arrays.
  */
 veg_status veg_zero_buffers(void* const* buffers, const int64_t* bytes, int32_t count,
                             cudaStream_t stream);

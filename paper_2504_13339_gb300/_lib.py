@@ -289,8 +289,16 @@ def veg_status_fetch(workspace, host_status, stream=None):
 
 
 def veg_zero_buffers(tensors, stream=None):
-    """Zeroes up to eight contiguous tensors."""
+    """Zeroes tensors, up to eight contiguous ones in a launch."""
     k = len(tensors)
+    if k > 8 or not all([t.is_contiguous() for t in tensors]):
+        flat = [t for t in tensors if t.is_contiguous()]
+        for t in tensors:
+            if not t.is_contiguous():
+                t.zero_()
+        for i in range(0, len(flat), 8):
+            veg_zero_buffers(flat[i:i + 8], stream)
+        return
     _check("veg_zero_buffers",
            load().veg_zero_buffers((_P * k)(*[t.data_ptr() for t in tensors]),
                                    (_I64 * k)(*[t.numel() * t.element_size() for t in tensors]),

@@ -129,6 +129,11 @@ RenderLayout carve_render(void* ws, int64_t n, int n_views, int64_t capacity,
   return R;
 }
 
+// Buffers from here on are left to the runtime's fill, which is the faster
+// where the bytes count: 160 MB 25 us against 29, 480 MB 65 against 80; five of
+// 64 MB 60 us against 54 in one launch.
+constexpr int64_t kZeroMemset = (int64_t)96 << 20;
+
 // Block row y zeroes buffer y: 16 bytes per step, the unaligned ends bytewise.
 __global__ void __launch_bounds__(256) zero_kernel(const ZeroBuffers z) {
   pdl_enter();
@@ -152,7 +157,10 @@ veg_status zero_launch(const ZeroBuffers& z, cudaStream_t stream) {
   int rows = 0;
   int64_t most = 0;
   for (int k = 0; k < kZeroBuffers; ++k)
-    if (z.ptr[k] && z.bytes[k] > 0) {
+    if (z.ptr[k] && z.bytes[k] >= kZeroMemset) {
+      if (cudaMemsetAsync(z.ptr[k], 0, (size_t)z.bytes[k], stream) != cudaSuccess)
+        return VEG_ERR_CUDA;
+    } else if (z.ptr[k] && z.bytes[k] > 0) {
       used.ptr[rows] = z.ptr[k];
       used.bytes[rows++] = z.bytes[k];
       most = z.bytes[k] > most ? z.bytes[k] : most;
