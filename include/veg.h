@@ -350,9 +350,11 @@ veg_status veg_composite_fwd_batch(const veg_camera* cams, int32_t n_views, int6
  * dL/ds_d and dL/ds_s per record, and veg_shade_bwd chains them to the
  * normals, the material coefficients and the means; the colour slopes in dv
  * are scaled by s_d.  Shading with stats returns VEG_ERR_UNSUPPORTED.
- * tf_group (0..8) and tile_batch (0, 128, 256 or 512) are checked and have
- * no effect: every pass takes one table and each warp stages the list chunks
- * it walks.
+ * tf_group: 1 takes a table per pass, 2 to 8 four (faster where the tables
+ * have opacity at the same scalars), 0 chooses by that overlap; the sums'
+ * order alone depends on it.  Not for view_tf or stats, which take one.
+ * tile_batch (0, 128, 256 or 512) is checked and has no effect: each warp
+ * stages the list chunks it walks.
  * stats: optional device uint64[7] accumulating (replayed pixel-splat pairs,
  * pairs walked after culling, pairs above the exponent cutoff, alpha
  * evaluations, blended pairs, blended pairs below the 0.99 clamp, pairs with

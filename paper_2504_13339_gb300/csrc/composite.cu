@@ -1,7 +1,7 @@
 // Entry points of the compositing stage: forward (Eq. 1) for a group of
 // transfer functions per pass, and the backward pass through the blend, the
 // transfer function and (optionally) the projection.
-#include "composite_kernels.cuh"
+#include "composite_bwd_group.cuh"
 
 namespace veg {
 
@@ -145,12 +145,23 @@ extern "C" veg_status veg_composite_bwd(const veg_camera* cams, int32_t n_views,
                          splat_shade);
   const float4* o4 = reinterpret_cast<const float4*>(out);
   const float4* d4 = reinterpret_cast<const float4*>(dL_dout);
-  if (lit)
-    st = launch_bwd<false, true>(A, n_views, o4, n_contrib, d4, g2, gsh, nullptr, stream);
-  else if (stats)
-    st = launch_bwd<true, false>(A, n_views, o4, n_contrib, d4, g2, nullptr, stats, stream);
-  else
-    st = launch_bwd<false, false>(A, n_views, o4, n_contrib, d4, g2, nullptr, nullptr, stream);
+  // tf_group 1: a table per pass, 2 and more: groups of four, 0: groups where
+  // the tables overlap and the items are many
+  const int64_t items =
+      total_tiles_of(cams, n_views) * ((tf.n_tf + kBwdGroup - 1) / kBwdGroup);
+  const bool may_group = !tf.view_tf && !stats && tf.n_tf > 2 && tf_group != 1;
+  A.by_overlap = may_group && tf_group == 0 && items >= kBwdGroupItems;
+  if (!may_group || tf_group == 0) {
+    if (lit)
+      st = launch_bwd<false, true>(A, n_views, o4, n_contrib, d4, g2, gsh, nullptr, stream);
+    else if (stats)
+      st = launch_bwd<true, false>(A, n_views, o4, n_contrib, d4, g2, nullptr, stats, stream);
+    else
+      st = launch_bwd<false, false>(A, n_views, o4, n_contrib, d4, g2, nullptr, nullptr, stream);
+  }
+  if (st == VEG_OK && may_group && (tf_group > 1 || A.by_overlap))
+    st = lit ? launch_bwd_group<true>(A, n_views, o4, n_contrib, d4, g2, gsh, stream)
+             : launch_bwd_group<false>(A, n_views, o4, n_contrib, d4, g2, nullptr, stream);
   if (st != VEG_OK || only_2d) return st;
   CamSet cs;
   fill_camset(cams, n_views, &cs);

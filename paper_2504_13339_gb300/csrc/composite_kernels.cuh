@@ -21,7 +21,8 @@
 // enters that item's lists, and each table stops at its own termination.
 // Walking a group of 2 or 4 tables at once shares a splat's geometry but
 // walks the union of their lists: on the 1M-Gaussian scene it took 2 to 4
-// times as long forward and 1.5 times backward.
+// times as long forward.  The backward, which shares more, does so where the
+// tables overlap (composite_bwd_group.cuh).
 //
 // What bounds both kernels is instruction issue: a tile's splats are read
 // from DRAM once (1-2% of its rate) and then meet up to 256 pixels each.  Two
@@ -247,6 +248,7 @@ struct CompArgs {
   int lut_size, n_tf;
   ViewMap vm;  // per-view tiles and output pixels (views may differ in size)
   float bg0, bg1, bg2;
+  bool by_overlap;  // backward: groups of overlapping tables go to the group kernel
 };
 
 // A work item: its tile, output image and table.
@@ -258,11 +260,13 @@ struct WorkItem {
   int2 rg;              // the tile's list
   const float4* lut;    // the table, or null
 };
-__device__ __forceinline__ WorkItem work_item(const CompArgs& A, int item, int block) {
+// (group: tables per work item, the first one's)
+__device__ __forceinline__ WorkItem work_item(const CompArgs& A, int item, int block,
+                                              int group = 1) {
   WorkItem w;
   const int wi = A.order ? A.order[item] : item;  // global tile id
   const int view = view_of_tile(A.vm, wi), tile = wi - A.vm.tile_off[view];
-  const int tiles_x = A.vm.tiles_x[view], t = (int)blockIdx.z;
+  const int tiles_x = A.vm.tiles_x[view], t = (int)blockIdx.z * group;
   w.width = A.vm.width[view];
   w.height = A.vm.height[view];
   w.rg = A.ranges[wi];
@@ -808,6 +812,86 @@ __device__ __forceinline__ void red_add_v4(float4* p, float a, float b, float c,
                : "memory");
 }
 
+// Over the warp, two splats' sums of a lane's two pixels, into their
+// accumulator slots: v = (dp, dL/dv (, dL/ds_d), dp dy, dp dy^2 (, dL/ds_s)) of
+// each, dx0 and dx1 their offsets.
+template <bool LIT>
+__device__ __forceinline__ void reduce_pair(const float* v, float dx0, float dx1, float* acc) {
+  constexpr int kSum = LIT ? 6 : 4, kAcc = LIT ? 12 : 8;
+  // over the columns' lanes: bit 4 selects the splat, bit 3 the half of its
+  // sums; then times the column's dx over the eight columns (slot bits 2 and
+  // 1): slots (S0, S0 dx, S0 dx^2, V) and (S1, S1 dx, -, S2)
+  const int lane = threadIdx.x & 31;
+  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
+  float w[kSum], x[kSum / 2], y[4], z[2];
+  exchange<kSum>(v, w, b4, 16);
+  exchange<kSum / 2>(w, x, b3, 8);
+  const float dx = b4 ? dx1 : dx0;
+  y[0] = x[0];
+  y[1] = x[0] * dx;
+  y[2] = y[1] * dx;
+  y[3] = x[1];
+  exchange<2>(y, z, b2, 4);
+  float f;
+  exchange<1>(z, &f, b1, 2);
+  f += __shfl_xor_sync(0xffffffffu, f, 1);
+  acc += b4 ? kAcc : 0;
+  if ((lane & 1) == 0) acc[(lane >> 1) & 7] = f;
+  if (LIT) {
+    float s = x[kSum / 2 - 1];
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+    if ((lane & 7) == 0) acc[8 + (b3 ? 1 : 0)] = s;
+  }
+}
+
+// Adds a splat's reduced sums to its record's gradients: moments of dp to the
+// screen gradients, du = (-a S_x - b S_y, -b S_x - c S_y), dconic = (-S_xx / 2,
+// -S_xy, -S_yy / 2).
+template <bool LIT>
+__device__ __forceinline__ void flush_splat(const float* sums, float weight, float4 aux,
+                                            uint32_t rec, float4* grad2d, float2* grad_shade) {
+  const float4* acc = reinterpret_cast<const float4*>(sums);
+  const float4 a0 = acc[0], a1 = acc[1];  // (S, Sx, Sxx, dv), (Sy, Sxy, -, Syy)
+  const bool any = a0.x != 0.f || a0.y != 0.f || a0.z != 0.f || a0.w != 0.f ||
+                   a1.x != 0.f || a1.y != 0.f || a1.w != 0.f;
+  if (any) {
+    const float4 cc = clean_conic(aux);
+    float4* dst = grad2d + 2 * (int64_t)rec;
+    const float dw = weight > 0.0f ? a0.x / weight : 0.0f;
+    red_add_v4(dst, -cc.x * a0.y - cc.y * a1.x, -cc.z * a1.x - cc.y * a0.y, -0.5f * a0.z, -a1.y);
+    red_add_v4(dst + 1, -0.5f * a1.w, a0.w, dw, 0.0f);
+  }
+  if (LIT) {
+    const float4 a2 = acc[2];
+    if (a2.x != 0.f || a2.y != 0.f) red_add_v2(grad_shade + rec, a2.x, a2.y);
+  }
+}
+
+// Whether the tables of the group from t0 on have opacity at the same scalars,
+// by 32 samples: of the samples that any table has, each has kBwdOverlap on
+// average.  Both backward kernels ask, and take the group or leave it to the
+// other.  Tables of three bumps come to 0.7 to 0.85 and are the faster one by one
+// (1M-Gaussian scene, four of them: 1105 us, in a group 1394), tables of eight to
+// 0.88 to 0.98 and are about even (1161 and 991 there; 512x512 under eight 1439
+// and 2143), one opacity under several colour maps to 1 (1045 and 764).
+constexpr int kBwdGroup = 4;
+constexpr float kBwdOverlap = 0.95f;
+__device__ __forceinline__ bool tables_overlap(const CompArgs& A, int t0) {
+  const int k = (int)(threadIdx.x & 31) * (A.lut_size - 1) / 31;
+  const int n = min(kBwdGroup, A.n_tf - t0);
+  unsigned any = 0u;
+  int sum = 0;
+#pragma unroll
+  for (int t = 0; t < kBwdGroup; ++t) {
+    const bool seen = t < n && __ldg(&A.lut[(int64_t)(t0 + t) * A.lut_size + k].w) >= kAlphaMin;
+    const unsigned m = __ballot_sync(0xffffffffu, seen);
+    any |= m;
+    sum += __popc(m);
+  }
+  return n > 2 && (float)sum >= kBwdOverlap * (float)(n * __popc(any));
+}
+
 // Walks each pixel's list back to front, from its last contribution to the
 // first splat.  Below n_contrib a pair blends exactly when its exponent is in
 // range and alpha >= 1/255 (the stop only ends the list), so every decision
@@ -881,6 +965,7 @@ __global__ void __launch_bounds__(kCompThreads, LIT || STATS ? 4 : 5)
   Warp& S = reinterpret_cast<Warp*>(smem)[warp];
   float2* s_sh = reinterpret_cast<float2*>(reinterpret_cast<Warp*>(smem) + kWarps) + threadIdx.x;
   const WorkItem W = work_item(A, (int)blockIdx.x, (int)(threadIdx.x >> 5));
+  if (A.by_overlap && tables_overlap(A, (int)blockIdx.z / kBwdGroup * kBwdGroup)) return;
   const float bx0 = W.tx0 + (float)((warp & 1) * 8), by0 = W.ty0 + (float)((warp >> 1) * 8);
   const float2 fx = dup((float)W.px), fy = make_float2((float)W.py, (float)(W.py + 4));
 
@@ -1061,53 +1146,13 @@ __global__ void __launch_bounds__(kCompThreads, LIT || STATS ? 4 : 5)
         }
         if (STATS) n_grad += (unsigned)(dp.x != 0.f) + (unsigned)(dp.y != 0.f);
       }
-      // over the columns' lanes: bit 4 selects the splat, bit 3 the half of
-      // its sums; then times the column's dx over the eight columns (slot
-      // bits 2 and 1): slots (S0, S0 dx, S0 dx^2, V) and (S1, S1 dx, -, S2)
-      const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
-      float w[kSum], x[kSum / 2], y[4], z[2];
-      exchange<kSum>(v, w, b4, 16);
-      exchange<kSum / 2>(w, x, b3, 8);
-      const float dx = b4 ? o[1].dx.x : o[0].dx.x;
-      y[0] = x[0];
-      y[1] = x[0] * dx;
-      y[2] = y[1] * dx;
-      y[3] = x[1];
-      exchange<2>(y, z, b2, 4);
-      float f;
-      exchange<1>(z, &f, b1, 2);
-      f += __shfl_xor_sync(0xffffffffu, f, 1);
-      float* acc = S.acc + (k + (b4 ? 1 : 0)) * kAcc;
-      if ((lane & 1) == 0) acc[(lane >> 1) & 7] = f;
-      if (LIT) {
-        float s = x[kSum / 2 - 1];
-#pragma unroll
-        for (int d = 4; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-        if ((lane & 7) == 0) acc[8 + (b3 ? 1 : 0)] = s;
-      }
+      reduce_pair<LIT>(v, o[0].dx.x, o[1].dx.x, S.acc + k * kAcc);
     }
     __syncwarp();
     // the lane that staged a splat adds its gradients to the record's
     if (hit) {
-      const float4* acc = reinterpret_cast<const float4*>(S.acc + slot * kAcc);
-      const float4 a0 = acc[0], a1 = acc[1];  // (S, Sx, Sxx, dv), (Sy, Sxy, -, Syy)
-      const bool any = a0.x != 0.f || a0.y != 0.f || a0.z != 0.f || a0.w != 0.f ||
-                       a1.x != 0.f || a1.y != 0.f || a1.w != 0.f;
-      if (any) {
-        // moments of dp to the screen gradients: du = (-a S_x - b S_y, -b S_x
-        // - c S_y), dconic = (-S_xx / 2, -S_xy, -S_yy / 2)
-        const float4 cc = clean_conic(S.raw[side][32 + lane]);
-        const float wt = S.raw[side][lane].w;
-        float4* dst = grad2d + 2 * (int64_t)rec;
-        const float dw = wt > 0.0f ? a0.x / wt : 0.0f;
-        red_add_v4(dst, -cc.x * a0.y - cc.y * a1.x, -cc.z * a1.x - cc.y * a0.y, -0.5f * a0.z,
-                   -a1.y);
-        red_add_v4(dst + 1, -0.5f * a1.w, a0.w, dw, 0.0f);
-      }
-      if (LIT) {
-        const float4 a2 = acc[2];
-        if (a2.x != 0.f || a2.y != 0.f) red_add_v2(grad_shade + rec, a2.x, a2.y);
-      }
+      flush_splat<LIT>(S.acc + slot * kAcc, S.raw[side][lane].w, S.raw[side][32 + lane], rec, grad2d,
+                       grad_shade);
     }
     __syncwarp();
   }
@@ -1147,6 +1192,11 @@ size_t bwd_smem_bytes(bool lit) {
          (lit ? (size_t)kCompThreads * 8 : 0);
 }
 
+// Items (tiles times groups) from which a call lets the tables' overlap choose:
+// fewer end with their longest lists, which one table at a time shortens (400x400,
+// 20,000 Gaussians, four tables of one opacity: 165 us, in groups 181; 512x512,
+// 100,000: 282 and 269).
+constexpr int64_t kBwdGroupItems = 1024;
 // Tile batch of the forward: the caller's choice (128, 256 or 512 splats),
 // else 256 (131 us on the 500k-Gaussian 512x512 frame against 135 at 128; 509
 // against 504 on the 1M-Gaussian scene under 4 tables; 512 stages less often
@@ -1171,6 +1221,7 @@ CompArgs make_args(const veg_camera* cams, int n_views, const float4* geo, const
   A.bg0 = bg ? bg[0] : 0.f;
   A.bg1 = bg ? bg[1] : 0.f;
   A.bg2 = bg ? bg[2] : 0.f;
+  A.by_overlap = false;
   return A;
 }
 
