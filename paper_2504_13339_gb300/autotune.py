@@ -1,16 +1,15 @@
-"""Tile-batch autotuner for the compositing kernels.
+"""Autotuner of the compositing launches.
 
-The compositor processes a group of TFs per pass over each tile's list
-(`tf_group` = 1, 2, 4 or 8 for the forward, up to 4 for the backward),
-staging the list in batches of `tile_batch` splats (128, 256 or 512)
-through shared memory.  A larger group shares each splat's geometry across
-more TFs but holds more state per pixel (registers) and more tables in
-shared memory; a larger batch takes fewer block barriers per list but more
-shared memory, and so fewer resident CTAs.  The best pair depends on the
-number of TFs, the image and the scene.  `tune` times every admissible
-(group, batch) pair on the caller's actual buffers with CUDA events and
-returns the fastest; results are cached per (device, problem signature) in
-a JSON file so a shape is tuned once.
+Two parameters of a launch change its time and no result: the forward's tile
+batch (the splats of a tile's list staged per pass through shared memory: a
+larger batch takes fewer barriers per list but more shared memory, and so
+fewer resident CTAs) and the backward's tables per pass (one, or groups of
+four, faster where the tables have opacity at the same scalars).  The best
+choice depends on the tables, the image and the scene.  `tune` times the
+launches that differ, as the pipeline names them (`launch_choices`; every
+(group, batch) pair for a pipeline that names none), on the caller's actual
+buffers with CUDA events and keeps the fastest; results are cached per
+(device, problem signature) in a JSON file so a shape is tuned once.
 """
 from __future__ import annotations
 
@@ -65,43 +64,49 @@ def signature(p, n_tf):
     return f"{dev}|n={p.n}|V={p.V}|{p.W}x{p.H}|T={n_tf}|cap={p.capacity // (1 << 20)}"
 
 
-def _best(times, prefix):
-    """The fastest (group, batch) among the keys '<prefix><group>x<batch>'."""
-    t, key = min((t, k) for k, t in times.items() if k.startswith(prefix))
-    g, b = key[len(prefix):].split("x")
-    return int(g), int(b)
+def _choices(p, luts, n_tf):
+    """({"fwd": [(group, batch), ...], "bwd": [...]}, cache tag)"""
+    own = getattr(p, "launch_choices", None)
+    if own is not None:
+        return own(luts), "|launches"
+    every = lambda groups: [(g, b) for g in groups if g == 1 or g // 2 < n_tf for b in BATCHES]
+    return {"fwd": every(FWD_GROUPS), "bwd": every(BWD_GROUPS)}, "|batch"
 
 
 def tune(p, luts, dout=None, reps=3, use_cache=True):
     """Chooses p.tf_group and p.tile_batch (forward), p.tf_group_bwd and
     p.tile_batch_bwd (backward, with `dout`) for pipeline `p` whose binning
     is current (project + bin_sort already run).  Returns {"fwd": group,
-    "fwd_batch": batch, "bwd": group, "bwd_batch": batch, "times": ...}."""
+    "fwd_batch": batch, "bwd": group, "bwd_batch": batch, "times": ...}; a pass
+    with a single launch to choose from is not timed."""
     n_tf = luts.shape[0]
-    key = signature(p, n_tf) + ("|bwd" if dout is not None else "") + "|batch"
+    choices, tag = _choices(p, luts, n_tf)
+    key = signature(p, n_tf) + ("|bwd" if dout is not None else "") + tag
     cache = _load() if use_cache else {}
     if key in cache:
         res = cache[key]
     else:
         times = {}
-        for g in FWD_GROUPS:
-            if g > 1 and g // 2 >= n_tf:
-                continue
-            for b in BATCHES:
-                p.tf_group, p.tile_batch = g, b
-                times[f"fwd{g}x{b}"] = _time(lambda: p.composite(luts), reps)
-        fwd, fwd_b = _best(times, "fwd")
-        p.tf_group, p.tile_batch = fwd, fwd_b
+
+        def fastest(kind, group, batch, run):
+            took = []
+            for g, b in choices[kind]:
+                setattr(p, group, g)
+                setattr(p, batch, b)
+                if len(choices[kind]) > 1:
+                    times[f"{kind}{g}x{b}"] = _time(run, reps)
+                    took.append((times[f"{kind}{g}x{b}"], (g, b)))
+            best = min(took)[1] if took else choices[kind][0]
+            setattr(p, group, best[0])
+            setattr(p, batch, best[1])
+            return best
+
+        fwd, fwd_b = fastest("fwd", "tf_group", "tile_batch", lambda: p.composite(luts))
         p.composite(luts)
-        bwd, bwd_b = 4, 256
+        bwd, bwd_b = (4, 256) if tag == "|batch" else (0, 0)
         if dout is not None:
-            for g in BWD_GROUPS:
-                if g > 1 and g // 2 >= n_tf:
-                    continue
-                for b in BATCHES:
-                    p.tf_group_bwd, p.tile_batch_bwd = g, b
-                    times[f"bwd{g}x{b}"] = _time(lambda: p.backward_2d(dout), reps)
-            bwd, bwd_b = _best(times, "bwd")
+            bwd, bwd_b = fastest("bwd", "tf_group_bwd", "tile_batch_bwd",
+                                 lambda: p.backward_2d(dout))
         res = {"fwd": fwd, "fwd_batch": fwd_b, "bwd": bwd, "bwd_batch": bwd_b, "times": times}
         if use_cache:
             cache[key] = res

@@ -1,6 +1,6 @@
-// Entry points of the compositing stage: forward (Eq. 1) for a group of
-// transfer functions per pass, and the backward pass through the blend, the
-// transfer function and (optionally) the projection.
+// Entry points of the compositing stage: forward (Eq. 1) under every transfer
+// function of a call, and the backward pass through the blend, the transfer
+// function and (optionally) the projection.
 #include "composite_bwd_group.cuh"
 
 namespace veg {

@@ -906,8 +906,8 @@ __device__ __forceinline__ bool tables_overlap(const CompArgs& A, int t0) {
 // summed first and keep their relative accuracy (a front-to-back prefix
 // K - S_i would leave them as a difference of two O(1) numbers).  Per splat,
 // the seven screen-space gradients are summed over a lane's two pixels,
-// reduced over the warp, summed over warps in shared memory and added to the
-// per-record gradient buffer once per tile.
+// reduced over the warp and added to the per-record gradient buffer, once per
+// warp and table.
 //
 // The screen gradients are linear in the sums of dp = dL/dpower times 1, dx,
 // dy, dx^2, dx dy, dy^2 (d = u - pixel; power = -a/2 dx^2 - b dx dy - c/2

@@ -46,10 +46,10 @@ class SplatPipeline:
         self.V = len(self.cams)
         self.W, self.H = self.cams[0].width, self.cams[0].height
         self.n_tf = int(n_tf)
-        self.tf_group = int(tf_group)      # TFs per compositing pass (forward)
-        self.tf_group_bwd = int(tf_group)  # TFs per pass (backward)
+        self.tf_group = int(tf_group)      # forward: no effect (one TF per pass)
+        self.tf_group_bwd = int(tf_group)  # backward: 1 one TF per pass, 2.. four, 0 by overlap
         self.tile_batch = 0                # splats staged per pass (forward; 0 = 256)
-        self.tile_batch_bwd = 0            # (backward)
+        self.tile_batch_bwd = 0            # backward: no effect
         self.device = torch.device(device)
         self.c_cams = _lib.cameras(self.cams)
         nrec = self.V * self.n
@@ -186,6 +186,14 @@ class SplatPipeline:
                                self.n_contrib, stats, stream, tile_order=self.order,
                                splat_shade=self._shade_buf(), tile_batch=self.tile_batch)
         return self.out
+
+    def launch_choices(self, luts):
+        """The (tf_group, tile_batch) pairs that make different launches, for the
+        autotuner: the forward's batches where it stages any, the backward's
+        tables per pass where there are more than two."""
+        staged = _lib.veg_composite_fwd_batch(self.c_cams, self.n, _lib.tf_desc(luts))
+        return {"fwd": [(0, b) for b in ((128, 256, 512) if staged else (0,))],
+                "bwd": [(g, 0) for g in ((1, 4) if luts.shape[0] > 2 else (0,))]}
 
     def _shade_buf(self):
         return self.splat_shade if self._lit is not None else None
