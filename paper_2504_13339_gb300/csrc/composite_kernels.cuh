@@ -289,7 +289,13 @@ __device__ __forceinline__ WorkItem work_item(const CompArgs& A, int item, int b
 template <int N>
 __device__ __forceinline__ void async_copy(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(N) : "memory");
+  // past the L1 cache, which the tables want (through it the backward of two
+  // tables over 177x170 with 2M Gaussians takes 3245 us, past it 3043); 8-byte
+  // copies exist through it only
+  if (N == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void async_commit() {
   asm volatile("cp.async.commit_group;" ::: "memory");
