@@ -50,13 +50,11 @@ struct Count {
   }
 };
 
-// The items of a kernel behind a sort that may have timed out (`after`, the
-// status header; null for sorts that wait for nothing): none if it did, since
-// the places that it did not write hold whatever the buffer held.  (The
-// look-back passes themselves set the flag, and their threads must agree on
-// the count: they check their places instead.)
-__device__ __forceinline__ int64_t count_after(const Count& c, const WsHeader* after) {
-  return after && (after->flags & FLAG_TIMEOUT) ? 0 : c.get();
+// A record of a sorted order: where a sort has timed out, the places that it
+// did not write hold whatever the buffer held, and must not be followed out of
+// the records (the lists are emptied at the end: ranges_kernel).
+__device__ __forceinline__ uint32_t record_of(const uint32_t* order, int64_t i, const Count& c) {
+  return min(order[i], (uint32_t)((c.dev ? c.cap : c.fixed) - 1));
 }
 
 __device__ __forceinline__ float rcp_approx_f(float x) {
@@ -372,8 +370,8 @@ __device__ __forceinline__ unsigned digit_peers(uint32_t d, bool valid) {
 // stride over the chunks) or found by look-back (blocks loop over tickets,
 // so a chunk's predecessors belong to blocks that are already running; a
 // look-back not answered within `spins` polls sets FLAG_TIMEOUT in the
-// header and stops waiting: the output is then void, and since later passes
-// read places that nothing was written to, look-back passes check theirs).  dtot: the digit
+// header and stops waiting: the output is then void, and as later passes would
+// read places that nothing was written to, no chunk is taken any more).  dtot: the digit
 // totals of the pass.
 template <bool TABLE, int ITEMS>
 __global__ void __launch_bounds__(kThreads, ITEMS == 4 ? 6 : 4)
@@ -416,7 +414,10 @@ __global__ void __launch_bounds__(kThreads, ITEMS == 4 ? 6 : 4)
       if (b >= nch) break;  // block-uniform
       if (digit) before_chunk = hist[(int64_t)tid * nblocks + b];
     } else {
-      if (tid == 0) s_chunk = (int)atomicAdd(ticket, 1u);
+      if (tid == 0) {  // (both on their way together)
+        const int next = (int)atomicAdd(ticket, 1u);
+        s_chunk = hdr->flags & FLAG_TIMEOUT ? nch : next;
+      }
       __syncthreads();
       b = s_chunk;
       if (b >= nch) break;  // block-uniform
@@ -521,7 +522,6 @@ __global__ void __launch_bounds__(kThreads, ITEMS == 4 ? 6 : 4)
       uint32_t key = s_keys[p];
       uint32_t d = ((key - kb) >> shift) & mask;
       uint32_t g = s_dbase[d] + (uint32_t)p;
-      if (!TABLE && (int64_t)g >= n) continue;  // only after a timeout
       kout[g] = key;
       if (vout) vout[g] = s_vals[p];  // keys-only sorts carry no values
     }
@@ -668,13 +668,13 @@ __global__ void __launch_bounds__(1024)
 // blocks of the emission kernel).
 __global__ void __launch_bounds__(256)
     count_reduce_kernel(const int32_t* __restrict__ tiles, SortedVals sorted, Count cnt,
-                        const WsHeader* after, unsigned long long* __restrict__ bsum) {
+                        unsigned long long* __restrict__ bsum) {
   pdl_enter();
   const uint32_t* __restrict__ order = sorted.get();
   __shared__ unsigned long long s_warp[8];
-  const int64_t nrec = count_after(cnt, after);
+  const int64_t nrec = cnt.get();
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  unsigned long long acc = i < nrec ? (unsigned)tiles[order[i]] : 0u;
+  unsigned long long acc = i < nrec ? (unsigned)tiles[record_of(order, i, cnt)] : 0u;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) s_warp[threadIdx.x >> 5] = acc;
@@ -741,18 +741,18 @@ __global__ void __launch_bounds__(1024)
 __global__ void __launch_bounds__(256)
     emit_kernel(const int32_t* __restrict__ tiles, const short4* __restrict__ rect,
                 SortedVals sorted, const unsigned long long* __restrict__ bsum, Count visible,
-                const WsHeader* after, int64_t n_per_view, ViewMap vm, int64_t capacity,
-                int rec_bits, uint32_t* __restrict__ ikeys, uint32_t* __restrict__ ivals) {
+                int64_t n_per_view, ViewMap vm, int64_t capacity, int rec_bits,
+                uint32_t* __restrict__ ikeys, uint32_t* __restrict__ ivals) {
   pdl_enter();
   __shared__ unsigned long long s_warp[8];
   const uint32_t* __restrict__ order = sorted.get();
   const int lane = threadIdx.x & 31;
-  const int64_t nrec = count_after(visible, after);
+  const int64_t nrec = visible.get();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t g = 0, cnt = 0;
   short4 rc = make_short4(0, 0, 0, 0);
   if (i < nrec) {
-    g = order[i];
+    g = record_of(order, i, visible);
     cnt = (uint32_t)tiles[g];
     if (cnt) rc = rect[g];
   }
@@ -834,11 +834,12 @@ __global__ void zero_ranges_kernel(int2* __restrict__ ranges, int64_t count,
 // aligned): a run starts where the key differs from its predecessor and
 // ends where it differs from its successor.  Keys are < 2^31, so 0xffffffff
 // marks "no neighbour".
-__global__ void ranges_kernel(const uint32_t* __restrict__ keys, Count cnt, const WsHeader* after,
+__global__ void ranges_kernel(const uint32_t* __restrict__ keys, Count cnt, const WsHeader* hdr,
                               int2* __restrict__ ranges, int key_shift,
                               uint32_t* __restrict__ vals) {
   pdl_enter();
-  const int64_t n = count_after(cnt, after);
+  if (hdr->flags & FLAG_TIMEOUT) return;  // void lists: every range stays empty
+  const int64_t n = cnt.get();
   // a bounded grid strides over the items: their count is far below the
   // capacity that the host knows
   for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i0 < n;
@@ -878,10 +879,11 @@ __global__ void ranges_kernel(const uint32_t* __restrict__ keys, Count cnt, cons
 // key = (view << (tb + 32)) | (tile of the view << 32) | depth bits, with tb
 // the tile bits of the largest view.
 __global__ void keys64_kernel(const uint32_t* __restrict__ tkeys, const uint32_t* __restrict__ vals,
-                              Count cnt, const WsHeader* after, const float4* __restrict__ geo,
+                              Count cnt, const WsHeader* hdr, const float4* __restrict__ geo,
                               ViewMap vm, int tb, int key_shift, uint64_t* __restrict__ keys64) {
   pdl_enter();
-  const int64_t n = count_after(cnt, after);
+  if (hdr->flags & FLAG_TIMEOUT) return;
+  const int64_t n = cnt.get();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   uint32_t tk = tkeys[i] >> key_shift;
@@ -1098,12 +1100,12 @@ __device__ __forceinline__ int64_t cell_item(int j) {
 constexpr uint32_t kNoCells = 0x0000ffffu;  // first cell beyond the last
 __global__ void __launch_bounds__(256)
     cell_reduce_kernel(const int32_t* __restrict__ tiles, const short4* __restrict__ rect,
-                       SortedVals sorted, Count cnt, const WsHeader* after,
-                       unsigned long long* __restrict__ esum, unsigned long long* __restrict__ csum, uint32_t* __restrict__ cells) {
+                       SortedVals sorted, Count cnt, unsigned long long* __restrict__ esum,
+                       unsigned long long* __restrict__ csum, uint32_t* __restrict__ cells) {
   pdl_enter();
   const uint32_t* __restrict__ order = sorted.get();
   __shared__ unsigned long long s_e[8], s_c[8];
-  const int64_t nrec = count_after(cnt, after);
+  const int64_t nrec = cnt.get();
   if ((int64_t)blockIdx.x * kCellBlock >= nrec) {  // block-uniform
     if (threadIdx.x == 0) esum[blockIdx.x] = csum[blockIdx.x] = 0ull;
     return;
@@ -1111,7 +1113,7 @@ __global__ void __launch_bounds__(256)
   uint32_t g[kCellRows], t[kCellRows];
   short4 rc[kCellRows];
 #pragma unroll
-  for (int j = 0; j < kCellRows; ++j) g[j] = cell_item(j) < nrec ? order[cell_item(j)] : 0u;
+  for (int j = 0; j < kCellRows; ++j)     g[j] = cell_item(j) < nrec ? record_of(order, cell_item(j), cnt) : 0u;
 #pragma unroll
   for (int j = 0; j < kCellRows; ++j) {
     const bool in = cell_item(j) < nrec;
@@ -1254,21 +1256,21 @@ __global__ void __launch_bounds__(256)
     cell_emit_kernel(const int32_t* __restrict__ tiles, const uint32_t* __restrict__ cells,
                      SortedVals sorted, const unsigned long long* __restrict__ esum,
                      const unsigned long long* __restrict__ csum, Count visible,
-                     const WsHeader* after, int64_t n_per_view,
-                     const __grid_constant__ CellMap cm, int64_t capacity, int rec_bits, uint32_t* __restrict__ ckeys, uint32_t* __restrict__ cvals,
+                     int64_t n_per_view, const __grid_constant__ CellMap cm, int64_t capacity,
+                     int rec_bits, uint32_t* __restrict__ ckeys, uint32_t* __restrict__ cvals,
                      WsHeader* __restrict__ hdr) {
   pdl_enter();
   __shared__ unsigned long long s_e[8], s_c[8];
   const uint32_t* __restrict__ order = sorted.get();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t nrec = count_after(visible, after);
+  const int64_t nrec = visible.get();
   const bool over = (hdr->flags & FLAG_CAPACITY) != 0u;
   if ((int64_t)blockIdx.x * kCellBlock >= nrec) return;  // block-uniform
   uint32_t g[kCellRows], packed[kCellRows];
 #pragma unroll
   for (int j = 0; j < kCellRows; ++j) {
     const bool in = cell_item(j) < nrec;
-    g[j] = in ? order[cell_item(j)] : 0u;
+    g[j] = in ? record_of(order, cell_item(j), visible) : 0u;
     packed[j] = in ? cells[cell_item(j)] : kNoCells;
   }
   auto count = [&](int j) {
@@ -1390,10 +1392,10 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// One chunk: its first pair and their number (an end could pass 2^31), the
-// cell's first tile, its view: (first, pairs, ox | oy << 16, view).  Every CTA
-// scans the cells' chunks (block 0 writes cstart [n_cells + 1]) and describes
-// its share of the cells.
+// One chunk: pairs [first, end) of a cell (compared unsigned: an index beyond the
+// end may pass 2^31), the cell's first tile, its view: (first, end, ox | oy << 16,
+// view).  Every CTA scans the cells' chunks (block 0 writes cstart [n_cells + 1])
+// and describes its share of the cells.
 __device__ __forceinline__ int cell_chunks(int2 r) {
   return (int)(((unsigned)(r.y - r.x) + kCellChunk - 1) / kCellChunk);
 }
@@ -1448,7 +1450,8 @@ __global__ void __launch_bounds__(kCellScanThreads)
       const int cell = cc - cm.cell_off[view], cx = cm.cells_x[view];
       const int origin = ((cell % cx) << kCellShift) | (((cell / cx) << kCellShift) << 16);
       for (int k = lane; k < n && f + k < max_chunks; k += 32)
-        desc[f + k] = make_int4(q.x + k * kCellChunk, min(kCellChunk, q.y - q.x - k * kCellChunk),
+        desc[f + k] = make_int4(q.x + k * kCellChunk,
+                                (int)min((unsigned)q.x + (k + 1) * kCellChunk, (unsigned)q.y),
                                 origin, view);
     }
     carry += s_total;
@@ -1512,11 +1515,13 @@ __global__ void __launch_bounds__(256)
     uint32_t g[8];
     short4 rc[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-      g[j] = j * 32 + lane < d.y ? __ldg(P.words + d.x + j * 32 + lane) & P.rec_mask : 0u;
+    for (int j = 0; j < 8; ++j) {
+      const unsigned i = (unsigned)d.x + j * 32 + lane;
+      g[j] = i < (unsigned)d.y ? __ldg(P.words + i) & P.rec_mask : 0u;
+    }
 #pragma unroll
     for (int j = 0; j < 8; ++j)
-      rc[j] = j * 32 + lane < d.y ? __ldg(P.rect + g[j]) : make_short4(0, 0, 0, 0);
+      rc[j] = (unsigned)d.x + j * 32 + lane < (unsigned)d.y ? __ldg(P.rect + g[j]) : make_short4(0, 0, 0, 0);
     uint32_t lo = 0, hi = 0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -1634,10 +1639,10 @@ __global__ void __launch_bounds__(kCellChunk)
   // the current chunk is staged and written
   auto chunk = [&](int k) { return k < total ? __ldg(desc + k) : make_int4(0, 0, 0, 0); };
   auto pair_of = [&](int4 d) {
-    return tid < d.y ? __ldg(P.words + d.x + tid) & P.rec_mask : 0u;
+    return (unsigned)d.x + tid < (unsigned)d.y ? __ldg(P.words + ((unsigned)d.x + tid)) & P.rec_mask : 0u;
   };
   auto rect_of = [&](int4 d, uint32_t g) {
-    return tid < d.y ? __ldg(P.rect + g) : make_short4(0, 0, 0, 0);
+    return (unsigned)d.x + tid < (unsigned)d.y ? __ldg(P.rect + g) : make_short4(0, 0, 0, 0);
   };
   auto start_of = [&](int4 d, int k) {
     uint32_t at = 0;
@@ -2049,7 +2054,6 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
   uint32_t* const dk[2] = {L.dk0, L.dk1};
   uint32_t* const dv[2] = {L.dv0, L.dv1};
   const SortedVals order = radix_sort(dk, dv, cr, 32, L.nb_rec, L, 0, L.hdr, stream);
-  const WsHeader* const after_depth = L.nb_rec <= kLookbackMaxChunks ? L.hdr : nullptr;
   const CellMap cm = make_cellmap(cams, n_views);
   const int64_t n_cells = cm.cell_off[n_views];
   int rec_bits = 1;
@@ -2067,8 +2071,8 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
     int* cstart = reinterpret_cast<int*>(L.dk1) + 2 * n_cells;
     int4* desc = reinterpret_cast<int4*>(L.hist);
     launch_k(cell_reduce_kernel, nb, 256, 0, stream,
-             nrec <= kSmallRecords ? tiles : (const int32_t*)nullptr, rect, order, cr, after_depth,
-             L.esum, csum, L.dk0);
+             nrec <= kSmallRecords ? tiles : (const int32_t*)nullptr, rect, order, cr, L.esum,
+             csum, L.dk0);
     launch_k(cell_top_kernel, 1, kCellScanThreads, 0, stream, L.esum, csum, nb, L.hdr, capacity,
              cranges, (int)n_cells);
     // sorted records end in iv0 (unpacked) or in the packed words' buffer
@@ -2080,7 +2084,7 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
       vbuf[(passes & 1) ^ 1] = vals;
     }
     launch_k(cell_emit_kernel, nb, 256, 0, stream, tiles, (const uint32_t*)L.dk0, order,
-             (const unsigned long long*)L.esum, (const unsigned long long*)csum, cr, after_depth, n, cm,
+             (const unsigned long long*)L.esum, (const unsigned long long*)csum, cr, n, cm,
              capacity, rec_bits, kbuf[0], vbuf[0], L.hdr);
     count_launch(3);
     const Count cc{0, &L.hdr->n_cells, capacity};
@@ -2089,7 +2093,7 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
     uint32_t* table = kbuf[(passes & 1) ^ 1];
     uint32_t* totals = table + kCellTiles * max_chunks;
     launch_k(ranges_kernel, pass_grid((int)grid_for(capacity, 1024), 8), 256, 0, stream, ckeys, cc,
-             (const WsHeader*)nullptr, cranges, rec_bits, (uint32_t*)nullptr);
+             (const WsHeader*)L.hdr, cranges, rec_bits, (uint32_t*)nullptr);
     launch_k(cell_map_kernel, 16, kCellScanThreads, 0, stream, (const int2*)cranges, (int)n_cells,
              cm, (int)max_chunks, cstart, desc);
     CellPairs P;
@@ -2110,7 +2114,7 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
     return launch_status();
   }
   // 2. instance offsets in depth order, total into the header
-  launch_k(count_reduce_kernel, L.nb_emit, 256, 0, stream, tiles, order, cr, after_depth, L.esum);
+  launch_k(count_reduce_kernel, L.nb_emit, 256, 0, stream, tiles, order, cr, L.esum);
   launch_k(count_top_kernel, 1, 1024, 0, stream, L.esum, L.nb_emit, L.hdr, capacity);
   count_launch(2);
   // 3. emit (tile key, record) pairs, then stable sort by tile key.  When
@@ -2129,20 +2133,18 @@ veg_status binsort_launch(const veg_camera* cams, int n_views, int64_t n, const 
     vbuf[passes % 2 == 0 ? 1 : 0] = L.iv0;
   }
   launch_k(emit_kernel, L.nb_emit, 256, 0, stream, tiles, rect, order,
-           (const unsigned long long*)L.esum, cr, after_depth, n, vm, capacity, rec_bits, kbuf[0],
-           vbuf[0]);
+           (const unsigned long long*)L.esum, cr, n, vm, capacity, rec_bits, kbuf[0], vbuf[0]);
   count_launch();
   radix_sort(kbuf, vbuf, ci, bits, nb_inst, L, 1, nullptr, stream, kLookbackSpins, rec_bits);
   const uint32_t* fkeys = kbuf[passes & 1];
-  const WsHeader* const after_tiles = nb_inst <= kLookbackMaxChunks ? L.hdr : nullptr;
   // 4. per-tile ranges (and the records, from packed words) and optional
   //    64-bit keys
   launch_k(ranges_kernel, pass_grid((int)grid_for(capacity, 1024), 8), 256, 0, stream, fkeys, ci,
-           after_tiles, ranges, rec_bits, packed ? vals : (uint32_t*)nullptr);
+           (const WsHeader*)L.hdr, ranges, rec_bits, packed ? vals : (uint32_t*)nullptr);
   count_launch();
   if (keys) {
-    launch_k(keys64_kernel, grid_for(capacity, 256), 256, 0, stream, fkeys, vals, ci, after_tiles,
-             geo, vm, tile_bits_of(vm.max_tiles), rec_bits, keys);
+    launch_k(keys64_kernel, grid_for(capacity, 256), 256, 0, stream, fkeys, vals, ci,
+             (const WsHeader*)L.hdr, geo, vm, tile_bits_of(vm.max_tiles), rec_bits, keys);
     count_launch();
   }
   return launch_status();
