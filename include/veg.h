@@ -236,8 +236,9 @@ veg_status veg_bin_sort_static(const veg_camera* cams, int32_t n_views, int64_t 
  * a CTA waits for the digit counts that the CTAs of the earlier chunks
  * publish; every such wait gives up after a bounded number of polls, sets a
  * timeout flag in the workspace header and lets the kernel finish, so a
- * fault in that chain shows as a status, never as a hang.  This call sorts n seeded keys (key i = (i * 2654435761) >> 4,
- * mod 2^32; value i) with that sort, each wait limited to `spins` polls,
+ * fault in that chain shows as a status, never as a hang.  This call sorts n
+ * seeded keys (key i = (i * 2654435761) >> 4, mod 2^32; value i) with that
+ * sort, each wait limited to `spins` polls,
  * and copies the sorted keys and values to keys_out and vals_out (device
  * uint32 [n], overwritten).  With starve_first != 0 the first chunk is
  * never taken, so the next chunk's wait runs out: veg_sync_status on the
@@ -310,9 +311,9 @@ veg_status veg_zero_buffers(void* const* buffers, const int64_t* bytes, int32_t 
  * bg: host float[3].  stats: optional device uint64[5] accumulating
  * (visited pixel-splat pairs -- every pair reached before the pixel stops --,
  * pairs walked by the kernel after its culling, pairs above the exponent
- * cutoff -- below it no TF of the group can reach alpha >= 1/255 --, alpha
- * evaluations, blended pairs), NULL to skip the instrumented kernel.  n is the per-view record count used by
- * veg_project.
+ * cutoff -- below it the splat cannot reach alpha >= 1/255 --, alpha
+ * evaluations, blended pairs), NULL to skip the instrumented kernel.  n is the
+ * per-view record count used by veg_project.
  */
 veg_status veg_composite_fwd(const veg_camera* cams, int32_t n_views, int64_t n,
                              const float* splat_geo, const float* splat_aux,

@@ -399,7 +399,8 @@ __global__ void __launch_bounds__(kThreads, ITEMS == 4 ? 6 : 4)
   const bool digit = (uint32_t)tid <= mask;  // rows of hist and dtot exist for digits only
   if (!TABLE && look_next) {  // the next pass's look-back words (unused during this pass)
     const int64_t nl = (int64_t)nch * 256;
-    for (int64_t i = (int64_t)blockIdx.x * kThreads + tid; i < nl; i += (int64_t)gridDim.x * kThreads)
+    for (int64_t i = (int64_t)blockIdx.x * kThreads + tid; i < nl;
+         i += (int64_t)gridDim.x * kThreads)
       look_next[i] = 0ull;
   }
   // the digit totals, whose exclusive prefix is each digit's first output
@@ -844,35 +845,35 @@ __global__ void ranges_kernel(const uint32_t* __restrict__ keys, Count cnt, cons
   // capacity that the host knows
   for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i0 < n;
        i0 += (int64_t)gridDim.x * blockDim.x * 4) {
-  // packed words (key_shift > 0): the list id above key_shift, the record
-  // below it (written to vals); 0xffffffff marks "no neighbour" after the
-  // shift (list ids are below 2^31)
-  uint32_t w[4];
-  if (i0 + 4 <= n) {
-    const uint4 q = *reinterpret_cast<const uint4*>(keys + i0);
-    w[0] = q.x;
-    w[1] = q.y;
-    w[2] = q.z;
-    w[3] = q.w;
-  } else {
+    // packed words (key_shift > 0): the list id above key_shift, the record
+    // below it (written to vals); 0xffffffff marks "no neighbour" after the
+    // shift (list ids are below 2^31)
+    uint32_t w[4];
+    if (i0 + 4 <= n) {
+      const uint4 q = *reinterpret_cast<const uint4*>(keys + i0);
+      w[0] = q.x;
+      w[1] = q.y;
+      w[2] = q.z;
+      w[3] = q.w;
+    } else {
 #pragma unroll
-    for (int t = 0; t < 4; ++t) w[t] = i0 + t < n ? keys[i0 + t] : 0u;
-  }
-  uint32_t k[6];
-  k[0] = i0 > 0 ? keys[i0 - 1] >> key_shift : 0xffffffffu;
+      for (int t = 0; t < 4; ++t) w[t] = i0 + t < n ? keys[i0 + t] : 0u;
+    }
+    uint32_t k[6];
+    k[0] = i0 > 0 ? keys[i0 - 1] >> key_shift : 0xffffffffu;
 #pragma unroll
-  for (int t = 0; t < 4; ++t) k[1 + t] = i0 + t < n ? w[t] >> key_shift : 0xffffffffu;
-  k[5] = i0 + 4 < n ? keys[i0 + 4] >> key_shift : 0xffffffffu;
-  const uint32_t rmask = key_shift > 0 ? (0xffffffffu >> (32 - key_shift)) : 0u;
+    for (int t = 0; t < 4; ++t) k[1 + t] = i0 + t < n ? w[t] >> key_shift : 0xffffffffu;
+    k[5] = i0 + 4 < n ? keys[i0 + 4] >> key_shift : 0xffffffffu;
+    const uint32_t rmask = key_shift > 0 ? (0xffffffffu >> (32 - key_shift)) : 0u;
 #pragma unroll
-  for (int t = 0; t < 4; ++t) {
-    const int64_t i = i0 + t;
-    if (i >= n) break;
-    const uint32_t kk = k[1 + t];
-    if (kk != k[t]) ranges[kk].x = (int)i;
-    if (kk != k[2 + t]) ranges[kk].y = (int)(i + 1);
-    if (vals) vals[i] = w[t] & rmask;
-  }
+    for (int t = 0; t < 4; ++t) {
+      const int64_t i = i0 + t;
+      if (i >= n) break;
+      const uint32_t kk = k[1 + t];
+      if (kk != k[t]) ranges[kk].x = (int)i;
+      if (kk != k[2 + t]) ranges[kk].y = (int)(i + 1);
+      if (vals) vals[i] = w[t] & rmask;
+    }
   }
 }
 
@@ -1050,8 +1051,10 @@ SortedVals radix_sort(uint32_t* const k[2], uint32_t* const v[2], Count cnt, int
 // What bounds it is the latency of each short kernel on L2-resident pairs up
 // to a few million instances, and beyond that the shared-memory traffic of
 // the placing.  Projection, binning and sort of 1M Gaussians (8.6M instances,
-// 1024x1024) take 225 us with it and 285 with the tile sort of all instances;
-// of two views of 3M Gaussians (58.8M instances, 1601x1199) 1041 and 1585.
+// 1024x1024) take 208 us with it and 272 with the tile sort of all instances;
+// of two views of 3M Gaussians (58.8M instances, 1601x1199) 930 and 1540.  Where
+// a record has few tiles and the tiles are few, it is the slower (1M Gaussians
+// within 25 pixels, two tiles each: 230 and 172): the host knows neither number.
 //
 // Overflow: instances beyond the capacity are dropped in depth order, a
 // record's tiles row-major.  Records past the capacity emit no pair; the one
@@ -1113,7 +1116,8 @@ __global__ void __launch_bounds__(256)
   uint32_t g[kCellRows], t[kCellRows];
   short4 rc[kCellRows];
 #pragma unroll
-  for (int j = 0; j < kCellRows; ++j)     g[j] = cell_item(j) < nrec ? record_of(order, cell_item(j), cnt) : 0u;
+  for (int j = 0; j < kCellRows; ++j)
+    g[j] = cell_item(j) < nrec ? record_of(order, cell_item(j), cnt) : 0u;
 #pragma unroll
   for (int j = 0; j < kCellRows; ++j) {
     const bool in = cell_item(j) < nrec;
@@ -1249,8 +1253,8 @@ __global__ void __launch_bounds__(kCellScanThreads)
 // writes its own; else lanes write consecutive positions of the pairs' run, each finding its
 // record by a binary search over the lanes' ends (as emit_kernel does for
 // instances), which no wide record slows down but which took 290 instructions
-// per 32 records everywhere (6M records: 57 us, 50 so).  rec_bits > 0: one packed word,
-// cell << rec_bits | record.
+// per 32 records everywhere (6M records: 57 us, 50 so).  rec_bits > 0: one packed
+// word, cell << rec_bits | record.
 constexpr uint32_t kCellOwnPairs = 9;
 __global__ void __launch_bounds__(256)
     cell_emit_kernel(const int32_t* __restrict__ tiles, const uint32_t* __restrict__ cells,
@@ -1337,8 +1341,9 @@ __global__ void __launch_bounds__(256)
       }
     }
     const int view = (int)(g[j] / (uint32_t)n_per_view);
-    const int cx = cm.cells_x[view], wx = (int)(packed[j] >> 16 & 0xffu) - (int)(packed[j] & 0xffu) + 1;
-    const int key0 = cm.cell_off[view] + (int)(packed[j] >> 8 & 0xffu) * cx + (int)(packed[j] & 0xffu);
+    const int x0 = (int)(packed[j] & 0xffu), y0 = (int)(packed[j] >> 8 & 0xffu);
+    const int cx = cm.cells_x[view], wx = (int)(packed[j] >> 16 & 0xffu) - x0 + 1;
+    const int key0 = cm.cell_off[view] + y0 * cx + x0;
     if (__reduce_max_sync(0xffffffffu, cnt) <= kCellOwnPairs) {
       // few pairs per record: each lane writes its own, next to its
       // neighbours'
@@ -1521,7 +1526,8 @@ __global__ void __launch_bounds__(256)
     }
 #pragma unroll
     for (int j = 0; j < 8; ++j)
-      rc[j] = (unsigned)d.x + j * 32 + lane < (unsigned)d.y ? __ldg(P.rect + g[j]) : make_short4(0, 0, 0, 0);
+      rc[j] = (unsigned)d.x + j * 32 + lane < (unsigned)d.y ? __ldg(P.rect + g[j])
+                                                            : make_short4(0, 0, 0, 0);
     uint32_t lo = 0, hi = 0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -1639,7 +1645,8 @@ __global__ void __launch_bounds__(kCellChunk)
   // the current chunk is staged and written
   auto chunk = [&](int k) { return k < total ? __ldg(desc + k) : make_int4(0, 0, 0, 0); };
   auto pair_of = [&](int4 d) {
-    return (unsigned)d.x + tid < (unsigned)d.y ? __ldg(P.words + ((unsigned)d.x + tid)) & P.rec_mask : 0u;
+    const unsigned i = (unsigned)d.x + tid;
+    return i < (unsigned)d.y ? __ldg(P.words + i) & P.rec_mask : 0u;
   };
   auto rect_of = [&](int4 d, uint32_t g) {
     return (unsigned)d.x + tid < (unsigned)d.y ? __ldg(P.rect + g) : make_short4(0, 0, 0, 0);
@@ -1728,9 +1735,9 @@ __global__ void __launch_bounds__(kCellChunk)
 // that the cell sort does not end in (the chunk counts, the tiles' totals).
 // Taken when the tile sort would need more than one pass and the capacity is
 // at least 1.3M instances.  Projection and binning with the cells and with
-// the tile sort, by capacity (1.25 times the instances): 0.56M 82 and 77 us
-// (100k Gaussians), 1.07M 106 and 103 (300k), 1.21M 98 and 104 (60k), 1.54M
-// 91 and 95 (100k), 1.95M 116 and 120 (500k).  Small images keep the one-pass
+// the tile sort, by capacity (1.25 times the instances): 0.56M 87 and 82 us
+// (100k Gaussians), 1.07M 105 and 104 (300k), 1.21M 98 and 105 (60k), 1.54M
+// 91 and 96 (100k), 1.95M 117 and 121 (500k).  Small images keep the one-pass
 // tile sort, and calls that ask for the 64-bit keys the sort that has them.
 constexpr int64_t kCellMinCapacity = (int64_t)5 << 18;
 bool cell_binning_fits(int64_t nrec, int64_t nranges, int64_t n_cells, int64_t capacity,

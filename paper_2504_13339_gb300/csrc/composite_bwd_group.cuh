@@ -8,10 +8,10 @@
 // pair's geometry, a splat's reduction and its update once.
 //
 // What bounds it is instruction issue, as there.  1M-Gaussian scene, 1024x1024,
-// four tables, a table per pass and four: one opacity under four colour maps 1045
-// and 764 us, opacity 0.05 throughout 3720 and 2467, 0.8 611 and 451; tables of
-// three bumps 1105 and 1394, of eight 1161 and 991.  The choice between them costs
-// a call 10 to 20 us.
+// four tables, a table per pass and four: one opacity under four colour maps 1019
+// and 760 us, opacity 0.05 throughout 3599 and 2437, 0.8 604 and 449; tables of
+// three bumps 1079 and 1374, of eight 1142 and 981.  Choosing between them takes
+// 8 us of the former's call and 20 of the latter's.
 #pragma once
 
 #include "composite_kernels.cuh"

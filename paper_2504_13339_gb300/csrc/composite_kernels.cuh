@@ -8,10 +8,10 @@
 // chosen by the caller or its autotuner) through shared memory; the
 // backward's warps each stage the chunks of 32 that they walk.  The stager
 // evaluates a splat's colour and opacity under the table (linear
-// interpolation, the table read through the L1 cache), the exponent below which it
-// cannot reach alpha = 1/255, and which warp blocks its visible ellipse can
-// touch; each warp walks only the splats that touch its block, so pairs that
-// provably cannot blend cost nothing.  A pixel leaves once it has terminated
+// interpolation, the table read through the L1 cache), the exponent below
+// which it cannot reach alpha = 1/255, and which warp blocks its visible
+// ellipse can touch; each warp walks only the splats that touch its block, so
+// pairs that provably cannot blend cost nothing.  A pixel leaves once it has terminated
 // (T (1 - alpha) < 1e-4); a work item ends once all its pixels have left.
 //
 // Launches of few work items take a second forward kernel, whose CTA holds one
@@ -29,9 +29,10 @@
 // pixels per lane halve what a splat costs per pixel beyond its own
 // arithmetic (list entry, shared-memory loads, loop, warp votes and, in the
 // backward, the warp reduction), and most of the pair's arithmetic runs in
-// the two-wide float32 instructions.  With one pixel per lane the 1M-Gaussian
-// scene (1024x1024, 4 tables) took 633 us forward and 1254 us backward
-// (1778 us with four tables per pass); with two 500 and 940 us.
+// the two-wide float32 instructions.  From one pixel per lane (and groups of
+// tables) to two, whole calls on the 1M-Gaussian scene (1024x1024, four tables)
+// went from 820 to 655 us forward and from 1812 to 1231 backward; the kernels
+// now take 518 and 1077.
 //
 // The per-pair arithmetic that decides skips, the 0.99 clamp and
 // termination uses explicitly rounded operations shared by the forward and
@@ -201,7 +202,8 @@ __device__ __forceinline__ int build_warp_list(const unsigned char* s_mask, List
   } else {
 #pragma unroll
     for (int w = 0; w < NW; ++w) {
-      const unsigned long long m = reinterpret_cast<const unsigned long long*>(s_mask)[lane * NW + w];
+      const unsigned long long m =
+          reinterpret_cast<const unsigned long long*>(s_mask)[lane * NW + w];
       bits[w] = (m >> warp) & 0x0101010101010101ull;  // bit 8k: position P l + 8 w + k
       c += __popcll(bits[w]);
     }
@@ -320,7 +322,7 @@ __device__ __forceinline__ void fetch_record(const CompArgs& A, RawSlot s, uint3
 // table entries around its scalar, aw = A w.  The entries come through the L1
 // cache: a copy of the table in shared memory costs each item its time and the
 // SMs their CTAs (1M-Gaussian scene under four tables, forward and backward:
-// 525 and 1086 us at 256 entries, 528 and 1105 at 4096; with the copy 563 and
+// 518 and 1077 us at 256 entries, 520 and 1095 at 4096; with the copy 563 and
 // 1125, 1158 and 1958).
 struct SplatTf {
   float4 lo, hi;
@@ -598,7 +600,7 @@ __global__ void __launch_bounds__(kCompThreads, 7)
 // passes as 0).  It issues more instructions per pair, so the large launches
 // stay with the other kernel (48.6M warp instructions against 26.5M on the
 // 512x512 frame of 500k Gaussians, most of the difference the staging, which
-// each of a tile's blocks does by itself; there it takes 100 us against 148,
+// each of a tile's blocks does by itself; there it takes 79 us against 105,
 // the SMs' busy share rising from 45% to 70%).
 //
 // Ending early: a consumer warp whose pixels have all left notes the chunk at
@@ -877,10 +879,10 @@ __device__ __forceinline__ void flush_splat(const float* sums, float weight, flo
 // Whether the tables of the group from t0 on have opacity at the same scalars,
 // by 32 samples: of the samples that any table has, each has kBwdOverlap on
 // average.  Both backward kernels ask, and take the group or leave it to the
-// other.  Tables of three bumps come to 0.7 to 0.85 and are the faster one by one
-// (1M-Gaussian scene, four of them: 1105 us, in a group 1394), tables of eight to
-// 0.88 to 0.98 and are about even (1161 and 991 there; 512x512 under eight 1439
-// and 2143), one opacity under several colour maps to 1 (1045 and 764).
+// other.  Tables of three bumps come to 0.64 to 0.91 and are the faster one by
+// one (1M-Gaussian scene, four of them: 1079 us, in a group 1374), tables of
+// eight to 0.88 to 0.98 and are about even (1142 and 981 there; 512x512 under
+// eight 1398 and 2084), one opacity under several colour maps to 1 (1019, 760).
 constexpr int kBwdGroup = 4;
 constexpr float kBwdOverlap = 0.95f;
 __device__ __forceinline__ bool tables_overlap(const CompArgs& A, int t0) {
@@ -954,8 +956,12 @@ struct BwdWarp {
   float acc[34 * kAcc];     // gradient sums of the chunk's splats
 };
 
-// Five CTAs per SM (95 registers): 1058 us against 1074 at four (116) on the
-// 1M-Gaussian scene under four tables; shaded, five take 711 us and four 599.
+// Five CTAs per SM (95 registers) unshaded: 862 us against 897 at four (122) on a
+// 1M-Gaussian training step's image under four tables, 692 and 734 on two views
+// of 1200x900 under three (258 and 239 on one table at 800x800, which ends with
+// its longest lists).  Shaded four (124): 650 us against 683 at five (96) on three
+// views of 641x479, 283 and 320 on one table at 800x800 (1053 and 1036 on the
+// 1M-Gaussian one).
 template <bool STATS, bool LIT>
 __global__ void __launch_bounds__(kCompThreads, LIT || STATS ? 4 : 5)
     composite_bwd_kernel(CompArgs A, const float4* __restrict__ out,
@@ -1156,10 +1162,9 @@ __global__ void __launch_bounds__(kCompThreads, LIT || STATS ? 4 : 5)
     }
     __syncwarp();
     // the lane that staged a splat adds its gradients to the record's
-    if (hit) {
-      flush_splat<LIT>(S.acc + slot * kAcc, S.raw[side][lane].w, S.raw[side][32 + lane], rec, grad2d,
-                       grad_shade);
-    }
+    if (hit)
+      flush_splat<LIT>(S.acc + slot * kAcc, S.raw[side][lane].w, S.raw[side][32 + lane], rec,
+                       grad2d, grad_shade);
     __syncwarp();
   }
   async_wait();  // no copy in flight past the CTA's end
@@ -1201,12 +1206,11 @@ size_t bwd_smem_bytes(bool lit) {
 // Items (tiles times groups) from which a call lets the tables' overlap choose:
 // fewer end with their longest lists, which one table at a time shortens (400x400,
 // 20,000 Gaussians, four tables of one opacity: 165 us, in groups 181; 512x512,
-// 100,000: 282 and 269).
+// 100,000: 274 and 262).
 constexpr int64_t kBwdGroupItems = 1024;
-// Tile batch of the forward: the caller's choice (128, 256 or 512 splats),
-// else 256 (131 us on the 500k-Gaussian 512x512 frame against 135 at 128; 509
-// against 504 on the 1M-Gaussian scene under 4 tables; 512 stages less often
-// but holds half the CTAs: 700 us there, 20% faster for one faint table).
+// Tile batch of the forward: the caller's choice (128, 256 or 512 splats), else
+// 256 (1M-Gaussian scene under four tables 518 us, 526 at 128; 512 stages less
+// often but holds fewer CTAs: 550 there, 333 against 432 for one faint table).
 int pick_batch(int tile_batch) { return tile_batch > 0 ? tile_batch : 256; }
 
 CompArgs make_args(const veg_camera* cams, int n_views, const float4* geo, const float4* aux,
@@ -1268,10 +1272,10 @@ veg_status launch_bwd(const CompArgs& A, int n_views, const float4* out, const i
 // item is mostly fixed (four CTAs that each stage a list), the other kernel's
 // is its longest lists until the SMs are full, so the line rises with the
 // lists' length, for which the records stand: forward with it against without,
-// 500 records at 576 items 15 and 17 us, 784 18 and 17, 1024 23 and 17; 5,000 at
-// 1024 36 and 45, 1296 44 and 46, 1600 53 and 46; 100,000 at 1296 65 and 80, 1600
-// 76 and 78, 2025 91 and 72; 400,000 at 1600 100 and 109, 2025 116 and 102;
-// 1,500,000 at 1764 162 and 177, 2025 171 and 171.
+// 500 records at 576 items 15 and 17 us, 784 19 and 17, 1024 24 and 17; 5,000 at
+// 1024 35 and 45, 1296 43 and 46, 1600 52 and 46; 100,000 at 1296 63 and 79, 1600
+// 73 and 77, 2025 88 and 72; 400,000 at 1600 97 and 107, 2025 112 and 100;
+// 1,500,000 at 1764 155 and 172, 2025 166 and 170.
 bool takes_deep(int64_t n, int64_t items) {
   return items < (n < 4096 ? 640 : n < 65536 ? 1280 : 1536);
 }

@@ -67,7 +67,8 @@ struct MarchArgs {
 };
 
 __global__ void __launch_bounds__(256)
-    volume_prepare_kernel(const float* __restrict__ vol, int R, float inv_h, float4* __restrict__ out) {
+    volume_prepare_kernel(const float* __restrict__ vol, int R, float inv_h,
+                          float4* __restrict__ out) {
   pdl_enter();
   const int64_t n = (int64_t)R * R * R;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -170,16 +171,17 @@ __device__ __forceinline__ Sample load_sample(const float4* p) {
 }
 
 // What bounds the march is instruction issue and the latency of a sample's
-// chain (ncu: 58% of the issue slots at three CTAs per SM), so a ray does as little as it can: one group marches up to 16
-// tables (each group takes the samples again); a run of samples in an empty
-// macrocell is one step, to the last sample that surely lies in it; and a
-// sample evaluates only the tables that have some opacity at its place (a
-// bit per table and entry), each lane its own next one.  The tables'
+// chain (ncu: 58% of the issue slots at three CTAs per SM), so a ray does as
+// little as it can: one group marches up to 16 tables (each group takes the
+// samples again); a run of samples in an empty macrocell is one step, to the
+// last sample that surely lies in it (raymarch_step.h); and a sample evaluates
+// only the tables that have some opacity at its place (a bit per table and
+// entry), each lane its own next one.  The tables'
 // transmittances and colours are kept in shared memory: as registers they
 // held the kernel at two CTAs per SM, and every table was a branch of every
-// sample.  Ten opacity maps over a 256^3 volume, three 800x800 views (with the macrocells' masks): 6300 us
-// in groups of eight with every sample visited and every table evaluated,
-// 4330 with the steps, bits and registers, 3430 so.  Without a material
+// sample.  Ten opacity maps over a 256^3 volume, three 800x800 views (with the
+// macrocells' masks): 6300 us in groups of eight with every sample visited and
+// every table evaluated, 4330 with the steps, bits and registers, 3430 so.  Without a material
 // (SHADE false) only the value is read and blended: ten tables over 64^3
 // vertices, one 400x300 view, 357 us (371 in the groups of eight, 409 with the
 // whole blend), one table 99 (194).
@@ -218,8 +220,9 @@ __global__ void __launch_bounds__(256, 3)
     unsigned m = 0u;
     for (int t = 0; known && t < ntg; ++t) {
       const float4 lo = __ldg(&lut[t * L + k]), hi = __ldg(&lut[t * L + min(k + 1, L - 1)]);
-      const float big = fmaxf(fmaxf(fmaxf(fabsf(lo.x), fabsf(lo.y)), fmaxf(fabsf(lo.z), fabsf(hi.x))),
-                              fmaxf(fabsf(hi.y), fabsf(hi.z)));
+      const float big =
+          fmaxf(fmaxf(fmaxf(fabsf(lo.x), fabsf(lo.y)), fmaxf(fabsf(lo.z), fabsf(hi.x))),
+                fmaxf(fabsf(hi.y), fabsf(hi.z)));
       const float sum = lo.x + lo.y + lo.z + hi.x + hi.y + hi.z;  // NaN of any entry stays
       if (lo.w > 0.0f || hi.w > 0.0f || !(big <= 1.0e30f) || sum != sum) m |= 1u << t;
     }

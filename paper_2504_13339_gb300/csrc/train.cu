@@ -429,10 +429,10 @@ extern "C" veg_status veg_l1_ssim_loss(const float* out, const float* target, in
   const dim3 grid((unsigned)(tx * ty), (unsigned)n_images);
   const float4* o4 = reinterpret_cast<const float4*>(out);
   const float4* t4 = reinterpret_cast<const float4*>(target);
-  launch_k(l1_ssim_stats_kernel, grid, kSsimThreads, sizeof(StatsSmem), stream, win, o4, t4, height, width,
-           tx, planes, part);
-  launch_k(l1_ssim_grad_kernel, grid, kSsimThreads, sizeof(GradSmem), stream, win, o4, t4, height, width,
-           tx, lambda, (float)(1.0 / count), planes, reinterpret_cast<float4*>(grad));
+  launch_k(l1_ssim_stats_kernel, grid, kSsimThreads, sizeof(StatsSmem), stream, win, o4, t4,
+           height, width, tx, planes, part);
+  launch_k(l1_ssim_grad_kernel, grid, kSsimThreads, sizeof(GradSmem), stream, win, o4, t4, height,
+           width, tx, lambda, (float)(1.0 / count), planes, reinterpret_cast<float4*>(grad));
   count_launch(2);
   launch_k(l1_ssim_final_kernel, 1, 1024, 0, stream, part, (int64_t)tx * ty * n_images, 1.0 / count,
                                                lambda, loss);
