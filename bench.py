@@ -1365,7 +1365,7 @@ def cpu_baseline_opt(cams, luts, g, lt, targets, args, n_samples=4, seed=21):
 # evaluation: table lerp 8, clamp 2, opacity correction 4, shaded colour 6,
 # compositing 7, stop test 1; a sample skipped as empty costs its position
 # and grid coordinates (12).
-MARCH_FLOPS = {"sample": 98, "table": 28, "skipped": 12}
+MARCH_FLOPS = {"sample": 98, "table": 28}
 MARCH_CELL = 8  # macrocell edge (vertex cells) of the empty-space masks
 
 
@@ -1422,8 +1422,7 @@ def run_raymarch(args):
     render_all(st)
     torch.cuda.synchronize()
     samples, tables, skipped = (int(x) for x in st.cpu().numpy())
-    flops = (MARCH_FLOPS["sample"] * samples + MARCH_FLOPS["table"] * tables +
-             MARCH_FLOPS["skipped"] * skipped)
+    flops = MARCH_FLOPS["sample"] * samples + MARCH_FLOPS["table"] * tables
     props = torch.cuda.get_device_properties(0)
     peaks = {}
     try:
@@ -1443,11 +1442,11 @@ def run_raymarch(args):
         "work": {"samples": samples, "table_evaluations": tables, "samples_skipped": skipped},
         "empty_space": f"macrocells of {MARCH_CELL}^3 vertex cells; a sample whose macrocell has "
                        "no opacity for any live table is skipped (images identical)",
-        "roofline": {"bound": "alu", "kernel": "raymarch_kernel<8>/<2>",
+        "roofline": {"bound": "alu", "kernel": "raymarch_kernel",
                      "achieved": round(achieved, 3), "peak": round(peak, 2), "unit": "TFLOP/s",
                      "frac": round(achieved / peak, 4),
-                     "flops_model": "98 per sample + 28 per table evaluation + 12 per skipped "
-                                    "sample (FMA = 2)"},
+                     "flops_model": "98 per sample taken + 28 per table evaluated (FMA = 2); "
+                                    "empty space is passed in steps"},
         "data": "synthetic"}
     if not args.no_cpu_baseline:
         rng = np.random.default_rng(3)

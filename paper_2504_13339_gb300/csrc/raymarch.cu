@@ -187,8 +187,7 @@ __device__ __forceinline__ Sample load_sample(const float4* p) {
 // whole blend), one table 99 (194).
 //
 // stats (instrumented build): samples taken (per ray and table group),
-// table evaluations (samples x live tables) and, with a cell mask, samples
-// skipped as empty.
+// table evaluations and, with a cell mask, samples skipped as empty.
 template <bool MANY, bool STATS, bool SHADE>
 __global__ void __launch_bounds__(256, 3)
     raymarch_kernel(MarchArgs A, const __grid_constant__ RaySet rs, float4* __restrict__ out,
@@ -353,7 +352,7 @@ __global__ void __launch_bounds__(256, 3)
       }
       if (STATS) {
         ++n_samp;
-        n_tab += (unsigned)__popc(live);
+        n_tab += (unsigned)__popc(on);
       }
       if (on == 0u) continue;
       // each lane its own next table: a step serves lanes at different ones
